@@ -18,9 +18,11 @@
 // both with the packed f32x2 FMA/add/multiply (same rounding per lane as
 // scalar code).  Each CTA owns up to 256 targets of one batch (128 threads x
 // 2 targets) and a contiguous segment
-// of the batch's interaction list; source tiles of 256 records are staged in
+// of the batch's interaction list; its four warps share out the targets and,
+// where there are at most 128, the sources as well (see Share); source tiles
+// of 256 records are staged in
 // shared memory with positions shifted from the record's frame (its leaf or
-// cluster center) to the batch center in float64 and rounded once.  Near-field
+// cluster center) to the batch center in two-float arithmetic and rounded once.  Near-field
 // values and weights are two-float (see tile_near); proxies are single float.
 // rsqrt and exp2 use the MUFU unit (rsqrt.approx, ex2.approx); their mean
 // bias is measured once per device (fp32_bias) and compensated in the SS
@@ -112,6 +114,47 @@ __device__ __forceinline__ void fold(float (&acc)[TPT][NF], float (&hi)[TPT][NF]
         }
 }
 
+// How the four warps of a CTA share its item.  A warp holds 64 targets (two
+// per lane), and batches of adaptive meshes are small: with one warp per 64
+// targets the item of a 100-target batch would leave half of the warps (and,
+// with a lane pair 128 targets apart, half of the packed arithmetic) on
+// padding.  On the Li, H2 and CO meshes the mean batch holds 340 to 500
+// targets and that padding is 23 to 36% of all pairs.  So items of at most
+// 128 (64) targets take two (four) groups of warps on the same targets, each
+// group every second (fourth) fold of the staged sources, and the groups' sums
+// are added at the end: 64-target granularity, 2 to 5% padding, every warp
+// busy.  Folds stay whole, so a pair's arithmetic and the float32 sum it
+// enters do not depend on the split.  With 129 to 192 targets the fourth warp
+// only helps staging.
+struct Share {
+    int grp, ngrp;  // this warp takes folds grp, grp + ngrp, ... of a tile
+    int slot;       // its lane's first target; the second is slot + 32
+    bool busy;      // the warp has targets
+    __device__ __forceinline__ Share(int nt, int warp, int lane)
+    {
+        const int lw = nt > 128 ? 2 : (nt > 64 ? 1 : 0);  // log2 of the warps across targets
+        const int tw = warp & ((1 << lw) - 1);
+        grp = warp >> lw;
+        ngrp = 4 >> lw;
+        slot = 64 * tw + lane;
+        busy = 64 * tw < nt;
+    }
+};
+
+// One coordinate of a staged source: the float32 nearest to (hi + lo) +
+// (oh + ol), its two-float position in its frame plus the two-float offset of
+// the frame from the batch center.  TwoSum(hi, oh) is exact and the low parts
+// add 2^-48 of the operands, as much as the two-floats themselves leave out;
+// the same sum in float64 costs 3 conversions and 2 additions at 2 a clock
+// and SM, 60 times what float32 costs here, and took 2000 clocks of that unit
+// per 256-source tile, against 9000 of arithmetic of a one-field tile.
+__device__ __forceinline__ float shifted(float hi, float lo, float oh, float ol)
+{
+    float s, e;
+    two_sum(hi, oh, s, e);
+    return __fadd_rn(s, __fadd_rn(e, __fadd_rn(lo, ol)));
+}
+
 // Shared-memory layout of a staged tile: per source one float4 of position
 // (relative to the batch center) and weight (high part), and the values
 // packed four to a float4: components [0, NF) hold fh (points) or qh
@@ -151,14 +194,15 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __
 // GZ: the entry's Gaussian of the Coulomb SS is below float32 resolution for
 // every pair (list flag bit2), so the Hartree term is q / r alone.
 template <int NY, bool HH, bool SS, int TPT, bool GZ>
-__device__ __forceinline__ void tile_far(const float4* __restrict__ srec, const float4* __restrict__ sv, int nk,
+__device__ __forceinline__ void tile_far(const Share& sh, const float4* __restrict__ srec,
+                                         const float4* __restrict__ sv, int nk,
                                          const float2 (&ntx)[TPT / 2], const float2 (&nty)[TPT / 2],
                                          const float2 (&ntz)[TPT / 2], const float2 (&nc)[TPT / 2][NY + HH],
                                          float (&hi)[TPT][NY + HH], float (&lo)[TPT][NY + HH], const KParams& kp)
 {
     constexpr int NF = NY + HH;
     constexpr int G = TileLayout<NF>::G;
-    for (int k0 = 0; k0 < nk; k0 += kFold) {
+    for (int k0 = sh.grp * kFold; k0 < nk; k0 += sh.ngrp * kFold) {
         float acc[TPT][NF];
 #pragma unroll
         for (int j = 0; j < TPT; j++)
@@ -255,7 +299,8 @@ struct TensorLayout {
 };
 
 template <int NY, bool HH, bool SS, int TPT, int M, bool GZ>
-__device__ __forceinline__ void tile_far_tensor(const float* __restrict__ sX, const float* __restrict__ sY,
+__device__ __forceinline__ void tile_far_tensor(const Share& sh, const float* __restrict__ sX,
+                                                const float* __restrict__ sY,
                                                 const float2* __restrict__ sZ2, const float4* __restrict__ st, int np,
                                                 const float2 (&ntx)[TPT / 2], const float2 (&nty)[TPT / 2],
                                                 const float2 (&ntz)[TPT / 2], const float2 (&nc)[TPT / 2][NY + HH],
@@ -265,7 +310,7 @@ __device__ __forceinline__ void tile_far_tensor(const float* __restrict__ sX, co
     constexpr int NF = NY + HH;
     constexpr int NP = TPT / 2;
     constexpr int GF2 = TensorLayout<NF>::GF2;
-    for (int pl = 0; pl < np; pl++) {
+    for (int pl = 0, k2 = sh.grp; pl < np; pl++, k2 -= M) {
         float2 dx2[NP];
         const float xk = sX[pl];
 #pragma unroll
@@ -273,7 +318,7 @@ __device__ __forceinline__ void tile_far_tensor(const float* __restrict__ sX, co
             const float2 d = add2(make_float2(xk, xk), ntx[j]);
             dx2[j] = mul2(d, d);
         }
-        for (int k2 = 0; k2 < M; k2++) {
+        for (; k2 < M; k2 += sh.ngrp) {  // the rows of all planes in turn, every ngrp-th
             float2 a[NP];
             const float yk = sY[k2];
 #pragma unroll
@@ -338,15 +383,16 @@ __device__ __forceinline__ void tile_far_tensor(const float* __restrict__ sX, co
 // Two targets per instruction (f32x2), each lane rounding exactly as the
 // scalar form would.
 template <int NY, bool HH, bool SS, bool SELF, int TPT, bool GZ>
-__device__ __forceinline__ void tile_near(const float4* __restrict__ sn, int nk, const float2 (&ntx)[TPT / 2],
-                                          const float2 (&nty)[TPT / 2], const float2 (&ntz)[TPT / 2],
+__device__ __forceinline__ void tile_near(const Share& sh, const float4* __restrict__ sn, int nk,
+                                          const float2 (&ntx)[TPT / 2], const float2 (&nty)[TPT / 2],
+                                          const float2 (&ntz)[TPT / 2],
                                           const float2 (&nc)[TPT / 2][NY + HH], float (&hi)[TPT][NY + HH],
                                           float (&lo)[TPT][NY + HH], const KParams2& kp)
 {
     constexpr int NF = NY + HH;
     constexpr int NP = TPT / 2;
     constexpr int NV4 = NearLayout<NF>::NV4;
-    for (int k0 = 0; k0 < nk; k0 += kFold) {
+    for (int k0 = sh.grp * kFold; k0 < nk; k0 += sh.ngrp * kFold) {
         float2 acc[NP][NF];
 #pragma unroll
         for (int j = 0; j < NP; j++)
@@ -423,6 +469,7 @@ __device__ __forceinline__ void chunk_sum(const Item& it, double* __restrict__ p
     __threadfence();  // the other CTAs' rows after their counts
     for (int q = threadIdx.x; q < nf * kTargetsPerItem; q += THREADS) {
         const int o = field0 + q / kTargetsPerItem, slot = q % kTargetsPerItem;
+        if (slot >= it.t1 - it.t0) continue;  // not a target: its row entry is not written
         const double* src = part + (size_t)o * kTargetsPerItem + slot;
         double S = 0.0;
         for (int i = it.i0; i < it.i0 + it.ni; i++) S += __ldcg(src + (size_t)i * nf_tot * kTargetsPerItem);
@@ -443,7 +490,7 @@ __device__ __forceinline__ void chunk_sum(const Item& it, double* __restrict__ p
 template <int NY, bool HH, bool SS, int M>
 __global__ void __launch_bounds__(Tpt<NY + HH>::threads) k_interact32(const Item* __restrict__ items,
                                                            const Entry* __restrict__ ents,
-                                                           const double* __restrict__ cen,
+                                                           const float4* __restrict__ eoff,
                                                            const float4* __restrict__ rec4,
                                                            const float4* __restrict__ rec4lo,
                                                            const float* __restrict__ fa, int64_t lda,
@@ -481,20 +528,23 @@ __global__ void __launch_bounds__(Tpt<NY + HH>::threads) k_interact32(const Item
 
     const Item it = items[blockIdx.x];
     const int tid = threadIdx.x;
+    const int nt = it.t1 - it.t0;
+    const Share sh(nt, tid >> 5, tid & 31);
+    static_assert(TPT == 2 && THREADS == 128, "Share's mapping: four warps of 64 targets");
     float2 ntx[NP], nty[NP], ntz[NP];
     float2 nc[NP][NF];
     float hi[TPT][NF], lo[TPT][NF];
 #pragma unroll
     for (int j = 0; j < TPT; j++) {
-        const int p = it.t0 + tid + j * THREADS;
+        const int p = it.t0 + sh.slot + j * 32;
         const bool ok = p < it.t1;
         const float4 r = ok ? rec4[p] : make_float4(0.f, 0.f, 0.f, 0.f);
         const float4 rl = ok ? rec4lo[p] : make_float4(0.f, 0.f, 0.f, 0.f);
-        // rounded exactly as a staged source of the batch's own leaf, so the
-        // self pair gives r = 0 bit for bit
-        const float x = -(float)(((double)r.x + (double)rl.x) + 0.0);
-        const float y = -(float)(((double)r.y + (double)rl.y) + 0.0);
-        const float z = -(float)(((double)r.z + (double)rl.z) + 0.0);
+        // rounded exactly as a staged source of the batch's own leaf (a zero
+        // offset in shifted()), so the self pair gives r = 0 bit for bit
+        const float x = -__fadd_rn(r.x, rl.x);
+        const float y = -__fadd_rn(r.y, rl.y);
+        const float z = -__fadd_rn(r.z, rl.z);
         if (j & 1) {
             ntx[j >> 1].y = x;
             nty[j >> 1].y = y;
@@ -514,13 +564,11 @@ __global__ void __launch_bounds__(Tpt<NY + HH>::threads) k_interact32(const Item
             hi[j][o] = lo[j][o] = 0.0f;
         }
     }
-    const double bx = cen[3 * it.batch], by = cen[3 * it.batch + 1], bz = cen[3 * it.batch + 2];
     constexpr bool GZOK = HH && SS;  // a Gaussian to leave out exists
 
     for (int e = it.e0; e < it.e1; e++) {
         const Entry en = ents[e];
-        const int f = en.frame;
-        const double ox = cen[3 * f] - bx, oy = cen[3 * f + 1] - by, oz = cen[3 * f + 2] - bz;
+        const float4 oh = eoff[2 * e], ol = eoff[2 * e + 1];  // frame center - batch center, two-float
         const bool far = en.flags & 2;
         const bool self = en.flags & 1;
         const bool gz = en.flags & 4;
@@ -536,9 +584,9 @@ __global__ void __launch_bounds__(Tpt<NY + HH>::threads) k_interact32(const Item
                     const float4 rx = rec4[en.src0 + tid * M * M];
                     const float4 ry = rec4[en.src0 + tid * M];
                     const float4 rz = rec4[en.src0 + tid];
-                    sX[tid] = (float)((double)rx.x + ox);
-                    sY[tid] = (float)((double)ry.y + oy);
-                    const float z = (float)((double)rz.z + oz);
+                    sX[tid] = shifted(rx.x, 0.0f, oh.x, ol.x);
+                    sY[tid] = shifted(ry.y, 0.0f, oh.y, ol.y);
+                    const float z = shifted(rz.z, 0.0f, oh.z, ol.z);
                     sZ2[tid] = make_float2(z, z);
                 }
                 for (int p0 = 0; p0 < M; p0 += PL) {
@@ -562,12 +610,13 @@ __global__ void __launch_bounds__(Tpt<NY + HH>::threads) k_interact32(const Item
                         }
                     }
                     __syncthreads();
+                    if (!sh.busy) continue;
                     if (GZOK && gz)
-                        tile_far_tensor<NY, HH, SS, TPT, M, GZOK>(sX + p0, sY, sZ2, st, np, ntx, nty, ntz, nc, hi, lo,
-                                                                  kp2);
+                        tile_far_tensor<NY, HH, SS, TPT, M, GZOK>(sh, sX + p0, sY, sZ2, st, np, ntx, nty, ntz, nc, hi,
+                                                                  lo, kp2);
                     else
-                        tile_far_tensor<NY, HH, SS, TPT, M, false>(sX + p0, sY, sZ2, st, np, ntx, nty, ntz, nc, hi, lo,
-                                                                   kp2);
+                        tile_far_tensor<NY, HH, SS, TPT, M, false>(sh, sX + p0, sY, sZ2, st, np, ntx, nty, ntz, nc, hi,
+                                                                   lo, kp2);
                 }
                 continue;
             }
@@ -586,9 +635,9 @@ __global__ void __launch_bounds__(Tpt<NY + HH>::threads) k_interact32(const Item
                     if (k < ns) {
                         // proxy = cluster center + delta; one rounding to float32
                         float4 r = rec4[s0 + k];
-                        r.x = (float)((double)r.x + ox);
-                        r.y = (float)((double)r.y + oy);
-                        r.z = (float)((double)r.z + oz);
+                        r.x = shifted(r.x, 0.0f, oh.x, ol.x);
+                        r.y = shifted(r.y, 0.0f, oh.y, ol.y);
+                        r.z = shifted(r.z, 0.0f, oh.z, ol.z);
                         srec[k] = r;
 #pragma unroll
                         for (int o = 0; o < NF; o++) v[o] = fa[o * lda + s0 + k];
@@ -612,9 +661,9 @@ __global__ void __launch_bounds__(Tpt<NY + HH>::threads) k_interact32(const Item
                         // point = leaf center + (delta_hi + delta_lo); one rounding
                         const float4 r = rec4[s0 + k];
                         const float4 rl = rec4lo[s0 + k];
-                        v[0] = (float)(((double)r.x + (double)rl.x) + ox);
-                        v[1] = (float)(((double)r.y + (double)rl.y) + oy);
-                        v[2] = (float)(((double)r.z + (double)rl.z) + oz);
+                        v[0] = shifted(r.x, rl.x, oh.x, ol.x);
+                        v[1] = shifted(r.y, rl.y, oh.y, ol.y);
+                        v[2] = shifted(r.z, rl.z, oh.z, ol.z);
                         v[3] = r.w;   // weight, high part
                         v[4] = rl.w;  // weight, low part
 #pragma unroll
@@ -633,25 +682,47 @@ __global__ void __launch_bounds__(Tpt<NY + HH>::threads) k_interact32(const Item
                 }
             }
             __syncthreads();
+            if (!sh.busy) continue;
             if (far) {
                 if (GZOK && gz)
-                    tile_far<NY, HH, SS, TPT, GZOK>(srec, sv, nk, ntx, nty, ntz, nc, hi, lo, kp);
+                    tile_far<NY, HH, SS, TPT, GZOK>(sh, srec, sv, nk, ntx, nty, ntz, nc, hi, lo, kp);
                 else
-                    tile_far<NY, HH, SS, TPT, false>(srec, sv, nk, ntx, nty, ntz, nc, hi, lo, kp);
+                    tile_far<NY, HH, SS, TPT, false>(sh, srec, sv, nk, ntx, nty, ntz, nc, hi, lo, kp);
             } else if (self) {
-                tile_near<NY, HH, SS, true, TPT, false>(sn, nk, ntx, nty, ntz, nc, hi, lo, kp2);
+                tile_near<NY, HH, SS, true, TPT, false>(sh, sn, nk, ntx, nty, ntz, nc, hi, lo, kp2);
             } else if (GZOK && gz) {
-                tile_near<NY, HH, SS, false, TPT, GZOK>(sn, nk, ntx, nty, ntz, nc, hi, lo, kp2);
+                tile_near<NY, HH, SS, false, TPT, GZOK>(sh, sn, nk, ntx, nty, ntz, nc, hi, lo, kp2);
             } else {
-                tile_near<NY, HH, SS, false, TPT, false>(sn, nk, ntx, nty, ntz, nc, hi, lo, kp2);
+                tile_near<NY, HH, SS, false, TPT, false>(sh, sn, nk, ntx, nty, ntz, nc, hi, lo, kp2);
             }
         }
     }
     double* out = part + ((size_t)blockIdx.x * nf_tot + field0) * kTargetsPerItem;
+    // at most 64 * 4 / ngrp targets: (ngrp - 1) NF rows of that many sums fit
+    // (the largest, 3 x 64 NF, against SB >= NF + 3 rows of 512)
+    double* const red = reinterpret_cast<double*>(sbuf);
+    const int rw = kTargetsPerItem / sh.ngrp;
+    if (sh.ngrp > 1) {
+        __syncthreads();  // every warp is done with the staged tile
+        if (sh.grp > 0 && sh.busy)
 #pragma unroll
-    for (int j = 0; j < TPT; j++)
+            for (int j = 0; j < TPT; j++)
 #pragma unroll
-        for (int o = 0; o < NF; o++) out[o * kTargetsPerItem + tid + j * THREADS] = (double)hi[j][o] + (double)lo[j][o];
+                for (int o = 0; o < NF; o++)
+                    red[((sh.grp - 1) * NF + o) * rw + sh.slot + j * 32] = (double)hi[j][o] + (double)lo[j][o];
+        __syncthreads();
+    }
+    if (sh.grp == 0)
+#pragma unroll
+        for (int j = 0; j < TPT; j++)
+#pragma unroll
+            for (int o = 0; o < NF; o++) {
+                const int slot = sh.slot + j * 32;
+                if (slot >= nt) continue;
+                double S = (double)hi[j][o] + (double)lo[j][o];
+                for (int g = 1; g < sh.ngrp; g++) S += red[((g - 1) * NF + o) * rw + slot];
+                out[o * kTargetsPerItem + slot] = S;
+            }
     chunk_sum<THREADS>(it, part, tsum, cnt, nf_tot, field0, NF);
 }
 
@@ -769,7 +840,7 @@ void launch32_m(Tree& T, const float* kyd, const float* q, const float* c, doubl
                 int nf_tot, int field0)
 {
     launch(k_interact32<NY, HH, SS, M>, (int)T.nitems, Tpt<NY + HH>::threads, 0, T.stream, T.items.as<Item>(),
-           T.ent.as<Entry>(), T.cl_cen.as<double>(), T.rec4.as<float4>(), T.rec4lo.as<float4>(), q, T.nrec, c, T.n,
+           T.ent.as<Entry>(), T.ent_shift.as<float4>(), T.rec4.as<float4>(), T.rec4lo.as<float4>(), q, T.nrec, c, T.n,
            kyd, part, tsum, cnt, nf_tot, field0);
 }
 

@@ -170,6 +170,7 @@ struct Tree {
 
     // lists (expanded): entries in batch order with CSR offsets by leaf index
     DevBuf ent;       // Entry[nent]
+    DevBuf ent_shift; // FP32C: float4[2 nent], frame center - batch center of each entry as a two-float (high, low)
     DevBuf ent_off;   // int64 -> int[nleaf+1]
     DevBuf ent_batch; // int[nent] (leaf cluster id), for export
     DevBuf ent_clus;  // int[nent] (source cluster id: leaf for direct, cluster for far)

@@ -539,6 +539,24 @@ __global__ void k_gauss_flags(int64_t nent, Entry* ent, const int* eb, const int
     }
 }
 
+// Offset of each entry's frame from its batch's center, as a two-float, so
+// that the near/far kernel shifts positions without float64.
+__global__ void k_entry_shift(int64_t nent, const Entry* __restrict__ ent, const int* __restrict__ eb,
+                              const double* __restrict__ cen, float4* __restrict__ out)
+{
+    int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (e >= nent) return;
+    const int f = ent[e].frame, b = eb[e];
+    float h[3], l[3];
+    for (int d = 0; d < 3; d++) {
+        const double o = cen[3 * f + d] - cen[3 * b + d];
+        h[d] = (float)o;
+        l[d] = (float)(o - (double)h[d]);
+    }
+    out[2 * e] = make_float4(h[0], h[1], h[2], 0.0f);
+    out[2 * e + 1] = make_float4(l[0], l[1], l[2], 0.0f);
+}
+
 // ---------------------------------------------------------------- work items
 __device__ __forceinline__ int padded(int v) { return (v + 7) & ~7; }
 
@@ -965,6 +983,11 @@ void build_tree(Tree& T, const double* xyz, const double* w)
     TAGI_REQUIRE(T.nrec < (int64_t)0x7fffffff, "too many source records");
     if (T.nent > 0)
         launch(k_far_ranges, nblocks(T.nent, 256), 256, 0, s, T.nent, T.ent.as<Entry>(), T.cl_far.as<int>(), n, T.P);
+    if (T.prec == TAGI_FP32C && T.nent > 0) {
+        T.ent_shift.ensure(2 * sizeof(float4) * (size_t)T.nent);
+        launch(k_entry_shift, nblocks(T.nent, 256), 256, 0, s, T.nent, T.ent.as<Entry>(), T.ent_batch.as<int>(),
+               T.cl_cen.as<double>(), T.ent_shift.as<float4>());
+    }
     T.near_pairs_ng = T.far_pairs_ng = 0;
     if (T.nent > 0) {
         DevBuf ng;

@@ -1,0 +1,61 @@
+"""The FP32C near/far kernel's split of an item over its warps: batches whose
+target counts sit at the edges of the groups (64 targets a warp, two or four
+source groups below 129 and 65 targets, 256 targets an item).  Parity with the
+float64 oracle within the stated FP32C tolerance, relative L2 1e-6 per field.
+"""
+import numpy as np
+import pytest
+
+import oracle
+from paper_2003_01833_gb300 import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+FP32C_TOL = 1e-6
+
+
+@pytest.fixture(scope="module")
+def T():
+    import __graft_entry__ as g
+
+    g.build()
+    import paper_2003_01833_gb300.tagi as T
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return T
+
+
+def dev(a):
+    return torch.tensor(np.ascontiguousarray(a), dtype=torch.float64, device="cuda")
+
+
+def check(T, n, leaf, degree, seed, ss=True):
+    xyz, w = W.random_cube(n, seed=seed)
+    f = 1.0 + 0.3 * np.sin(3 * xyz[0]) * np.cos(2 * xyz[1])
+    rho = np.exp(-np.sum(xyz * xyz, axis=0))
+    with T.Tree(dev(xyz), dev(w), theta=0.7, degree=degree, leaf_size=leaf, prec=T.TAGI_FP32C, ss=ss) as tr:
+        u, vh = torch.empty((1, n), dtype=torch.float64, device="cuda"), torch.empty(n, dtype=torch.float64,
+                                                                                    device="cuda")
+        T.tagi_fields_conv(tr.handle, dev(f), [1.7], u, rho=dev(rho), vh=vh)
+        u, vh = u.cpu().numpy()[0], vh.cpu().numpy()
+    ot = oracle.Tree(xyz, leaf)
+    for got, ref in ((u, oracle.treecode_yukawa(ot, 0.7, degree, f, 1.7, w, ss=ss)),
+                     (vh, oracle.treecode_coulomb(ot, 0.7, degree, rho, w, ss=ss))):
+        assert np.linalg.norm(got - ref) <= FP32C_TOL * np.linalg.norm(ref)
+
+
+@pytest.mark.parametrize("n", [2, 17, 33, 63, 64, 65, 127, 128, 129, 191, 193, 255, 256, 257, 300, 513])
+def test_one_batch_at_the_edges(T, n):
+    check(T, n, 600, 6, seed=n)
+
+
+@pytest.mark.parametrize("degree", [5, 6, 8])  # record path, tensor-grid path with 7 and 9 nodes
+@pytest.mark.parametrize("leaf", [40, 90, 180, 700])
+def test_far_field_over_groups(T, degree, leaf):
+    check(T, 12007, leaf, degree, seed=leaf + degree)
+
+
+def test_without_subtraction(T):
+    check(T, 5003, 90, 6, seed=4, ss=False)
