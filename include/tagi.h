@@ -58,9 +58,9 @@ typedef enum {
  *   alpha      Gaussian width of the Coulomb subtraction (Eq. coulomb-conv-ss), > 0.
  *   segment    sources per work item of the near/far kernel (a batch's 256
  *              targets against a run of its interaction list), 1024 <= segment
- *              <= 65536, or 0 for 8192.  Longer segments mean fewer partial
- *              sums, shorter ones a finer balance of the work; the float32
- *              sums of the FP32C form are grouped by segment. */
+ *              <= 65536, or 0: chosen from the number of pairs, at most 2048.
+ *              Longer segments mean fewer partial sums, shorter ones a finer
+ *              balance of the work; partial sums are added in float64. */
 typedef struct {
     double theta;
     int degree;

@@ -295,7 +295,7 @@ tagi_status tagi_tree_build(const double* xyz, const double* w, int64_t n, const
         TAGI_REQUIRE(std::isfinite(p.alpha) && p.alpha > 0.0, "alpha must be finite and > 0");
         TAGI_REQUIRE(p.segment == 0 || (p.segment >= 1024 && p.segment <= 65536), "segment must be 0 or in [1024, 65536]");
         std::unique_ptr<Tree> T(new Tree());
-        T->segment = p.segment ? p.segment : 8192;
+        T->segment = p.segment;
         T->n = n;
         T->theta = p.theta;
         T->degree = p.degree;

@@ -621,8 +621,11 @@ __global__ void __launch_bounds__(Tpt<NY + HH>::threads) k_interact32(const Item
                 continue;
             }
         }
-        for (int s0 = en.src0; s0 < en.src1; s0 += kTile) {
-            const int ns = min(kTile, en.src1 - s0);
+        // an item may begin and end inside an entry (never inside a cluster's grid)
+        const int src0 = en.src0 + (e == it.e0 ? it.skip : 0);
+        const int src1 = it.stop > 0 && e == it.e1 - 1 ? en.src0 + it.stop : en.src1;
+        for (int s0 = src0; s0 < src1; s0 += kTile) {
+            const int ns = min(kTile, src1 - s0);
             const int nk = (ns + 15) & ~15;
             __syncthreads();
             if (far) {
@@ -805,8 +808,10 @@ __global__ void __launch_bounds__(kThreads64) k_interact64(const Item* __restric
     double acc = 0.0;
     for (int e = it.e0; e < it.e1; e++) {
         const Entry en = ents[e];
-        for (int s0 = en.src0; s0 < en.src1; s0 += kTile64) {
-            const int ns = min(kTile64, en.src1 - s0);
+        const int src0 = en.src0 + (e == it.e0 ? it.skip : 0);
+        const int src1 = it.stop > 0 && e == it.e1 - 1 ? en.src0 + it.stop : en.src1;
+        for (int s0 = src0; s0 < src1; s0 += kTile64) {
+            const int ns = min(kTile64, src1 - s0);
             __syncthreads();
             if (tid < ns) {
                 sx[tid] = rx[s0 + tid];

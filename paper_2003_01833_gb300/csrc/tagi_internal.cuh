@@ -122,11 +122,13 @@ struct Entry {
 };
 
 // Work item of the near/far kernel: targets [t0, t1) of batch `batch`
-// (tree positions), list entries [e0, e1); target chunk `tchunk` of the
+// (tree positions), list entries [e0, e1), the first from its source skip on
+// and the last up to source stop (0: all of it); target chunk `tchunk` of the
 // current chunk tables, whose items are [i0, i0 + ni) of the item array.
 struct Item {
     int t0, t1, e0, e1;
     int batch, tchunk, i0, ni;
+    int skip, stop;
 };
 
 // Anterpolation work item: positions [p0, p1) of cluster `cluster`, whose
@@ -144,7 +146,7 @@ struct Tree {
     int prec = TAGI_FP32C;
     int ss = 1;
     double alpha = 1.0;
-    int segment = 8192;  // sources per work item of the near/far kernel
+    int segment = 0;  // sources per work item of the near/far kernel, 0: chosen by build_tree
     int P = 0;  // (degree+1)^3
     cudaStream_t stream = nullptr;
 

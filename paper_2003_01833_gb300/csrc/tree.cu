@@ -558,63 +558,121 @@ __global__ void k_entry_shift(int64_t nent, const Entry* __restrict__ ent, const
 }
 
 // ---------------------------------------------------------------- work items
-__device__ __forceinline__ int padded(int v) { return (v + 7) & ~7; }
+// A batch's list as a row of source positions: each entry padded to whole
+// folds of 16, cut into units where an item may begin -- every kItemUnit
+// sources of a direct entry (the kernel's tile), an approximated cluster as
+// one unit.  Item s of a target chunk starts at the first unit at or after
+// position s * seg.  A unit is no longer than seg, so no item is empty, and
+// units are whole folds, so the cut moves no float32 sum.
+constexpr int kItemUnit = 256;
+constexpr int kSegmentMax = 2048;
+constexpr int kItemsWanted = 8192;
+static_assert(kItemUnit % 16 == 0, "whole folds");
 
-__global__ void k_item_counts(int nleaf, const int* leaves, const int* begin, const int* end, const int64_t* eoff,
-                              const Entry* ent, int seg_src, int64_t* nchunk, int64_t* nitem)
+__host__ __device__ __forceinline__ int padded(int v) { return (v + 15) & ~15; }
+// offset of the entry's last unit from its start
+__device__ __forceinline__ int last_unit(const Entry& x)
 {
-    int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= nleaf) return;
-    int b = leaves[j];
-    int nb = end[b] - begin[b];
-    int ch = (nb + kTargetsPerItem - 1) / kTargetsPerItem;
-    int segs = 0, acc = 0;
-    for (int64_t e = eoff[j]; e < eoff[j + 1]; e++) {
-        acc += padded(ent[e].src1 - ent[e].src0);
-        if (acc >= seg_src) {
-            segs++;
-            acc = 0;
-        }
-    }
-    if (acc > 0 || segs == 0) segs++;
-    nchunk[j] = ch;
-    nitem[j] = (int64_t)ch * segs;
+    return (x.flags & 2) ? 0 : (x.src1 - x.src0 - 1) / kItemUnit * kItemUnit;
 }
 
-__global__ void k_item_fill(int nleaf, const int* leaves, const int* begin, const int* end, const int64_t* eoff,
-                            const Entry* ent, int seg_src, const int64_t* chunk_off, const int64_t* item_off,
-                            Item* items, int* tc_item0, int* tc_t0, int* tc_t1, int* tc_batch)
+// One warp per batch: target chunks and items (chunks times segments).
+__global__ void k_item_counts(int nleaf, const int* leaves, const int* begin, const int* end, const int64_t* eoff,
+                              const Entry* ent, int seg, int64_t* nchunk, int64_t* nitem)
 {
-    // one block per leaf, one thread per target chunk of the leaf
+    const int j = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32), lane = threadIdx.x & 31;
+    if (j >= nleaf) return;  // uniform per warp
+    const int64_t e0 = eoff[j], e1 = eoff[j + 1];
+    int64_t sum = 0;
+    for (int64_t e = e0 + lane; e < e1; e += 32) {
+        const Entry x = ent[e];
+        sum += e + 1 < e1 ? padded(x.src1 - x.src0) : last_unit(x);
+    }
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) {
+        const int b = leaves[j];
+        const int ch = (end[b] - begin[b] + kTargetsPerItem - 1) / kTargetsPerItem;
+        nchunk[j] = ch;
+        nitem[j] = ch * (sum / seg + 1);  // sum: where the last unit starts
+    }
+}
+
+// One block per batch.  First its warp 0 finds the first unit of every
+// segment (32 entries at a time, a warp prefix sum of their padded lengths)
+// and leaves it in the first chunk's items; then all threads complete the
+// items of all chunks.
+__global__ void __launch_bounds__(128) k_item_fill(int nleaf, const int* leaves, const int* begin, const int* end,
+                                                   const int64_t* eoff, const Entry* ent, int seg,
+                                                   const int64_t* chunk_off, const int64_t* item_off, Item* items,
+                                                   int* tc_item0, int* tc_t0, int* tc_t1, int* tc_batch)
+{
     const int j = blockIdx.x;
-    if (j >= nleaf) return;
-    int b = leaves[j];
-    int nb = end[b] - begin[b];
-    int ch = (int)(chunk_off[j + 1] - chunk_off[j]);
-    int segs = ch ? (int)((item_off[j + 1] - item_off[j]) / ch) : 0;
-    for (int ci = threadIdx.x; ci < ch; ci += blockDim.x) {
-        int64_t tc = chunk_off[j] + ci;
-        int t0 = begin[b] + ci * kTargetsPerItem;
-        int t1 = min(begin[b] + nb, t0 + kTargetsPerItem);
-        int64_t first = item_off[j] + (int64_t)ci * segs;
-        tc_item0[tc] = (int)first;
-        tc_t0[tc] = t0;
-        tc_t1[tc] = t1;
-        tc_batch[tc] = b;
-        int s = 0, acc = 0;
-        int64_t e0 = eoff[j];
-        for (int64_t e = eoff[j]; e < eoff[j + 1]; e++) {
-            acc += padded(ent[e].src1 - ent[e].src0);
-            bool last = e + 1 == eoff[j + 1];
-            if (acc >= seg_src || last) {
-                if (s < segs) items[first + s] = Item{t0, t1, (int)e0, (int)(e + 1), b, (int)tc, (int)first, segs};
-                s++;
-                acc = 0;
-                e0 = e + 1;
-            }
+    const int b = leaves[j];
+    const int nb = end[b] - begin[b];
+    const int64_t c0 = chunk_off[j], i0 = item_off[j], e0 = eoff[j], e1 = eoff[j + 1];
+    const int ch = (int)(chunk_off[j + 1] - c0);
+    const int segs = (int)((item_off[j + 1] - i0) / ch);
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x;
+        int64_t at = 0, prev = -1;  // start of this round's first entry; of the unit before it
+        if (e0 == e1 && lane == 0) {
+            items[i0].e0 = (int)e0;
+            items[i0].skip = 0;
         }
-        for (; s < segs; s++)
-            items[first + s] = Item{t0, t1, (int)eoff[j + 1], (int)eoff[j + 1], b, (int)tc, (int)first, segs};
+        for (int64_t base = e0; base < e1; base += 32) {
+            const int64_t e = base + lane;
+            const Entry x = e < e1 ? ent[e] : Entry{0, 0, 0, 2};
+            const int len = padded(x.src1 - x.src0);
+            int64_t incl = len;
+            for (int o = 1; o < 32; o <<= 1) {
+                const int64_t v = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += v;
+            }
+            const int64_t a = at + incl - len, last = a + (e < e1 ? last_unit(x) : 0);
+            int64_t before = __shfl_up_sync(0xffffffffu, last, 1);
+            if (lane == 0) before = prev;
+            if (e < e1)
+                for (int64_t s = before < 0 ? 0 : before / seg + 1; s <= last / seg && s < segs; s++) {
+                    const int64_t off = s * seg - a;  // first unit at or after off
+                    items[i0 + s].e0 = (int)e;
+                    items[i0 + s].skip = off <= 0 ? 0 : (int)((off + kItemUnit - 1) / kItemUnit * kItemUnit);
+                }
+            const int m = (int)min((int64_t)31, e1 - 1 - base);
+            prev = __shfl_sync(0xffffffffu, last, m);
+            at = __shfl_sync(0xffffffffu, a + len, m);
+        }
+    }
+    __syncthreads();
+    for (int q = threadIdx.x; q < ch * segs; q += blockDim.x) {
+        const int ci = q / segs, s = q % segs;
+        const int64_t tc = c0 + ci;
+        const int t0 = begin[b] + ci * kTargetsPerItem, t1 = min(begin[b] + nb, t0 + kTargetsPerItem);
+        const int64_t first = i0 + (int64_t)ci * segs;
+        int f0 = items[i0 + s].e0, skip = items[i0 + s].skip, f1 = (int)e1, stop = 0;
+        if (s + 1 < segs) {  // up to where the next segment starts
+            f1 = items[i0 + s + 1].e0;
+            stop = items[i0 + s + 1].skip;
+            if (stop > 0) f1++;
+        }
+        Item& it = items[first + s];
+        it.t0 = t0;
+        it.t1 = t1;
+        it.e1 = f1;
+        it.stop = stop;
+        it.batch = b;
+        it.tchunk = (int)tc;
+        it.i0 = (int)first;
+        it.ni = segs;
+        if (ci > 0) {
+            it.e0 = f0;
+            it.skip = skip;
+        }
+        if (s == 0) {
+            tc_item0[tc] = (int)first;
+            tc_t0[tc] = t0;
+            tc_t1[tc] = t1;
+            tc_batch[tc] = b;
+        }
     }
 }
 
@@ -1003,13 +1061,28 @@ void build_tree(Tree& T, const double* xyz, const double* w)
     TAGI_LAUNCH_CHECK();
 
     // ---- work items of the near/far kernel
-    const int seg_src = T.segment;
+    // Sources per item.  Where the caller leaves it open: short enough for
+    // kItemsWanted items (nine waves of 152 SMs at 6 CTAs), so that the SMs end
+    // together, and not shorter than a unit.  With one length of 8192 the 5,003
+    // point cube ran 64 CTAs over 5,003 sources each: 204 us, 91 with this
+    // rule; the uniform hydrogen mesh 663 -> 498 us.  At most kSegmentMax: an
+    // item of 8192 sources runs about a millisecond, and the last ones leave
+    // SMs idle.  1024 / 2048 / 4096 / 8192 gave 38.93 / 38.75 / 38.76 / 38.93
+    // ms for the Li step, 26.89 / 26.91 / 27.14 / 27.66 for three H2
+    // iterations and 252.8 / 251.0 / 250.4 / 250.5 for the CO fields.
+    const int unit = std::max(kItemUnit, padded(T.P));
+    int seg = T.segment;
+    if (seg == 0) {
+        const int64_t rows = (T.near_pairs + T.far_pairs) / kTargetsPerItem;
+        seg = (int)std::min<int64_t>(std::max<int64_t>(rows / kItemsWanted, unit), kSegmentMax);
+    }
+    const int seg_src = std::max(seg, unit);
     DevBuf nch, nit, choff, itoff;
     nch.ensure(8 * (size_t)nleaf);
     nit.ensure(8 * (size_t)nleaf);
     choff.ensure(8 * ((size_t)nleaf + 1));
     itoff.ensure(8 * ((size_t)nleaf + 1));
-    launch(k_item_counts, nblocks(nleaf, 128), 128, 0, s, nleaf, T.leaves.as<int>(), T.cl_begin.as<int>(),
+    launch(k_item_counts, nblocks(32 * (int64_t)nleaf, 128), 128, 0, s, nleaf, T.leaves.as<int>(), T.cl_begin.as<int>(),
                                                       T.cl_end.as<int>(), T.ent_off.as<int64_t>(), T.ent.as<Entry>(),
                                                       seg_src, nch.as<int64_t>(), nit.as<int64_t>());
     exclusive_scan_i64(nch.as<int64_t>(), choff.as<int64_t>(), nleaf, s);
@@ -1022,7 +1095,7 @@ void build_tree(Tree& T, const double* xyz, const double* w)
     T.tc_t0.ensure(4 * (size_t)T.ntchunk);
     T.tc_t1.ensure(4 * (size_t)T.ntchunk);
     T.tc_batch.ensure(4 * (size_t)T.ntchunk);
-    launch(k_item_fill, nleaf, 32, 0, s, nleaf, T.leaves.as<int>(), T.cl_begin.as<int>(),
+    launch(k_item_fill, nleaf, 128, 0, s, nleaf, T.leaves.as<int>(), T.cl_begin.as<int>(),
                                                     T.cl_end.as<int>(), T.ent_off.as<int64_t>(), T.ent.as<Entry>(),
                                                     seg_src, choff.as<int64_t>(), itoff.as<int64_t>(),
                                                     T.items.as<Item>(), T.tc_item0.as<int>(), T.tc_t0.as<int>(),

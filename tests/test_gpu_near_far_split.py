@@ -59,3 +59,22 @@ def test_far_field_over_groups(T, degree, leaf):
 
 def test_without_subtraction(T):
     check(T, 5003, 90, 6, seed=4, ss=False)
+
+
+@pytest.mark.parametrize("prec", ["FP32C", "FP64"])
+@pytest.mark.parametrize("n,leaf,degree", [(12007, 3000, 8), (12007, 333, 6), (3001, 4000, 9)])
+def test_items_may_cut_an_entry(T, n, leaf, degree, prec):
+    """The item length regroups whole folds of 16 sources: two-float sums
+    (2^-48 of the partial sums a fold, about 1e3 folds, SS cancellation of at
+    most 1e2 on the cube) and float64 ones move by less than 1e-9."""
+    xyz, w = W.random_cube(n, seed=7)
+    f = 1.0 + 0.3 * np.sin(3 * xyz[0]) * np.cos(2 * xyz[1])
+    out = []
+    for segment in (0, 1024, 65536):
+        with T.Tree(dev(xyz), dev(w), theta=0.6, degree=degree, leaf_size=leaf, prec=getattr(T, "TAGI_" + prec),
+                    segment=segment) as tr:
+            u = torch.empty((1, n), dtype=torch.float64, device="cuda")
+            T.tagi_yukawa_conv(tr.handle, dev(f), [2.3], u)
+            out.append(u.cpu().numpy()[0])
+    for a in out[:2]:
+        assert np.linalg.norm(a - out[2]) <= 1e-9 * np.linalg.norm(out[2])
