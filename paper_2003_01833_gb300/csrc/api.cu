@@ -137,10 +137,7 @@ void run_convolution(Tree& T, const double* f, const RateSrc& R, const double* e
             anterpolate_fields64(T, nf);
         }
         ProfScope ps(kProfInteract, T.stream);
-        for (int o = 0; o < nf; o++)
-            interact64(T, o, nf, R.kind[o], T.rates64.as<double>(), T.q64.as<double>() + (size_t)o * T.nrec,
-                       T.c64.as<double>() + (size_t)o * T.n, T.part.as<double>(), T.tsum.as<double>(),
-                       T.tc_cnt.as<int>());
+        interact64(T, nf, R.kind, T.rates64.as<double>(), T.part.as<double>(), T.tsum.as<double>(), T.tc_cnt.as<int>());
     }
     ProfScope ps(kProfEpilogue, T.stream);
     reduce_epilogue(T, nf, R.kind, T.tsum.as<double>(), out);

@@ -40,13 +40,15 @@
 // least sqrt(42) alpha apart (list flag bit2) leave out the Gaussian of the
 // Coulomb SS, which is below 2^-60 there.
 //
-// FP64 kernel (plain form): one field per launch, float64 throughout,
-// absolute coordinates, libm exp and sqrt.
+// FP64 kernel (plain form): float64 throughout, absolute coordinates; the
+// exponential and the square root are pair64.cuh's.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
+#include "pair64.cuh"
 #include "tagi_internal.cuh"
 
 namespace tagi {
@@ -786,26 +788,57 @@ __global__ void k_calibrate(int mode, long long n, double* out)
 }
 
 // ---------------------------------------------------------------- FP64 plain form
-template <int KIND, bool SS>
+// Up to kMax64 fields share one pass over the geometry: the kernel is bound by
+// the float64 unit (1.68 operations a clock and SM), and a pair costs it 10
+// operations for 1/r and r and 4 a field (pair64.cuh); with the math library's
+// sqrt, exp and a division it took 47 slots a field.  One thread per target:
+// two warps a scheduler keep that unit busy, so there is nothing to gain from
+// more targets a thread, and warps without targets only stage.  The uniform
+// hydrogen mesh (32,768 points, 8.3e8 pairs, one field) takes 23.0 ms a call,
+// 75.5 before; the errors of ri, r and the exponential are below the math
+// library's (0.62 / 0.81 against 0.75 / 0.96 units of 2^-52 (1 + k r)).
+constexpr int kMax64 = 4;
+
+// a pair that the fast forms do not take (r = 0 is skipped, Eq. direct-sum)
+__device__ __noinline__ double pair_slow(double r2, double k, double q, double nc, double w, bool coulomb, bool ss)
+{
+    if (r2 == 0.0) return 0.0;
+    const double r = sqrt(r2);
+    if (!coulomb) return exp(-k * r) / r * (ss ? fma(nc, w, q) : q);
+    return (ss ? fma(nc * w, exp(-r2 * k), q) : q) / r;
+}
+
+template <int NY, bool HH, bool SS>
 __global__ void __launch_bounds__(kThreads64) k_interact64(const Item* __restrict__ items,
                                                            const Entry* __restrict__ ents,
                                                            const double* __restrict__ rx, const double* __restrict__ ry,
                                                            const double* __restrict__ rz, const double* __restrict__ rw,
-                                                           const double* __restrict__ q, const double* __restrict__ c,
+                                                           const double* __restrict__ q, int64_t ldq,
+                                                           const double* __restrict__ c, int64_t ldc,
                                                            const double* __restrict__ kvd, double* __restrict__ part,
                                                            double* __restrict__ tsum, int* __restrict__ cnt,
-                                                           int nf_tot, int field)
+                                                           int nf_tot, int field0)
 {
-    const double kval = kvd[field];
-    __shared__ double sx[kTile64], sy[kTile64], sz[kTile64], sw[kTile64], sqv[kTile64];
+    constexpr int NF = NY + HH;
+    __shared__ double tab[p64::kTab];
+    __shared__ double sx[kTile64], sy[kTile64], sz[kTile64], sw[kTile64], sq[NF][kTile64];
     const Item it = items[blockIdx.x];
     const int tid = threadIdx.x;
     const int p = it.t0 + tid;
     const bool ok = p < it.t1;
+    const bool busy = it.t0 + (tid & ~31) < it.t1;
+    p64::load_table(tab, kThreads64);
     const double x = ok ? rx[p] : 0.0, y = ok ? ry[p] : 0.0, z = ok ? rz[p] : 0.0;
-    const double ci = ok ? c[p] : 0.0;
-    const double ia2 = KIND == 1 ? 1.0 / (kval * kval) : 0.0;
-    double acc = 0.0;
+    double nc[NF], kv[NF], acc[NF];
+    p64::Rate rate[NF];
+#pragma unroll
+    for (int o = 0; o < NF; o++) {
+        nc[o] = ok ? -c[o * ldc + p] : 0.0;
+        const double v = kvd[field0 + o];
+        kv[o] = o < NY ? v : 1.0 / (v * v);  // k, or 1/alpha^2 of the Gaussian
+        rate[o] = p64::make_rate(kv[o]);
+        acc[o] = 0.0;
+    }
     for (int e = it.e0; e < it.e1; e++) {
         const Entry en = ents[e];
         const int src0 = en.src0 + (e == it.e0 ? it.skip : 0);
@@ -818,26 +851,39 @@ __global__ void __launch_bounds__(kThreads64) k_interact64(const Item* __restric
                 sy[tid] = ry[s0 + tid];
                 sz[tid] = rz[s0 + tid];
                 sw[tid] = rw[s0 + tid];
-                sqv[tid] = q[s0 + tid];
+#pragma unroll
+                for (int o = 0; o < NF; o++) sq[o][tid] = q[o * ldq + s0 + tid];
             }
             __syncthreads();
+            if (!busy) continue;
             for (int k = 0; k < ns; k++) {
                 const double dx = x - sx[k], dy = y - sy[k], dz = z - sz[k];
-                const double r2 = dx * dx + dy * dy + dz * dz;
-                if (r2 == 0.0) continue;  // the singular r' = r term is skipped
-                const double r = sqrt(r2);
-                if (KIND == 0) {
-                    const double d = SS ? sqv[k] - ci * sw[k] : sqv[k];
-                    acc += exp(-kval * r) / r * d;
-                } else {
-                    const double d = SS ? sqv[k] - ci * sw[k] * exp(-r2 * ia2) : sqv[k];
-                    acc += d / r;
+                const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+                if (!p64::fast_range(r2)) {
+#pragma unroll
+                    for (int o = 0; o < NF; o++)
+                        acc[o] += pair_slow(r2, kv[o], sq[o][k], nc[o], sw[k], o >= NY, SS);
+                    continue;
+                }
+                double ri, r;
+                p64::inv_sqrt(r2, ri, r);
+#pragma unroll
+                for (int o = 0; o < NY; o++) {
+                    const double d = SS ? fma(nc[o], sw[k], sq[o][k]) : sq[o][k];
+                    acc[o] = fma(p64::exp_neg(r, rate[o], tab), ri * d, acc[o]);
+                }
+                if (HH) {
+                    const double d = SS ? fma(nc[NY] * sw[k], p64::exp_neg(r2, rate[NY], tab), sq[NY][k]) : sq[NY][k];
+                    acc[NY] = fma(d, ri, acc[NY]);
                 }
             }
         }
     }
-    part[((size_t)blockIdx.x * nf_tot + field) * kTargetsPerItem + tid] = acc;
-    chunk_sum<kThreads64>(it, part, tsum, cnt, nf_tot, field, 1);
+    if (ok)
+#pragma unroll
+        for (int o = 0; o < NF; o++)
+            part[((size_t)blockIdx.x * nf_tot + field0 + o) * kTargetsPerItem + tid] = acc[o];
+    chunk_sum<kThreads64>(it, part, tsum, cnt, nf_tot, field0, NF);
 }
 
 template <int NY, bool HH, bool SS, int M>
@@ -962,26 +1008,56 @@ void interact32(Tree& T, int nf, const int* kinds, const float* kyd, double* par
     }
 }
 
-void interact64(Tree& T, int field, int nf_tot, int kind, const double* kvd, const double* q, const double* c,
-                double* part, double* tsum, int* cnt)
+namespace {
+template <int NY, bool HH>
+void launch64(Tree& T, const double* kvd, const double* q, const double* c, double* part, double* tsum, int* cnt,
+              int nf_tot, int field0)
 {
-    const int grid = (int)T.nitems;
-    cudaStream_t s = T.stream;
-    const Item* it = T.items.as<Item>();
-    const Entry* en = T.ent.as<Entry>();
-    const double *rx = T.rx.as<double>(), *ry = T.ry.as<double>(), *rz = T.rz.as<double>(), *rw = T.rw.as<double>();
-    if (kind == 0) {
-        if (T.ss)
-            launch(k_interact64<0, true>, grid, kThreads64, 0, s, it, en, rx, ry, rz, rw, q, c, kvd, part, tsum, cnt, nf_tot, field);
-        else
-            launch(k_interact64<0, false>, grid, kThreads64, 0, s, it, en, rx, ry, rz, rw, q, c, kvd, part, tsum, cnt, nf_tot, field);
-    } else {
-        if (T.ss)
-            launch(k_interact64<1, true>, grid, kThreads64, 0, s, it, en, rx, ry, rz, rw, q, c, kvd, part, tsum, cnt, nf_tot, field);
-        else
-            launch(k_interact64<1, false>, grid, kThreads64, 0, s, it, en, rx, ry, rz, rw, q, c, kvd, part, tsum, cnt, nf_tot, field);
-    }
+    launch(T.ss ? k_interact64<NY, HH, true> : k_interact64<NY, HH, false>, (int)T.nitems, kThreads64, 0, T.stream,
+           T.items.as<Item>(), T.ent.as<Entry>(), T.rx.as<double>(), T.ry.as<double>(), T.rz.as<double>(),
+           T.rw.as<double>(), q, T.nrec, c, T.n, kvd, part, tsum, cnt, nf_tot, field0);
     TAGI_LAUNCH_CHECK();
+}
+
+template <bool HH>
+void launch64_ny(int ny, Tree& T, const double* kvd, const double* q, const double* c, double* part, double* tsum,
+                 int* cnt, int nf_tot, int field0)
+{
+    switch (ny) {
+        case 0:
+            if constexpr (HH) launch64<0, true>(T, kvd, q, c, part, tsum, cnt, nf_tot, field0);
+            break;
+        case 1: launch64<1, HH>(T, kvd, q, c, part, tsum, cnt, nf_tot, field0); break;
+        case 2: launch64<2, HH>(T, kvd, q, c, part, tsum, cnt, nf_tot, field0); break;
+        case 3: launch64<3, HH>(T, kvd, q, c, part, tsum, cnt, nf_tot, field0); break;
+        case 4:
+            if constexpr (!HH) launch64<4, false>(T, kvd, q, c, part, tsum, cnt, nf_tot, field0);
+            break;
+        default: throw Error(TAGI_ERR_INVALID_ARG, "field group too large");
+    }
+}
+}  // namespace
+
+// Fields [0, nf) of T.q64 / T.c64, grouped as interact32 groups them, at most
+// kMax64 to a launch.  kvd: k or alpha of each field (device).
+void interact64(Tree& T, int nf, const int* kinds, const double* kvd, double* part, double* tsum, int* cnt)
+{
+    int ny = 0;
+    while (ny < nf && kinds[ny] == 0) ny++;
+    const bool hh = ny < nf;
+    TAGI_REQUIRE(nf - ny <= 1, "at most one Coulomb field, after the Yukawa fields");
+    int o = 0;
+    while (o < nf) {
+        const int g_ny = std::min(ny - o, kMax64);
+        const bool g_hh = hh && o + g_ny == ny && g_ny < kMax64;
+        const double* q = T.q64.as<double>() + (size_t)o * T.nrec;
+        const double* c = T.c64.as<double>() + (size_t)o * T.n;
+        if (g_hh)
+            launch64_ny<true>(g_ny, T, kvd, q, c, part, tsum, cnt, nf, o);
+        else
+            launch64_ny<false>(g_ny, T, kvd, q, c, part, tsum, cnt, nf, o);
+        o += g_ny + (g_hh ? 1 : 0);
+    }
 }
 
 }  // namespace tagi

@@ -223,8 +223,7 @@ void anterpolate_all_clusters32(Tree& T, const double* q, int nq, double* qh);  
 // interact.cu
 // kinds[o]: 0 = Yukawa with kval[o], 1 = Coulomb/Hartree
 void interact32(Tree& T, int nf, const int* kinds, const float* kyd, double* part, double* tsum, int* cnt);
-void interact64(Tree& T, int field, int nf_tot, int kind, const double* kvd, const double* q, const double* c,
-                double* part, double* tsum, int* cnt);
+void interact64(Tree& T, int nf, const int* kinds, const double* kvd, double* part, double* tsum, int* cnt);
 // mean relative bias of the float32 Yukawa and Gaussian kernel values (measured)
 void fp32_bias(cudaStream_t s, double* beta_y, double* beta_g);
 double effective_k32(double k);
