@@ -17,6 +17,8 @@
 #include <new>
 #include <string>
 
+#include "bf16.cuh"
+#include "mlp64.cuh"
 #include "tagi_internal.cuh"
 
 namespace tagi {
@@ -47,24 +49,6 @@ struct Nuclei {
     int ordered;  // 1: two nuclei taken in list order (r1 to the first) instead of by distance
 };
 
-// Nearest bfloat16 value of x, ties to even, from the float64 value: x / q
-// with q the spacing of bfloat16 values at x (a power of two, so exact),
-// rounded to an integer half-to-even, scaled back.  The result has 8
-// significant bits within float32's exponent range, so the float32
-// conversion is exact and its high half is the bfloat16 encoding.
-__device__ __forceinline__ uint16_t bf16_bits(double x)
-{
-    if (isnan(x)) return 0x7FC0;
-    if (x == 0.0) return signbit(x) ? 0x8000 : 0;
-    int e;
-    frexp(x, &e);
-    const double q = ldexp(1.0, max(e - 8, -133));
-    const double r = rint(x / q) * q;
-    return (uint16_t)(__float_as_uint((float)r) >> 16);
-}
-
-__device__ __forceinline__ float bf16_float(uint32_t b) { return __uint_as_float(b << 16); }
-
 __device__ __forceinline__ bool is_weight(int e)
 {
     return (e >= oW1 && e < oB1) || (e >= oW2 && e < oB2) || (e >= oW3 && e < oB3);
@@ -74,7 +58,7 @@ __device__ __forceinline__ bool is_weight(int e)
 __device__ __forceinline__ void load_params(float* sw, const double* __restrict__ master)
 {
     for (int e = threadIdx.x; e < kP; e += blockDim.x)
-        sw[e] = is_weight(e) ? bf16_float(bf16_bits(master[e])) : (float)master[e];
+        sw[e] = is_weight(e) ? bf16_float(bf16_of_double(master[e])) : (float)master[e];
 }
 
 __device__ __forceinline__ void load_x(const uint16_t* __restrict__ feat, int64_t i, float x[kF])
@@ -153,7 +137,7 @@ __global__ void k_features(const double* __restrict__ xyz, int64_t n, Nuclei nuc
                           exp(-__dsub_rn(s12, R))};
     uint32_t u[4];
 #pragma unroll
-    for (int k = 0; k < 4; k++) u[k] = (uint32_t)bf16_bits(f[2 * k]) | ((uint32_t)bf16_bits(f[2 * k + 1]) << 16);
+    for (int k = 0; k < 4; k++) u[k] = (uint32_t)bf16_of_double(f[2 * k]) | ((uint32_t)bf16_of_double(f[2 * k + 1]) << 16);
     *reinterpret_cast<uint4*>(feat + i * kF) = make_uint4(u[0], u[1], u[2], u[3]);
 }
 
@@ -312,18 +296,34 @@ __global__ void __launch_bounds__(kThreads) k_mlp_grad(const uint16_t* __restric
     }
 }
 
-// Gradient and loss from the per-block partials [nblk][np + 1] (block
-// order), then, if apply, one Adam step on the float64 master weights
-// (c1 = 1 - beta1^t, c2 = 1 - beta2^t).
-__global__ void k_mlp_adam(const double* __restrict__ partial, int nblk, int np, double* __restrict__ master,
-                           double* __restrict__ m, double* __restrict__ v, double lr, double beta1, double beta2,
-                           double eps, double c1, double c2, int apply, double* __restrict__ grad_out,
-                           double* __restrict__ loss_out)
+// Gradient and loss from the per-block partials [nblk][np + 1], then, if
+// apply, one Adam step on the float64 master weights (c1 = 1 - beta1^t, c2 =
+// 1 - beta2^t).  A block sums 32 entries, each by kAdamSlices threads over
+// every kAdamSlices-th row whose sums are then added in order: one thread
+// alone waits for one row after another (38 us for 304 rows).  tc: the rows
+// are in the order of mlp64.cuh.
+constexpr int kAdamSlices = 16;
+__global__ void __launch_bounds__(32 * kAdamSlices) k_mlp_adam(const double* __restrict__ partial, int nblk, int np,
+                                                               int tc, double* __restrict__ master,
+                                                               double* __restrict__ m, double* __restrict__ v,
+                                                               double lr, double beta1, double beta2, double eps,
+                                                               double c1, double c2, int apply,
+                                                               double* __restrict__ grad_out,
+                                                               double* __restrict__ loss_out)
 {
-    const int e = blockIdx.x * blockDim.x + threadIdx.x;
-    if (e > np) return;
+    __shared__ double part[kAdamSlices][32];
+    const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
+    const int e = blockIdx.x * 32 + lane;
     double g = 0.0;
-    for (int b = 0; b < nblk; b++) g += partial[(size_t)b * (np + 1) + e];
+    if (e <= np) {
+        const double* row = partial + (tc ? mlp64::slot(e) : e);
+        for (int b = slice; b < nblk; b += kAdamSlices) g += row[(size_t)b * (np + 1)];
+    }
+    part[slice][lane] = g;
+    __syncthreads();
+    if (slice > 0 || e > np) return;
+#pragma unroll
+    for (int q = 1; q < kAdamSlices; q++) g += part[q][lane];
     if (e == np) {
         *loss_out = g;
         return;
@@ -431,7 +431,7 @@ void grad_pass(Mlp& M, const uint16_t* feat, const float* target, const float* w
     const int grid = M.H == 64 ? mlp64_grad_grid(n, M.sms) : grad_grid(M, n);
     M.partial.ensure(sizeof(double) * (size_t)grid * (M.np + 1));
     if (M.H == 64)
-        mlp64_gradient(feat, target, wt, n, M.master.as<double>(), M.partial.as<double>(), grid, M.errd.as<int>(), s);
+        mlp64_gradient(feat, target, wt, n, M.master.as<double>(), M.partial.as<double>(), M.sms, M.errd.as<int>(), s);
     else
         launch(k_mlp_grad, grid, kThreads, kGradSmem, s, feat, target, wt, n, M.master.as<double>(),
                M.partial.as<double>());
@@ -445,8 +445,8 @@ void grad_pass(Mlp& M, const uint16_t* feat, const float* target, const float* w
         c1 = 1.0 - std::pow(b1, (double)M.step);
         c2 = 1.0 - std::pow(b2, (double)M.step);
     }
-    launch(k_mlp_adam, (M.np + 1 + 127) / 128, 128, 0, s, M.partial.as<double>(), grid, M.np, M.master.as<double>(),
-           M.m.as<double>(), M.v.as<double>(), lr, b1, b2, eps, c1, c2, apply ? 1 : 0, M.grad.as<double>(),
+    launch(k_mlp_adam, M.np / 32 + 1, 32 * kAdamSlices, 0, s, M.partial.as<double>(), grid, M.np, M.H == 64 ? 1 : 0,
+           M.master.as<double>(), M.m.as<double>(), M.v.as<double>(), lr, b1, b2, eps, c1, c2, apply ? 1 : 0, M.grad.as<double>(),
            M.loss.as<double>());
     TAGI_LAUNCH_CHECK();
 }

@@ -13,27 +13,41 @@
 //   dW1 = sum bf16(dz1) x^T,        db1 = sum bf16(dz1),
 //   dW3 = sum bf16(dy) bf16(h2),    db3 = sum bf16(dy).
 //
-// One CTA of four warpgroups (512 threads) per SM, persistent over 128-point
-// tiles.  Point p of a tile is TMEM lane p of the per-point products, and
-// warpgroup g handles hidden units [16 g, 16 g + 16) of every point (a warp
-// reads its own 32-lane quarter of TMEM, so thread 128 g + p owns point p's
-// units of block g).  Four warps per scheduler hide the latency of the
-// activation work (tanh, rounding, operand stores), which is what bounds a
-// tile; the products are:
+// Tiles of 128 points; point p of a tile is TMEM lane p of the per-point
+// products, and warpgroup g of a CTA's two handles hidden units [32 g, 32 g +
+// 32) of every point (a warp reads its own 32-lane quarter of TMEM).  The
+// products are
 //   Z1 = X W1^T           (M 128 points, N 64, K 16: features padded)
 //   Z2 = H1 W2^T          (M 128, N 64, K 64)
 //   dH1 = dZ2 W2          (M 128, N 64, K 64)
-// and the weight gradients are contractions over the tile's points,
-// accumulated in TMEM over up to kFold tiles:
-//   D1 = [dZ2^T; dZ1^T] [H1^T; X^T; 1]^T   (M 128 = 64 + 64, N 80, K 128)
-//   D2 = [H2^T; 1] [dy]^T                  (M 128, N 16, K 128)
-// then added to the CTA's float64 partial row in global memory (each entry
-// is one TMEM lane and column, read by one thread: one writer).  All operand tiles are
-// K-major with the 128-byte swizzle (64 bf16 per row); an operand with K =
-// 128 points is two such tiles.  Every wait is bounded; one that gives up
-// sets *err and the CTA returns after a bounded wait for its MMAs.
+// and the weight gradients contractions over the tile's points, accumulated
+// in TMEM over up to kFold tiles:
+//   D1 = [dZ2 dZ1]^T [H1 X 1]   (M 128 = 64 + 64, N 128 of which 73 are used, K 128)
+//   D2 = [H2 X 1]^T dy          (M 128 of which 65 are used, N 16, K 128)
+// then added to a float64 partial row in global memory.
+//
+// What bounds it: a tile is a chain of four products with the activations of
+// 128 points between them, about 3,500 issue slots a scheduler (64 accurate
+// tanh a unit pair), so the tensor pipe idles and latency shows.  Every
+// activation is stored once, one 128-byte row of 64 units a point with the
+// 128-byte swizzle, in 16-byte pieces: read along its rows it is the K-major A
+// operand of the next product, read across (MN-major) the operand of the
+// weight gradients, whose K are the points; W2 likewise serves Z2 and dH1.
+// That takes 100 KB, so two CTAs share an SM and one computes while the other
+// waits.  With transposed copies stored value by value (160 KB, one CTA of 512
+// threads) a training step over 10.9M points took 4.63 ms, now 1.77 (131 and 50
+// SM clocks a point), the same bits.
+//
+// The float32 sums in TMEM are those of one CTA per SM: virtual CTA v owns
+// tiles v, v + V, ..., in groups of kFold, and the two CTAs of an SM's worth of
+// work take its groups in turn (mlp64_plan).
+//
+// Every wait is bounded; one that gives up sets *err and the CTA returns after
+// a bounded wait for its MMAs.
 #include <cuda_runtime.h>
 
+#include "bf16.cuh"
+#include "mlp64.cuh"
 #include "tagi_internal.cuh"
 #include "tc.cuh"
 
@@ -41,58 +55,48 @@ namespace tagi {
 
 namespace {
 
-constexpr int kF = 8;
-constexpr int kH = 64;
-constexpr int oW1 = 0, oB1 = kH * kF, oW2 = oB1 + kH, oB2 = oW2 + kH * kH, oW3 = oB2 + kH, oB3 = oW3 + kH;
-constexpr int kP64 = oB3 + 1;  // 4801 parameters
+using namespace mlp64;
 constexpr int kT = 128;        // points per tile
-constexpr int kWG = 4;         // warpgroups per CTA
-constexpr int kCB = 64 / kWG;  // hidden units per warpgroup
+constexpr int kWG = 2;         // warpgroups per CTA
+constexpr int kCB = 64 / kWG;  // hidden units per thread
 constexpr int kThreads = kT * kWG;
 constexpr int kFold = 8;       // tiles accumulated in tensor memory between float64 folds
 constexpr long long kWait = 2000000000LL;
-constexpr uint32_t kCols = 512;
 
-// byte layout of the shared memory (every tile 1024-aligned)
-constexpr int sX = 0;                    // 128 rows (points) x 128 B: features 0..7, zeros
-constexpr int sW1 = sX + 128 * 128;      // 64 rows (units) x 128 B: W1 row, zeros
+// byte layout of the shared memory (every tile 1024-aligned).  Point tiles:
+// 128 rows x 128 B.
+constexpr int kPointTile = 128 * 128;
+constexpr int sDZ2 = 0;                  // bf16(dz2)
+constexpr int sDZ1 = sDZ2 + kPointTile;  // bf16(dz1)
+constexpr int sH2 = sDZ1 + kPointTile;   // bf16(h2)
+constexpr int sB2 = sH2 + kPointTile;    // 2 tiles of 16 rows ([dy; 0]) x 64 points
+constexpr int sFwd = sB2 + 2 * 16 * 128; // from here on: what the forward pass needs
+constexpr int sH1 = sFwd;                // bf16(h1)
+constexpr int sX = sH1 + kPointTile;     // features 0..7, 1, zeros
+constexpr int sW1 = sX + kPointTile;     // 64 rows (units) x 128 B: W1 row, zeros
 constexpr int sW2 = sW1 + 64 * 128;      // 64 rows (out j) x 64 (in i)
-constexpr int sW2T = sW2 + 64 * 128;     // 64 rows (in i) x 64 (out j)
-constexpr int sH1 = sW2T + 64 * 128;     // 128 rows (points) x 64 (i): bf16(h1)
-constexpr int sDZ2 = sH1 + 128 * 128;    // 128 rows (points) x 64 (j): bf16(dz2)
-constexpr int sAT = sDZ2 + 128 * 128;    // 2 tiles of 128 rows ([dz2 j; dz1 i]) x 64 points
-constexpr int sBT = sAT + 2 * 128 * 128; // 2 tiles of 80 rows ([h1 i; x f; 1; 0]) x 64 points
-constexpr int sA2 = sBT + 2 * 80 * 128;  // 2 tiles of 128 rows ([h2 k; 1; 0]) x 64 points
-constexpr int sB2 = sA2 + 2 * 128 * 128; // 2 tiles of 16 rows ([dy; 0]) x 64 points
-constexpr int kSmem = sB2 + 2 * 16 * 128;
-constexpr int kSmemAlloc = kSmem + 1024;
+constexpr int kSmem = sW2 + 64 * 128;
+static_assert(sFwd % 1024 == 0, "tiles are 1024-aligned");
 // TMEM columns
-constexpr uint32_t cZ1 = 0, cZ2 = 64, cDH1 = 128, cD1 = 192, cD2 = 272;
+constexpr uint32_t cZ = 0, cD1 = 64, cD2 = 192;
 
 __device__ __forceinline__ uint32_t swz2(int r, int k)  // bf16 element k of row r, 128B swizzle
 {
     return r * 128 + ((((k >> 3) ^ (r & 7))) << 4) + ((k & 7) << 1);
 }
 
-__device__ __forceinline__ uint16_t bf16_rn(float x)  // nearest, ties to even (finite x)
-{
-    const uint32_t u = __float_as_uint(x);
-    return (uint16_t)((u + 0x7FFFu + ((u >> 16) & 1u)) >> 16);
-}
-
-__device__ __forceinline__ float bf16_f(uint16_t b) { return __uint_as_float((uint32_t)b << 16); }
-
-// nearest bfloat16 of a float64 value, ties to even, as the H = 32 kernels round
-__device__ __forceinline__ uint16_t bf16_of_double(double x)
-{
-    if (x == 0.0) return signbit(x) ? 0x8000 : 0;
-    int e;
-    frexp(x, &e);
-    const double q = ldexp(1.0, max(e - 8, -133));
-    return (uint16_t)(__float_as_uint((float)(rint(x / q) * q)) >> 16);
-}
-
 __device__ __forceinline__ void st16(uint8_t* sm, uint32_t off, uint16_t v) { *reinterpret_cast<uint16_t*>(sm + off) = v; }
+
+// units [c0, c0 + N) of row r, rounded to bfloat16
+template <int N>
+__device__ __forceinline__ void store_row(uint8_t* tile, int r, int c0, const float (&v)[N])
+{
+#pragma unroll
+    for (int c = 0; c < N; c += 8)
+        *reinterpret_cast<uint4*>(tile + swz2(r, c0 + c)) =
+            make_uint4(bf16x2(v[c], v[c + 1]), bf16x2(v[c + 2], v[c + 3]), bf16x2(v[c + 4], v[c + 5]),
+                       bf16x2(v[c + 6], v[c + 7]));
+}
 
 struct Bias {
     float b1[kH], b2[kH], w3[kH], b3;
@@ -111,10 +115,11 @@ struct Sync {
     }
 };
 
-__device__ __forceinline__ void mma_chain(uint32_t d, uint32_t a, uint32_t b, int ksteps, uint32_t idesc, bool acc0)
+// A and B K-major, `ksteps` K-steps of 16 from the start of a row
+__device__ __forceinline__ void mma_chain(uint32_t d, uint32_t a, uint32_t b, int ksteps, uint32_t idesc)
 {
     const uint64_t da = tc::sdesc_sw128(a), db = tc::sdesc_sw128(b);
-    for (int k = 0; k < ksteps; k++) tc::mma_bf16(d, da + 2 * k, db + 2 * k, idesc, (k > 0 || acc0) ? 1u : 0u);
+    for (int k = 0; k < ksteps; k++) tc::mma_bf16(d, da + 2 * k, db + 2 * k, idesc, k > 0 ? 1u : 0u);
 }
 
 // the thread's place: point (TMEM lane) pl of the tile, hidden units
@@ -133,114 +138,107 @@ struct Who {
 };
 
 // Weights (bf16 operand tiles) and float32 biases from the float64 master
-// weights; zero every operand tile; the constant rows of the transposed tiles.
-__device__ void setup(uint8_t* sm, Bias* B, const double* __restrict__ master)
+// weights; zero the operand tiles from byte `from` on; the column of ones.
+__device__ void setup(uint8_t* sm, int from, Bias* B, const double* __restrict__ master)
 {
-    for (int e = threadIdx.x; e < kSmem / 16; e += kThreads) reinterpret_cast<uint4*>(sm)[e] = make_uint4(0, 0, 0, 0);
+    for (int e = from / 16 + threadIdx.x; e < kSmem / 16; e += kThreads)
+        reinterpret_cast<uint4*>(sm)[e] = make_uint4(0, 0, 0, 0);
     __syncthreads();
     for (int e = threadIdx.x; e < kH * kF; e += kThreads)
         st16(sm, sW1 + swz2(e / kF, e % kF), bf16_of_double(master[oW1 + e]));
-    for (int e = threadIdx.x; e < kH * kH; e += kThreads) {
-        const int j = e / kH, i = e % kH;
-        const uint16_t v = bf16_of_double(master[oW2 + e]);
-        st16(sm, sW2 + swz2(j, i), v);
-        st16(sm, sW2T + swz2(i, j), v);
-    }
+    for (int e = threadIdx.x; e < kH * kH; e += kThreads)
+        st16(sm, sW2 + swz2(e / kH, e % kH), bf16_of_double(master[oW2 + e]));
     for (int e = threadIdx.x; e < kH; e += kThreads) {
         B->b1[e] = (float)master[oB1 + e];
         B->b2[e] = (float)master[oB2 + e];
-        B->w3[e] = bf16_f(bf16_of_double(master[oW3 + e]));
+        B->w3[e] = bf16_float(bf16_of_double(master[oW3 + e]));
     }
     if (threadIdx.x == 0) B->b3 = (float)master[oB3];
-    // ones rows: BT row 72 (bias of the first layer's gradient), A2 row 64
-    for (int e = threadIdx.x; e < 2 * 64; e += kThreads) {
-        const int t = e / 64, p = e % 64;
-        st16(sm, sBT + t * 80 * 128 + swz2(72, p), 0x3F80);
-        st16(sm, sA2 + t * 128 * 128 + swz2(64, p), 0x3F80);
+    // W1's column 8 is zero, so the ones do not enter Z1
+    for (int e = threadIdx.x; e < kT; e += kThreads) st16(sm, sX + swz2(e, kF), 0x3F80);
+}
+
+// tanh(z + b) of this thread's units of the product in TMEM column cZ
+__device__ __forceinline__ void activate(const Who& w, const float* b, float (&h)[kCB])
+{
+#pragma unroll
+    for (int c = 0; c < kCB; c += 16) {
+        float v[16];
+        tc::tmem_ld16(w.lane_base + cZ + w.c0 + c, v);
+#pragma unroll
+        for (int i = 0; i < 16; i++) h[c + i] = tanhf(v[i] + b[w.c0 + c + i]);
     }
 }
 
-// Forward pass of point p (lane pl) for this warpgroup's units; returns y.
-// h1, h2: this warpgroup's activations of the point (float32), xb: the
-// point's features (warpgroup 0 only).  ypart: [kWG][kT] shared partial
-// sums of W3 . h2, one per warpgroup, added in warpgroup order.
-__device__ float forward_tile(uint8_t* sm, const Bias& B, const uint16_t* __restrict__ feat, int64_t p, bool valid,
-                              const Who& w, uint32_t tmem, Sync& sy, float* ypart, float h1[kCB], float h2[kCB],
-                              uint16_t xb[kF])
+// Forward pass of point pl of the tile whose features xv (warpgroup 0) holds;
+// returns y, false in sy.ok if a wait of any thread gave up.  h1, h2: this
+// thread's activations (float32).  ypart: [4][kT] shared partial sums of
+// W3 . h2 over 16 units each, added in unit order.
+__device__ float forward_tile(uint8_t* sm, const Bias& B, uint4 xv, const Who& w, uint32_t tmem, Sync& sy,
+                              float* ypart, float (&h1)[kCB], float (&h2)[kCB])
 {
-    if (w.g == 0) {
-        uint4 xv = make_uint4(0, 0, 0, 0);
-        if (valid) xv = *reinterpret_cast<const uint4*>(feat + p * kF);
-        const uint32_t xu[4] = {xv.x, xv.y, xv.z, xv.w};
-#pragma unroll
-        for (int k = 0; k < 4; k++) {
-            xb[2 * k] = (uint16_t)(xu[k] & 0xFFFFu);
-            xb[2 * k + 1] = (uint16_t)(xu[k] >> 16);
-        }
-#pragma unroll
-        for (int f = 0; f < kF; f++) st16(sm, sX + swz2(w.pl, f), xb[f]);
+    if (w.g == 0) *reinterpret_cast<uint4*>(sm + sX + swz2(w.pl, 0)) = xv;
+    tc::fence_async_smem();
+    tc::fence_before_sync();
+    sy.ok = __syncthreads_and(sy.ok);
+    if (!sy.ok) return 0.0f;
+    if (w.t == 0) {
+        tc::fence_after_sync();
+        mma_chain(tmem + cZ, tc::smem_u32(sm + sX), tc::smem_u32(sm + sW1), 1, tc::idesc_bf16(128, 64));
+        tc::commit(sy.bar);
     }
+    sy.wait();
+    activate(w, B.b1, h1);
+    store_row<kCB>(sm + sH1, w.pl, w.c0, h1);
     tc::fence_async_smem();
     tc::fence_before_sync();
     __syncthreads();
     if (w.t == 0) {
         tc::fence_after_sync();
-        mma_chain(tmem + cZ1, tc::smem_u32(sm + sX), tc::smem_u32(sm + sW1), 1, tc::idesc_bf16(128, 64), false);
+        mma_chain(tmem + cZ, tc::smem_u32(sm + sH1), tc::smem_u32(sm + sW2), 4, tc::idesc_bf16(128, 64));
         tc::commit(sy.bar);
     }
     sy.wait();
-    // h1 = tanh(z1 + b1) -> bf16 into the second layer's A tile
+    activate(w, B.b2, h2);
 #pragma unroll
-    for (int c = 0; c < kCB; c += 8) {
-        float v[8];
-        tc::tmem_ld8(w.lane_base + cZ1 + w.c0 + c, v);
+    for (int c = 0; c < kCB; c += 16) {
+        float yp = 0.0f;
 #pragma unroll
-        for (int i = 0; i < 8; i++) {
-            h1[c + i] = tanhf(v[i] + B.b1[w.c0 + c + i]);
-            st16(sm, sH1 + swz2(w.pl, w.c0 + c + i), bf16_rn(h1[c + i]));
-        }
+        for (int i = 0; i < 16; i++) yp = fmaf(B.w3[w.c0 + c + i], h2[c + i], yp);
+        ypart[(w.c0 + c) / 16 * kT + w.pl] = yp;
     }
-    tc::fence_async_smem();
     tc::fence_before_sync();
-    __syncthreads();
-    if (w.t == 0) {
-        tc::fence_after_sync();
-        mma_chain(tmem + cZ2, tc::smem_u32(sm + sH1), tc::smem_u32(sm + sW2), 4, tc::idesc_bf16(128, 64), false);
-        tc::commit(sy.bar);
-    }
-    sy.wait();
-    float yp = 0.0f;
-#pragma unroll
-    for (int c = 0; c < kCB; c += 8) {
-        float v[8];
-        tc::tmem_ld8(w.lane_base + cZ2 + w.c0 + c, v);
-#pragma unroll
-        for (int i = 0; i < 8; i++) {
-            h2[c + i] = tanhf(v[i] + B.b2[w.c0 + c + i]);
-            yp = fmaf(B.w3[w.c0 + c + i], h2[c + i], yp);
-        }
-    }
-    ypart[w.g * kT + w.pl] = yp;
     __syncthreads();
     float y = B.b3;
 #pragma unroll
-    for (int q = 0; q < kWG; q++) y += ypart[q * kT + w.pl];
+    for (int q = 0; q < 4; q++) y += ypart[q * kT + w.pl];
     return y;
 }
 
-__global__ void __launch_bounds__(kThreads, 1) k_mlp64_fwd(const uint16_t* __restrict__ feat, int64_t n,
+// features of point p (zeros beyond n)
+__device__ __forceinline__ uint4 load_features(const uint16_t* __restrict__ feat, int64_t p, int64_t n)
+{
+    return p < n ? *reinterpret_cast<const uint4*>(feat + p * kF) : make_uint4(0, 0, 0, 0);
+}
+
+constexpr uint32_t kColsFwd = 64, kColsGrad = 256;
+
+// dynamic shared memory: the tiles from sFwd on (four CTAs of 48 KB fit an SM;
+// 4 x 64 TMEM columns)
+__global__ void __launch_bounds__(kThreads, 2) k_mlp64_fwd(const uint16_t* __restrict__ feat, int64_t n,
                                                            const double* __restrict__ master, float* __restrict__ y,
                                                            int* __restrict__ err)
 {
     extern __shared__ uint8_t raw[];
-    uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
+    uint8_t* sm =
+        reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023)) - sFwd;
     __shared__ Bias B;
     __shared__ uint64_t bar;
     __shared__ uint32_t slot;
-    __shared__ float ypart[kWG * kT];
+    __shared__ float ypart[4 * kT];
     const int t = threadIdx.x;
-    setup(sm, &B, master);
-    if ((t >> 5) == 0) tc::tmem_alloc(&slot, kCols);
+    setup(sm, sFwd, &B, master);
+    if ((t >> 5) == 0) tc::tmem_alloc(&slot, kColsFwd);
     if (t == 0) tc::mbar_init(&bar, 1);
     tc::fence_async_smem();
     tc::fence_before_sync();
@@ -250,12 +248,16 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp64_fwd(const uint16_t* __res
     const Who w(tmem);
     Sync sy{&bar, 0, true};
     const int64_t ntiles = (n + kT - 1) / kT;
-    for (int64_t tile = blockIdx.x; tile < ntiles && __syncthreads_and(sy.ok); tile += gridDim.x) {
+    uint4 next = make_uint4(0, 0, 0, 0);
+    if (w.g == 0) next = load_features(feat, (int64_t)blockIdx.x * kT + w.pl, n);
+    for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
         const int64_t p = tile * kT + w.pl;
+        const uint4 xv = next;
+        if (w.g == 0) next = load_features(feat, p + (int64_t)gridDim.x * kT, n);
         float h1[kCB], h2[kCB];
-        uint16_t xb[kF];
-        const float out = forward_tile(sm, B, feat, p, p < n, w, tmem, sy, ypart, h1, h2, xb);
-        if (w.g == 0 && p < n && sy.ok) y[p] = out;
+        const float out = forward_tile(sm, B, xv, w, tmem, sy, ypart, h1, h2);
+        if (!sy.ok) break;
+        if (w.g == 0 && p < n) y[p] = out;
     }
     if (!__syncthreads_and(sy.ok) && t == 0) {
         atomicOr(err, 1);
@@ -265,29 +267,31 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp64_fwd(const uint16_t* __res
     __syncthreads();
     if ((t >> 5) == 0) {
         tc::fence_after_sync();
-        tc::tmem_dealloc(tmem, kCols);
+        tc::tmem_dealloc(tmem, kColsFwd);
     }
 }
 
-// partial[blockIdx.x][kP64 + 1] (the loss last): this CTA's gradient sums
-__global__ void __launch_bounds__(kThreads, 1) k_mlp64_grad(const uint16_t* __restrict__ feat,
+// partial[blockIdx.x][kParams + 1]: this CTA's gradient sums and loss (in the
+// order of mlp64.cuh).  Block b works for virtual CTA b % V of V, on its groups of
+// kFold tiles b / V, b / V + gridDim.x / V, ...
+__global__ void __launch_bounds__(kThreads, 2) k_mlp64_grad(const uint16_t* __restrict__ feat,
                                                             const float* __restrict__ target,
                                                             const float* __restrict__ wt, int64_t n,
                                                             const double* __restrict__ master,
-                                                            double* __restrict__ partial, int* __restrict__ err)
+                                                            double* __restrict__ partial, int V, int* __restrict__ err)
 {
     extern __shared__ uint8_t raw[];
     uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
     __shared__ Bias B;
     __shared__ uint64_t bar;
     __shared__ uint32_t slot;
-    __shared__ float ypart[kWG * kT];
+    __shared__ float ypart[4 * kT];
     __shared__ double lsum[kT];
     const int t = threadIdx.x;
-    double* out = partial + (size_t)blockIdx.x * (kP64 + 1);
-    for (int e = t; e <= kP64; e += kThreads) out[e] = 0.0;
-    setup(sm, &B, master);
-    if ((t >> 5) == 0) tc::tmem_alloc(&slot, kCols);
+    double* out = partial + (size_t)blockIdx.x * (kParams + 1);
+    for (int e = t; e <= kParams; e += kThreads) out[e] = 0.0;
+    setup(sm, 0, &B, master);
+    if ((t >> 5) == 0) tc::tmem_alloc(&slot, kColsGrad);
     if (t == 0) tc::mbar_init(&bar, 1);
     tc::fence_async_smem();
     tc::fence_before_sync();
@@ -298,107 +302,123 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp64_grad(const uint16_t* __re
     Sync sy{&bar, 0, true};
     double loss = 0.0;
     const int64_t ntiles = (n + kT - 1) / kT;
-    // the tiles of this CTA: blockIdx.x, blockIdx.x + gridDim.x, ...
-    const int64_t mine = ntiles > blockIdx.x ? (ntiles - 1 - blockIdx.x) / gridDim.x + 1 : 0;
-    const int tp = w.pl & 63, tt = w.pl >> 6;  // column of this point in the transposed tiles, and which tile
+    const int vcta = blockIdx.x % V, split = gridDim.x / V;
+    // tiles vcta, vcta + V, ... of the virtual CTA
+    const int64_t mine = ntiles > vcta ? (ntiles - 1 - vcta) / V + 1 : 0;
 
-    // TMEM lane r of D1 and D2 into the parameters: D1's 8-column chunks go
-    // round-robin over the warpgroups, D2 (one column) to warpgroup 0; every
-    // entry has one writer
+    // TMEM lane r of D1 and D2 into the partial row; every entry has one writer
     auto fold = [&]() {
         const int r = w.pl;
+        if (r < 64) {
 #pragma unroll 1
-        for (int q = w.g; q < 10; q += kWG) {
-            const int c8 = q * 8;
-            float v[8];
-            tc::tmem_ld8(w.lane_base + cD1 + c8, v);
+            for (int c = w.g * 16; c < 64; c += 16 * kWG) {
+                float v[16];
+                double s[16];
 #pragma unroll
-            for (int i = 0; i < 8; i++) {
-                const int c = c8 + i;
-                int e = -1;
-                if (r < 64) {
-                    if (c < 64) e = oW2 + r * kH + c;
-                    else if (c == 72) e = oB2 + r;
-                } else {
-                    if (c >= 64 && c < 72) e = oW1 + (r - 64) * kF + (c - 64);
-                    else if (c == 72) e = oB1 + (r - 64);
-                }
-                if (e >= 0) out[e] += (double)v[i];
+                for (int i = 0; i < 16; i++) s[i] = out[pW2 + (c + i) * kH + r];
+                tc::tmem_ld16(w.lane_base + cD1 + c, v);
+#pragma unroll
+                for (int i = 0; i < 16; i++) out[pW2 + (c + i) * kH + r] = s[i] + (double)v[i];
             }
         }
+        float v[16];  // columns 64..71: W1, 72: the biases
+        tc::tmem_ld16(w.lane_base + cD1 + 64, v);
         if (w.g == 0) {
-            float v[8];
-            tc::tmem_ld8(w.lane_base + cD2, v);
-            if (r < 64) out[oW3 + r] += (double)v[0];
-            if (r == 64) out[oB3] += (double)v[0];
+            if (r < 64) {
+                out[pB2 + r] += (double)v[8];
+            } else {
+#pragma unroll
+                for (int f = 0; f < kF; f++) out[pW1 + f * kH + r - 64] += (double)v[f];
+                out[pB1 + r - 64] += (double)v[8];
+            }
+        } else {
+            float d[8];
+            tc::tmem_ld8(w.lane_base + cD2, d);
+            if (r < 64) out[pW3 + r] += (double)d[0];
+            if (r == 64 + kF) out[pB3] += (double)d[0];  // the column of ones
         }
     };
 
-    for (int64_t k = 0; k < mine && __syncthreads_and(sy.ok); k++) {
-        const int64_t tile = blockIdx.x + k * gridDim.x;
-        const int64_t p = tile * kT + w.pl;
-        const bool valid = p < n;
+    // the k-th tile of the virtual CTA after k in this CTA's order
+    auto after = [&](int64_t k) { return (k % kFold) == kFold - 1 ? k + 1 + (int64_t)(split - 1) * kFold : k + 1; };
+    int64_t k = (int64_t)(blockIdx.x / V) * kFold;
+    uint4 nx = make_uint4(0, 0, 0, 0);
+    float nt = 0.0f, nw = 0.0f;
+    auto load = [&](int64_t kk) {
+        const int64_t p = (vcta + kk * V) * kT + w.pl;
+        const bool valid = kk < mine && p < n;
+        if (w.g == 0) nx = load_features(feat, valid ? p : n, n);
+        nt = valid ? target[p] : 0.0f;
+        nw = valid ? wt[p] : 0.0f;
+    };
+    load(k);
+    while (k < mine) {
+        const int64_t p = (vcta + k * V) * kT + w.pl;
+        const uint4 xv = nx;
+        const float tv = nt, wv = nw;
+        const int64_t knext = after(k);
+        load(knext);
         float h1[kCB], h2[kCB];
-        uint16_t xb[kF];
-        const float yv = forward_tile(sm, B, feat, p, valid, w, tmem, sy, ypart, h1, h2, xb);
-        const float r = valid ? yv - target[p] : 0.0f;
-        const float wv = valid ? wt[p] : 0.0f;
+        const float yv = forward_tile(sm, B, xv, w, tmem, sy, ypart, h1, h2);
+        if (!sy.ok) break;
+        const float r = p < n ? yv - tv : 0.0f;
         if (w.g == 0) loss += (double)wv * (double)r * (double)r;
         const float dy = 2.0f * wv * r;
-        // dz2 (A of dH1, and rows j of D1's A), h2 (rows j of D2's A) and
-        // bf16(h1) (rows i of D1's B) for this warpgroup's units
+        // h2 and dz2 = dy W3 (1 - h2^2)
+        store_row<kCB>(sm + sH2, w.pl, w.c0, h2);
 #pragma unroll
-        for (int j = 0; j < kCB; j++) {
-            const int jj = w.c0 + j;
-            const uint16_t d = bf16_rn(dy * B.w3[jj] * (1.0f - h2[j] * h2[j]));
-            st16(sm, sDZ2 + swz2(w.pl, jj), d);
-            st16(sm, sAT + tt * 128 * 128 + swz2(jj, tp), d);
-            st16(sm, sA2 + tt * 128 * 128 + swz2(jj, tp), bf16_rn(h2[j]));
-            st16(sm, sBT + tt * 80 * 128 + swz2(jj, tp), bf16_rn(h1[j]));
-        }
-        if (w.g == 0) {
-            // dy (D2's B) and x (rows 64..71 of D1's B)
-            st16(sm, sB2 + tt * 16 * 128 + swz2(0, tp), bf16_rn(dy));
-#pragma unroll
-            for (int f = 0; f < kF; f++) st16(sm, sBT + tt * 80 * 128 + swz2(64 + f, tp), xb[f]);
-        }
+        for (int j = 0; j < kCB; j++) h2[j] = dy * B.w3[w.c0 + j] * (1.0f - h2[j] * h2[j]);
+        store_row<kCB>(sm + sDZ2, w.pl, w.c0, h2);
+        if (w.g == 0)
+            st16(sm, sB2 + (w.pl >> 6) * 16 * 128 + swz2(0, w.pl & 63), (uint16_t)(bf16x2(dy, 0.0f) & 0xFFFFu));
         tc::fence_async_smem();
         tc::fence_before_sync();
         __syncthreads();
         if (w.t == 0) {
             tc::fence_after_sync();
-            mma_chain(tmem + cDH1, tc::smem_u32(sm + sDZ2), tc::smem_u32(sm + sW2T), 4, tc::idesc_bf16(128, 64), false);
+            const uint64_t da = tc::sdesc_sw128(tc::smem_u32(sm + sDZ2));
+            const uint64_t db = tc::sdesc_mn_sw128(tc::smem_u32(sm + sW2), 0);
+#pragma unroll
+            for (int q = 0; q < 4; q++)  // 16 rows j of W2 a step
+                tc::mma_bf16(tmem + cZ, da + 2 * q, db + 128 * q, tc::idesc_bf16(128, 64, false, true), q > 0);
             tc::commit(sy.bar);
         }
         sy.wait();
-        // dz1 = dh1 (1 - h1^2) (rows 64 + i of D1's A)
+        // dz1 = dh1 (1 - h1^2)
 #pragma unroll
-        for (int c = 0; c < kCB; c += 8) {
-            float a[8];
-            tc::tmem_ld8(w.lane_base + cDH1 + w.c0 + c, a);
+        for (int c = 0; c < kCB; c += 16) {
+            float a[16];
+            tc::tmem_ld16(w.lane_base + cZ + w.c0 + c, a);
 #pragma unroll
-            for (int i = 0; i < 8; i++)
-                st16(sm, sAT + tt * 128 * 128 + swz2(64 + w.c0 + c + i, tp), bf16_rn(a[i] * (1.0f - h1[c + i] * h1[c + i])));
+            for (int i = 0; i < 16; i++) h1[c + i] = a[i] * (1.0f - h1[c + i] * h1[c + i]);
         }
+        store_row<kCB>(sm + sDZ1, w.pl, w.c0, h1);
         tc::fence_async_smem();
         tc::fence_before_sync();
         __syncthreads();
         if (w.t == 0) {
             tc::fence_after_sync();
             const bool acc = (k % kFold) != 0;
-            const uint32_t aT = tc::smem_u32(sm + sAT), bT = tc::smem_u32(sm + sBT);
-            const uint32_t a2 = tc::smem_u32(sm + sA2), b2 = tc::smem_u32(sm + sB2);
-            // K = 128 points: two 64-point tiles of each operand
-            mma_chain(tmem + cD1, aT, bT, 4, tc::idesc_bf16(128, 80), acc);
-            mma_chain(tmem + cD1, aT + 128 * 128, bT + 80 * 128, 4, tc::idesc_bf16(128, 80), true);
-            mma_chain(tmem + cD2, a2, b2, 4, tc::idesc_bf16(128, 16), acc);
-            mma_chain(tmem + cD2, a2 + 128 * 128, b2 + 16 * 128, 4, tc::idesc_bf16(128, 16), true);
+            const uint64_t a1 = tc::sdesc_mn_sw128(tc::smem_u32(sm + sDZ2), sDZ1 - sDZ2);
+            const uint64_t b1 = tc::sdesc_mn_sw128(tc::smem_u32(sm + sH1), sX - sH1);
+            const uint64_t a2 = tc::sdesc_mn_sw128(tc::smem_u32(sm + sH2), sX - sH2);
+            const uint64_t b2 = tc::sdesc_sw128(tc::smem_u32(sm + sB2));
+            // K = 128 points, 16 rows of the point tiles a step; dy: two tiles of 64
+#pragma unroll
+            for (int q = 0; q < 8; q++)
+                tc::mma_bf16(tmem + cD1, a1 + 128 * q, b1 + 128 * q, tc::idesc_bf16(128, 128, true, true),
+                             q > 0 || acc);
+#pragma unroll
+            for (int q = 0; q < 8; q++)
+                tc::mma_bf16(tmem + cD2, a2 + 128 * q, b2 + 128 * (q >> 2) + 2 * (q & 3),
+                             tc::idesc_bf16(128, 16, true, false), q > 0 || acc);
             tc::commit(sy.bar);
         }
         // the next tile rewrites these operand tiles: wait here
         sy.wait();
         if ((k % kFold) == kFold - 1 || k == mine - 1) fold();
         tc::fence_before_sync();
+        k = knext;
     }
     if (w.g == 0) lsum[w.pl] = loss;
     const bool ok = __syncthreads_and(sy.ok);
@@ -409,56 +429,68 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp64_grad(const uint16_t* __re
     if (ok && t == 0) {
         double s = 0.0;
         for (int q = 0; q < kT; q++) s += lsum[q];
-        out[kP64] = s;
+        out[pLoss] = s;
     }
     tc::fence_before_sync();
     __syncthreads();
     if ((t >> 5) == 0) {
         tc::fence_after_sync();
-        tc::tmem_dealloc(tmem, kCols);
+        tc::tmem_dealloc(tmem, kColsGrad);
+    }
+}
+
+template <class K>
+void allow_smem(K kern, int bytes, bool (&set)[64])
+{
+    int dev = 0;
+    TAGI_CUDA(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= 64 || !set[dev]) {
+        TAGI_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+        if (dev >= 0 && dev < 64) set[dev] = true;
     }
 }
 
 }  // namespace
 
-int mlp64_params() { return kP64; }
+int mlp64_params() { return kParams; }
 
-// Launchers (one CTA per SM, persistent over the tiles): y[n] of the network,
-// and the per-CTA gradient partials [grid][kP64 + 1].  err: device int.
+// y[n] of the network.  err: device int.
 void mlp64_forward(const uint16_t* feat, int64_t n, const double* master, float* y, int* err, int sms, cudaStream_t s)
 {
     static bool set[64] = {};
-    int dev = 0;
-    TAGI_CUDA(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64 || !set[dev]) {
-        TAGI_CUDA(cudaFuncSetAttribute(k_mlp64_fwd, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAlloc));
-        if (dev >= 0 && dev < 64) set[dev] = true;
-    }
+    const int smem = kSmem - sFwd + 1024;
+    allow_smem(k_mlp64_fwd, smem, set);
     const int64_t tiles = (n + kT - 1) / kT;
-    const int grid = (int)(tiles < sms ? tiles : sms);
-    launch(k_mlp64_fwd, grid, kThreads, kSmemAlloc, s, feat, n, master, y, err);
+    const int64_t most = 2LL * sms;
+    launch(k_mlp64_fwd, (int)(tiles < most ? tiles : most), kThreads, smem, s, feat, n, master, y, err);
     TAGI_LAUNCH_CHECK();
+}
+
+// Virtual CTAs (one per SM) and CTAs that share each one's groups of kFold
+// tiles: two where it has more than one group.
+static void mlp64_plan(int64_t n, int sms, int* virt, int* split)
+{
+    const int64_t tiles = (n + kT - 1) / kT;
+    *virt = (int)(tiles < sms ? tiles : sms);
+    *split = (tiles + *virt - 1) / *virt > kFold ? 2 : 1;
 }
 
 int mlp64_grad_grid(int64_t n, int sms)
 {
-    // one CTA per SM; the float32 tensor-memory sums span at most kFold
-    // tiles before they are added to the CTA's float64 row
-    const int64_t tiles = (n + kT - 1) / kT;
-    return (int)(tiles < sms ? tiles : sms);
+    int v, split;
+    mlp64_plan(n, sms, &v, &split);
+    return v * split;
 }
 
+// per-CTA gradient partials [mlp64_grad_grid][kParams + 1]
 void mlp64_gradient(const uint16_t* feat, const float* target, const float* wt, int64_t n, const double* master,
-                    double* partial, int grid, int* err, cudaStream_t s)
+                    double* partial, int sms, int* err, cudaStream_t s)
 {
     static bool set[64] = {};
-    int dev = 0;
-    TAGI_CUDA(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64 || !set[dev]) {
-        TAGI_CUDA(cudaFuncSetAttribute(k_mlp64_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemAlloc));
-        if (dev >= 0 && dev < 64) set[dev] = true;
-    }
-    launch(k_mlp64_grad, grid, kThreads, kSmemAlloc, s, feat, target, wt, n, master, partial, err);
+    allow_smem(k_mlp64_grad, kSmem + 1024, set);
+    int v, split;
+    mlp64_plan(n, sms, &v, &split);
+    launch(k_mlp64_grad, v * split, kThreads, kSmem + 1024, s, feat, target, wt, n, master, partial, v, err);
     TAGI_LAUNCH_CHECK();
 }
 

@@ -280,7 +280,7 @@ int mlp64_params();
 void mlp64_forward(const uint16_t* feat, int64_t n, const double* master, float* y, int* err, int sms, cudaStream_t s);
 int mlp64_grad_grid(int64_t n, int sms);
 void mlp64_gradient(const uint16_t* feat, const float* target, const float* wt, int64_t n, const double* master,
-                    double* partial, int grid, int* err, cudaStream_t s);
+                    double* partial, int sms, int* err, cudaStream_t s);
 
 // sets the message tagi_last_error returns on this thread; returns status
 tagi_status report_error(tagi_status status, const char* msg);

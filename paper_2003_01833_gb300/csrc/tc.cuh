@@ -41,16 +41,31 @@ __device__ __forceinline__ uint64_t sdesc_sw128(uint32_t addr)
     return d;
 }
 
+// shared-memory matrix descriptor of an MN-major operand with the 128-byte
+// swizzle: rows are K (8-row groups 1024 B apart), each row holds 64 16-bit
+// M (or N) values, the next 64 of them `block` bytes further
+__device__ __forceinline__ uint64_t sdesc_mn_sw128(uint32_t addr, uint32_t block)
+{
+    uint64_t d = (uint64_t)((addr & 0x3FFFF) >> 4);  // start address / 16
+    d |= (uint64_t)(block >> 4) << 16;               // leading offset: between 64-wide blocks
+    d |= (uint64_t)(1024 >> 4) << 32;                // stride offset: between 8-row groups of K
+    d |= (uint64_t)1 << 46;                          // descriptor version of sm_10x
+    d |= (uint64_t)2 << 61;                          // 128-byte swizzle
+    return d;
+}
+
 // instruction descriptor: D float32, A and B tf32 (kind::tf32), both K-major
 __host__ __device__ constexpr uint32_t idesc_tf32(int M, int N)
 {
     return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
-// instruction descriptor: D float32, A and B bf16 (kind::f16), both K-major
-__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N)
+// instruction descriptor: D float32, A and B bf16 (kind::f16), K-major unless
+// amn / bmn say MN-major
+__host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, bool amn = false, bool bmn = false)
 {
-    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+    return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)amn << 15) | ((uint32_t)bmn << 16) |
+           ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 __device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count)
@@ -138,6 +153,21 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, float* v)
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
     for (int i = 0; i < 8; i++) v[i] = __uint_as_float(r[i]);
+}
+
+// 16 consecutive columns
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v)
+{
+    uint32_t r[16];
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 16; i++) v[i] = __uint_as_float(r[i]);
 }
 
 }  // namespace tc

@@ -60,19 +60,24 @@ def test_direct_sums_over_ranges(T, scale, nf):
 
 
 @pytest.mark.parametrize("ss", [True, False])
-@pytest.mark.parametrize("nf_y", [0, 3, 4])
-def test_coulomb_shares_a_group(T, ss, nf_y):
+@pytest.mark.parametrize("nf_y", [0, 1, 3, 4, 5])
+def test_groups_of_fields(T, ss, nf_y):
+    """A field's sums do not depend on the fields it shares a launch with: bit
+    for bit those of the field alone.  The Hartree field also against the
+    oracle."""
     n = 1003
     xyz, w = points(n, 3.0, seed=9)
     rho = np.exp(-np.sum(xyz * xyz, axis=0))
-    f = np.stack([np.cos(xyz[0] + o) for o in range(nf_y)]) if nf_y else None
+    f = dev(np.stack([np.cos(xyz[0] + o) for o in range(nf_y)])) if nf_y else None
     k = [0.5 + o for o in range(nf_y)]
-    u = torch.empty((nf_y, n), dtype=torch.float64, device="cuda") if nf_y else None
-    vh = torch.empty(n, dtype=torch.float64, device="cuda")
+    u = torch.empty_like(f) if nf_y else None
+    vh, alone = torch.empty(n, dtype=torch.float64, device="cuda"), torch.empty(n, dtype=torch.float64, device="cuda")
     with T.Tree(dev(xyz), dev(w), theta=0.0, degree=2, leaf_size=300, prec=T.TAGI_FP64, ss=ss) as tr:
-        T.tagi_fields_conv(tr.handle, dev(f) if nf_y else None, k, u, rho=dev(rho), vh=vh)
+        T.tagi_fields_conv(tr.handle, f, k, u, rho=dev(rho), vh=vh)
+        T.tagi_coulomb_conv(tr.handle, dev(rho), alone)
+        assert torch.equal(alone, vh)
+        for o in range(nf_y):
+            T.tagi_yukawa_conv(tr.handle, f[o].contiguous(), [k[o]], alone)
+            assert torch.equal(alone, u[o])
     ref = oracle.direct_coulomb(xyz, w, rho, ss=ss)
     assert np.abs(vh.cpu().numpy() - ref).max() <= TOL * np.abs(ref).max()
-    for o in range(nf_y):
-        ref = oracle.direct_yukawa(xyz, w, f[o], k[o], ss=ss)
-        assert np.abs(u[o].cpu().numpy() - ref).max() <= TOL * np.abs(ref).max()
