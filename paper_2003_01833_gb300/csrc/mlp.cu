@@ -19,6 +19,7 @@
 
 #include "bf16.cuh"
 #include "mlp64.cuh"
+#include "pair64.cuh"
 #include "tagi_internal.cuh"
 
 namespace tagi {
@@ -98,16 +99,36 @@ __device__ __forceinline__ float layer2_unit(const float* sw, const float h1[kH]
 // separation, [e^-(z1 r1), e^-(z2 r2), tanh r1, tanh r2, (r2 - r1)/R,
 // tanh((r1 + r2)/R - 1), R - 1.5, e^-(r1 + r2 - R)].  Sums of squares are
 // formed left to right without contraction.
-__global__ void k_features(const double* __restrict__ xyz, int64_t n, Nuclei nuc, uint16_t* __restrict__ feat)
+//
+// Only 8 bits of each value are kept, and float64 runs at 1/73 of the float32
+// rate here: the distances are float64 (pair64.cuh's root), the exponentials
+// and tangents float32 with a bound on their relative error.  A value whose
+// bound reaches a rounding boundary of bfloat16 (one in a thousand) is
+// evaluated again in float64, a point whose distances tie or cancel to within
+// rounding takes the float64 form throughout (features_exact), so the bits
+// are those of the float64 form.  192,000 points take 22 us, 130 in float64 alone.
+struct Pair {
+    double R, invR;
+    uint16_t f6;
+};
+
+__device__ __forceinline__ double distance2(const Nuclei& nuc, int a, double px, double py, double pz)
 {
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const double px = xyz[i], py = xyz[n + i], pz = xyz[2 * n + i];
+    const double dx = px - nuc.x[a], dy = py - nuc.y[a], dz = pz - nuc.z[a];
+    return __dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz));
+}
+
+__device__ __forceinline__ double separation(const Nuclei& nuc, int a1, int a2)
+{
+    return sqrt(distance2(nuc, a2, nuc.x[a1], nuc.y[a1], nuc.z[a1]));
+}
+
+__device__ __noinline__ uint4 features_exact(const Nuclei& nuc, double px, double py, double pz)
+{
     double d1 = INFINITY, d2 = INFINITY;
     int a1 = 0, a2 = 1;
     for (int a = 0; a < (nuc.ordered ? 0 : nuc.m); a++) {
-        const double dx = px - nuc.x[a], dy = py - nuc.y[a], dz = pz - nuc.z[a];
-        const double d = sqrt(__dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz)));
+        const double d = sqrt(distance2(nuc, a, px, py, pz));
         if (d < d1) {
             d2 = d1;
             a2 = a1;
@@ -119,13 +140,10 @@ __global__ void k_features(const double* __restrict__ xyz, int64_t n, Nuclei nuc
         }
     }
     if (nuc.ordered) {
-        const double dx1 = px - nuc.x[0], dy1 = py - nuc.y[0], dz1 = pz - nuc.z[0];
-        const double dx2 = px - nuc.x[1], dy2 = py - nuc.y[1], dz2 = pz - nuc.z[1];
-        d1 = sqrt(__dadd_rn(__dadd_rn(__dmul_rn(dx1, dx1), __dmul_rn(dy1, dy1)), __dmul_rn(dz1, dz1)));
-        d2 = sqrt(__dadd_rn(__dadd_rn(__dmul_rn(dx2, dx2), __dmul_rn(dy2, dy2)), __dmul_rn(dz2, dz2)));
+        d1 = sqrt(distance2(nuc, 0, px, py, pz));
+        d2 = sqrt(distance2(nuc, 1, px, py, pz));
     }
-    const double ex = nuc.x[a1] - nuc.x[a2], ey = nuc.y[a1] - nuc.y[a2], ez = nuc.z[a1] - nuc.z[a2];
-    const double R = sqrt(__dadd_rn(__dadd_rn(__dmul_rn(ex, ex), __dmul_rn(ey, ey)), __dmul_rn(ez, ez)));
+    const double R = separation(nuc, a1, a2);
     const double s12 = __dadd_rn(d1, d2);
     const double f[kF] = {exp(-__dmul_rn(nuc.zs[a1], d1)),
                           exp(-__dmul_rn(nuc.zs[a2], d2)),
@@ -137,8 +155,106 @@ __global__ void k_features(const double* __restrict__ xyz, int64_t n, Nuclei nuc
                           exp(-__dsub_rn(s12, R))};
     uint32_t u[4];
 #pragma unroll
-    for (int k = 0; k < 4; k++) u[k] = (uint32_t)bf16_of_double(f[2 * k]) | ((uint32_t)bf16_of_double(f[2 * k + 1]) << 16);
-    *reinterpret_cast<uint4*>(feat + i * kF) = make_uint4(u[0], u[1], u[2], u[3]);
+    for (int k = 0; k < 4; k++)
+        u[k] = (uint32_t)bf16_of_double(f[2 * k]) | ((uint32_t)bf16_of_double(f[2 * k + 1]) << 16);
+    return make_uint4(u[0], u[1], u[2], u[3]);
+}
+
+// bfloat16 of a float32 in normal range, if `units` of its last place do not
+// reach a rounding boundary
+__device__ __forceinline__ bool round_safe(float v, float units, uint32_t& b)
+{
+    const uint32_t u = __float_as_uint(v);
+    b = (u + 0x8000u) >> 16;
+    return (float)abs((int)(u & 0xffffu) - 0x8000) > units + 1.0f;
+}
+
+__device__ __noinline__ uint32_t exp_exact(double x) { return bf16_of_double(exp(-x)); }
+__device__ __noinline__ uint32_t tanh_exact(double x) { return bf16_of_double(tanh(x)); }
+
+// e^-x, x to 2^-22: float32 argument and product within x 2^-22, expf within
+// 2^-21 (units of the last place are at most 2^-24 of the value each)
+__device__ __forceinline__ uint32_t exp_bits(double x)
+{
+    const float xf = (float)x;
+    if (xf >= 94.0f) return 0;  // below half the least bfloat16, 2^-133
+    uint32_t b;
+    if (xf < 69.0f && round_safe(expf(-xf), 8.0f + 4.0f * fabsf(xf), b)) return b;
+    return exp_exact(x);
+}
+
+// tanh x, x to 2^-22: tanhf within 2^-22, tanh no steeper than x relatively
+__device__ __forceinline__ uint32_t tanh_bits(double x)
+{
+    uint32_t b;
+    const float xf = (float)x;
+    if (fabsf(xf) > 1e-30f && round_safe(tanhf(xf), 16.0f, b)) return b;
+    return tanh_exact(x);
+}
+
+__global__ void __launch_bounds__(256) k_features(const double* __restrict__ xyz, int64_t n,
+                                                  const __grid_constant__ Nuclei nuc, uint16_t* __restrict__ feat)
+{
+    __shared__ Pair pairs[kMaxNuclei * kMaxNuclei];
+    for (int q = threadIdx.x; q < nuc.m * nuc.m; q += blockDim.x) {
+        const double R = separation(nuc, q / nuc.m, q % nuc.m);
+        pairs[q] = Pair{R, 1.0 / R, bf16_of_double(__dsub_rn(R, 1.5))};
+    }
+    __syncthreads();
+    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const double px = xyz[i], py = xyz[n + i], pz = xyz[2 * n + i];
+    // the two nearest by squared distance (positive float64 compare as
+    // integers); squares a few units apart may have equal roots: not safe
+    long long q1 = 0x7ff0000000000000ll, q2 = q1;
+    int a1 = 0, a2 = 1;
+    bool safe = true;
+    if (nuc.ordered) {
+        q1 = __double_as_longlong(distance2(nuc, 0, px, py, pz));
+        q2 = __double_as_longlong(distance2(nuc, 1, px, py, pz));
+    } else {
+        for (int a = 0; a < nuc.m; a++) {
+            const long long q = __double_as_longlong(distance2(nuc, a, px, py, pz));
+            safe = safe && (q == q1 || llabs(q - q1) > 8) && (q == q2 || llabs(q - q2) > 8);
+            if (q < q1) {
+                q2 = q1;
+                a2 = a1;
+                q1 = q;
+                a1 = a;
+            } else if (q < q2) {
+                q2 = q;
+                a2 = a;
+            }
+        }
+    }
+    const double r21 = __longlong_as_double(q1), r22 = __longlong_as_double(q2);
+    uint4 out = make_uint4(0, 0, 0, 0);
+    safe = safe && p64::fast_range(r21) && p64::fast_range(r22);
+    if (safe) {
+        const Pair pr = pairs[a1 * nuc.m + a2];
+        double ri, d1, d2;
+        p64::inv_sqrt(r21, ri, d1);
+        p64::inv_sqrt(r22, ri, d2);
+        const double s12 = d1 + d2, diff = d2 - d1, x5 = fma(s12, pr.invR, -1.0);
+        const double f4 = diff * pr.invR;
+        // the roots are within 2^-51 of their values: not safe where the
+        // difference cancels below 2^-26 of them, or where f4 is as near a
+        // rounding boundary (the middle of its 45 dropped bits) as the
+        // cancellation has left it exact
+        const long long b4 = __double_as_longlong(f4);
+        const float s32 = (float)s12, rest = fabsf((float)diff);
+        safe = fabsf((float)x5) > 1.5e-8f &&
+               (q1 == q2 || (rest > 1.5e-8f * s32 &&
+                             (float)llabs((b4 & 0x1fffffffffffll) - 0x100000000000ll) > 64.0f + 8.0f * s32 / rest));
+        if (safe) {
+            const uint32_t f0 = exp_bits(nuc.zs[a1] * d1), f1 = exp_bits(nuc.zs[a2] * d2);
+            const uint32_t f2 = tanh_bits(d1), f3 = tanh_bits(d2);
+            const uint32_t f5 = tanh_bits(x5), f7 = exp_bits(s12 - pr.R);
+            out = make_uint4(f0 | f1 << 16, f2 | f3 << 16, bf16_of_double(f4) | f5 << 16, pr.f6 | f7 << 16);
+        }
+    }
+    if (!safe) out = features_exact(nuc, px, py, pz);
+    *reinterpret_cast<uint4*>(feat + i * kF) = out;
 }
 
 __global__ void __launch_bounds__(kThreads) k_mlp_forward(const uint16_t* __restrict__ feat, int64_t n,
@@ -358,17 +474,23 @@ __global__ void __launch_bounds__(256) k_warm_apply(const float* __restrict__ y,
     if (threadIdx.x == 0) part[blockIdx.x] = red[0];
 }
 
-// psi /= sqrt(sum of the partials): one thread of each block sums them in
-// block order (every block gets the same value) and shares the factor.
-__global__ void k_warm_scale(double* __restrict__ psi, int64_t n, const double* __restrict__ part, int nblk)
+// psi /= sqrt(sum of the partials): every block sums them in the same order
+// (256 strided sums, then a tree), so every block has the same factor.  One
+// thread that adds 608 partials one after another took 35 of this kernel's 39
+// us.
+__global__ void __launch_bounds__(256) k_warm_scale(double* __restrict__ psi, int64_t n,
+                                                    const double* __restrict__ part, int nblk)
 {
-    __shared__ double inv;
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int b = 0; b < nblk; b++) s += part[b];
-        inv = 1.0 / sqrt(s);
-    }
+    __shared__ double red[256];
+    double s = 0.0;
+    for (int b = threadIdx.x; b < nblk; b += 256) s += part[b];
+    red[threadIdx.x] = s;
     __syncthreads();
+    for (int h = 128; h > 0; h >>= 1) {
+        if (threadIdx.x < h) red[threadIdx.x] += red[threadIdx.x + h];
+        __syncthreads();
+    }
+    const double inv = 1.0 / sqrt(red[0]);
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         psi[i] *= inv;
 }
@@ -641,7 +763,7 @@ tagi_status tagi_mlp_warm_start(const tagi_mlp* mlp, const uint16_t* feat, const
         const int nb = (int)std::min<int64_t>((n + 255) / 256, 4LL * M->sms);
         M->part.ensure(sizeof(double) * nb);
         launch(k_warm_apply, nb, 256, 0, s, (const float*)y.as<float>(), s0, w, n, psi, M->part.as<double>());
-        launch(k_warm_scale, (unsigned)std::min<int64_t>((n + 255) / 256, 8LL * M->sms), 256, 0, s, psi, n,
+        launch(k_warm_scale, (unsigned)std::min<int64_t>((n + 255) / 256, 2LL * M->sms), 256, 0, s, psi, n,
                (const double*)M->part.as<double>(), nb);
         TAGI_LAUNCH_CHECK();
     });
