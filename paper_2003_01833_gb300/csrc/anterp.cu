@@ -4,8 +4,8 @@
 // Eq. barycentric_weights on Chebyshev points of the second kind mapped to the
 // cluster box (Section 5.2).
 //
-// Two kernels, both over work items (a chunk of at most kAntChunk points of
-// one cluster), with chunk partials summed in a fixed order afterwards, so
+// Two kernels, both over work items (a chunk of at most T.ant_chunk points of
+// one cluster, a multiple of 64), with chunk partials summed in a fixed order afterwards, so
 // results are reproducible run to run:
 //   k_ant (SIMT): each thread owns up to four proxies; the points stream
 //     through shared memory 64 at a time with their 3 (n+1) basis values, so a
@@ -148,15 +148,14 @@ constexpr int kAntLP = 12;  // padded basis row of the cache (degree <= 11)
 static_assert(kMaxDegree + 1 <= kAntLP, "basis row fits");
 
 constexpr int kTcK = 32;                             // points per tensor-core tile
-constexpr int kTilesPerItem = kAntChunk / kTcK;      // 64
 constexpr int kTileFloats = 3 * kAntLP * kTcK;       // basis floats of one tile (4608 bytes)
-static_assert(kAntChunk % kTcK == 0, "whole tiles per item");
+static_assert(kAntTile % kTcK == 0, "whole tiles per item");
 
-// index of basis value k of dimension d of point j (0 <= j < kAntChunk) of
-// item `item` in the basis cache: tiles of 32 points, each [3][kAntLP][32]
-__host__ __device__ inline size_t antl_index(size_t item, int j, int d, int k)
+// index of basis value k of dimension d of point j of item `item` in the basis
+// cache: tpi tiles of 32 points an item, each [3][kAntLP][32]
+__host__ __device__ inline size_t antl_index(size_t item, int tpi, int j, int d, int k)
 {
-    return ((item * kTilesPerItem + (j >> 5)) * 3 + d) * (size_t)(kAntLP * kTcK) + k * kTcK + (j & 31);
+    return ((item * tpi + (j >> 5)) * 3 + d) * (size_t)(kAntLP * kTcK) + k * kTcK + (j & 31);
 }
 
 // Basis cache of the float32 path: for every point of every anterpolation
@@ -171,7 +170,7 @@ __global__ void __launch_bounds__(kAntThreads) k_ant_basis(const AntItem* __rest
                                                            const double* __restrict__ py,
                                                            const double* __restrict__ pz,
                                                            const double* __restrict__ lo,
-                                                           const double* __restrict__ hi, int degree,
+                                                           const double* __restrict__ hi, int degree, int tpi,
                                                            float* __restrict__ antL)
 {
     __shared__ double dnodes[kMaxDegree + 1], inv[kMaxDegree + 1];
@@ -213,7 +212,7 @@ __global__ void __launch_bounds__(kAntThreads) k_ant_basis(const AntItem* __rest
         if (j < np) basis_df(df_of(deg ? 0.0 : (x[it.p0 + j] - ccd) * ihd), deg, degree, fnodes, finv, Lf);
 #pragma unroll
         for (int k = 0; k < kAntLP; k++)
-            antL[antl_index(blockIdx.x, j, d, k)] = (j < np && k <= degree && k <= kMaxDegree) ? Lf[k] : 0.0f;
+            antL[antl_index(blockIdx.x, tpi, j, d, k)] = (j < np && k <= degree && k <= kMaxDegree) ? Lf[k] : 0.0f;
     }
 }
 
@@ -226,7 +225,7 @@ __global__ void __launch_bounds__(kAntThreads) k_ant(const AntItem* __restrict__
                                                      const double* __restrict__ lo, const double* __restrict__ hi,
                                                      int degree, int f32nodes, const R* __restrict__ q,
                                                      int64_t ldq, double* __restrict__ part,
-                                                     const float* __restrict__ antL)
+                                                     const float* __restrict__ antL, int tpi)
 {
     __shared__ R Ls[kAntTile][3][kMaxDegree + 1];
     __shared__ R qs[NQ][kAntTile];
@@ -273,7 +272,7 @@ __global__ void __launch_bounds__(kAntThreads) k_ant(const AntItem* __restrict__
             int j = threadIdx.x / 3, d = threadIdx.x % 3;
             R L[kMaxDegree + 1];
             if (j < nt && antL) {
-                for (int k = 0; k <= degree; k++) L[k] = (R)antL[antl_index(blockIdx.x, (p0 - it.p0) + j, d, k)];
+                for (int k = 0; k <= degree; k++) L[k] = (R)antL[antl_index(blockIdx.x, tpi, (p0 - it.p0) + j, d, k)];
             } else if (j < nt) {
                 const double* x = d == 0 ? px : (d == 1 ? py : pz);
                 bool deg = hh[d] == 0.0;
@@ -327,25 +326,27 @@ __global__ void __launch_bounds__(kAntThreads) k_ant(const AntItem* __restrict__
 // w^ of the FP32C tree from the two-float weight columns (w_hi, w_lo) and
 // the basis cache, in proxy pencils: thread t < M^2 owns the M proxies
 // (k1, k2, k3 = 0 .. M-1) with k1 = t / M, k2 = t % M.  L1 L2 is formed once
-// per point and pencil and the k3 values are broadcast from shared memory,
-// so a point costs 2 + M + 2 shared loads per pencil instead of 5 per proxy
-// (k_ant is bound by its shared loads).  The products, (L1 L2) L3 times each
-// column, and the summation order (float sums over 64-point tiles in point
-// order, float64 across tiles) are those of k_ant, so w^ is bit-identical.
+// per point and pencil and the k3 values are broadcast from shared memory four
+// at a time, so a point costs 2 + ceil(M / 4) + 1 shared loads per pencil for
+// its 3 M products (k_ant: 5 loads per proxy).  The products, (L1 L2) L3 times
+// each column, and the float sums over 64-point tiles in point order are those
+// of k_ant.
 template <int M>
 struct Pencil {
     static constexpr int threads = (M * M + 31) / 32 * 32;
+    static constexpr int row = (M + 3) / 4 * 4;
 };
 
 template <int M>
 __global__ void __launch_bounds__(Pencil<M>::threads) k_ant_pencil(const AntItem* __restrict__ items,
                                                                    const float* __restrict__ q, int64_t ldq,
                                                                    double* __restrict__ part,
-                                                                   const float* __restrict__ antL)
+                                                                   const float* __restrict__ antL, int tpi)
 {
-    constexpr int P = M * M * M;
-    __shared__ float Ls[kAntTile][3][M];
-    __shared__ float qs[2][kAntTile];
+    constexpr int P = M * M * M, LR = Pencil<M>::row;
+    __shared__ float Ls[2][M][kAntTile];  // L1, L2: [dimension][node][point]
+    __shared__ float4 L3[kAntTile][LR / 4];
+    __shared__ float2 qs[kAntTile];
     const AntItem it = items[blockIdx.x];
     const int t = threadIdx.x;
     const bool own = t < M * M;
@@ -356,26 +357,38 @@ __global__ void __launch_bounds__(Pencil<M>::threads) k_ant_pencil(const AntItem
     for (int p0 = it.p0; p0 < it.p1; p0 += kAntTile) {
         const int nt = min(kAntTile, it.p1 - p0);
         __syncthreads();
-        for (int e = t; e < kAntTile * 3 * M; e += Pencil<M>::threads) {
-            const int j = e / (3 * M), d = (e / M) % 3, k = e % M;
-            Ls[j][d][k] = j < nt ? antL[antl_index(blockIdx.x, (p0 - it.p0) + j, d, k)] : 0.0f;
+        for (int e = t; e < 3 * M * kAntTile; e += Pencil<M>::threads) {
+            const int j = e % kAntTile, k = (e / kAntTile) % M, d = e / (kAntTile * M);
+            const float v = j < nt ? antL[antl_index(blockIdx.x, tpi, (p0 - it.p0) + j, d, k)] : 0.0f;
+            if (d < 2)
+                Ls[d][k][j] = v;
+            else
+                reinterpret_cast<float*>(L3[j])[k] = v;
         }
-        for (int e = t; e < 2 * kAntTile; e += Pencil<M>::threads) {
-            const int col = e / kAntTile, j = e % kAntTile;
-            qs[col][j] = j < nt ? q[col * ldq + p0 + j] : 0.0f;
-        }
+        for (int j = t; j < kAntTile; j += Pencil<M>::threads)
+            qs[j] = j < nt ? make_float2(q[p0 + j], q[ldq + p0 + j]) : make_float2(0.0f, 0.0f);
         __syncthreads();
         float tacc[M][2];
 #pragma unroll
         for (int k = 0; k < M; k++) tacc[k][0] = tacc[k][1] = 0.0f;
+#pragma unroll 2
         for (int j = 0; j < nt; j++) {
-            const float l12 = Ls[j][0][k1] * Ls[j][1][k2];
-            const float q0 = qs[0][j], q1 = qs[1][j];
+            const float l12 = Ls[0][k1][j] * Ls[1][k2][j];
+            const float2 qj = qs[j];
+            float l3[LR];
+#pragma unroll
+            for (int g = 0; g < LR / 4; g++) {
+                const float4 v = L3[j][g];
+                l3[4 * g] = v.x;
+                l3[4 * g + 1] = v.y;
+                l3[4 * g + 2] = v.z;
+                l3[4 * g + 3] = v.w;
+            }
 #pragma unroll
             for (int k = 0; k < M; k++) {
-                const float L = l12 * Ls[j][2][k];
-                tacc[k][0] += L * q0;
-                tacc[k][1] += L * q1;
+                const float L = l12 * l3[k];
+                tacc[k][0] += L * qj.x;
+                tacc[k][1] += L * qj.y;
             }
         }
 #pragma unroll
@@ -449,7 +462,7 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
                  : "memory");
 }
 
-// One CTA per item (at most 2048 points of one cluster): 8 warps form the
+// One CTA per item (a chunk of one cluster's points): 8 warps form the
 // operands and fold the accumulators, one more warp (its lane 0) issues the
 // MMAs and the bulk copies.  The basis rows of the item's points (basis
 // cache, tile layout) and its charges (charge tiles of k_qtiles, columns q0
@@ -473,7 +486,7 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
 // its MMAs and copies in flight, *err is set and no output is written.
 template <int NH>
 __global__ void __launch_bounds__(kTcThreads, 2)
-    k_ant_tc(const float* __restrict__ antL, const float* __restrict__ qT, int nqt, int q0, int nq,
+    k_ant_tc(const float* __restrict__ antL, const float* __restrict__ qT, int tpi, int nqt, int q0, int nq,
              const AntItem* __restrict__ items, int degree, double* __restrict__ part, int* __restrict__ err)
 {
     constexpr int NPAD = 2 * NH;
@@ -561,7 +574,7 @@ __global__ void __launch_bounds__(kTcThreads, 2)
         if (lane == 0) {
             auto load_tile = [&](int t) {
                 const int u = t % kTcSlots;
-                const size_t tile = (size_t)blockIdx.x * kTilesPerItem + t;
+                const size_t tile = (size_t)blockIdx.x * tpi + t;
                 float* dst = Lb + u * kSlot;
                 tc::fence_async_smem();
                 mbar_expect_tx(&ld_full[u], (uint32_t)kTileFloats * 4 + qbytes);
@@ -697,20 +710,20 @@ __global__ void __launch_bounds__(kTcThreads, 2)
     }
 }
 
-// Charge tiles of the tensor-core anterpolation: qT[(item * 64 + tile) * nf +
+// Charge tiles of the tensor-core anterpolation: qT[(item * tpi + tile) * nf +
 // col][32] = q[col][p0 + 32 tile + j] (zero beyond the item's end).
-__global__ void k_qtiles(const AntItem* __restrict__ items, int64_t nitems, const float* __restrict__ q, int nf,
-                         int64_t ldq, float* __restrict__ qT)
+__global__ void k_qtiles(const AntItem* __restrict__ items, int64_t nitems, int tpi, const float* __restrict__ q,
+                         int nf, int64_t ldq, float* __restrict__ qT)
 {
     const int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (e >= nitems * kAntChunk * nf) return;
+    if (e >= nitems * tpi * kTcK * nf) return;
     const int jj = (int)(e & 31);
     const int64_t rest = e >> 5;
     const int col = (int)(rest % nf);
     const int64_t tile = rest / nf;
-    const int64_t item = tile / kTilesPerItem;
+    const int64_t item = tile / tpi;
     const AntItem it = items[item];
-    const int j = (int)(tile % kTilesPerItem) * kTcK + jj;
+    const int j = (int)(tile % tpi) * kTcK + jj;
     qT[e] = it.p0 + j < it.p1 ? q[col * ldq + it.p0 + j] : 0.0f;
 }
 
@@ -759,13 +772,13 @@ __global__ void k_split_w(const double* w, int64_t n, float* out)
 
 template <class R, class A>
 void launch_ant(int nq, int nitems, const AntItem* items, Tree& T, const R* q, int64_t ldq, double* part,
-                cudaStream_t s, const float* antL = nullptr)
+                cudaStream_t s, const float* antL = nullptr, int tpi = 0)
 {
 #define TAGI_ANT_CASE(NQ)                                                                                   \
     case NQ:                                                                                                \
         launch(k_ant<R, A, NQ>, nitems, kAntThreads, 0, s, items, T.px.as<double>(), T.py.as<double>(),         \
                                                        T.pz.as<double>(), T.cl_lo.as<double>(),             \
-                                                       T.cl_hi.as<double>(), T.degree, T.prec == TAGI_FP32C, q, ldq, part, antL); \
+                                                       T.cl_hi.as<double>(), T.degree, T.prec == TAGI_FP32C, q, ldq, part, antL, tpi); \
         break;
     switch (nq) {
         TAGI_ANT_CASE(1)
@@ -785,8 +798,8 @@ void launch_ant(int nq, int nitems, const AntItem* items, Tree& T, const R* q, i
 
 
 template <int NH>
-void launch_ant_tc_nh(int nq, int nitems, const AntItem* items, int degree, const float* antL, const float* qT,
-                      int nqt, int q0, double* part, int* err, cudaStream_t s)
+void launch_ant_tc_nh(int nq, int nitems, const AntItem* items, int tpi, int degree, const float* antL,
+                      const float* qT, int nqt, int q0, double* part, int* err, cudaStream_t s)
 {
     const int ra = ((degree + 1) * (degree + 1) + 7) / 8 * 8;
     const int need = tc_smem_bytes(ra, 2 * NH);
@@ -799,7 +812,7 @@ void launch_ant_tc_nh(int nq, int nitems, const AntItem* items, int degree, cons
         TAGI_CUDA(cudaFuncSetAttribute(k_ant_tc<NH>, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxSmem));
         if (dev >= 0 && dev < 64) attr_set[dev] = true;
     }
-    launch(k_ant_tc<NH>, nitems, kTcThreads, smem, s, antL, qT, nqt, q0, nq, items, degree, part, err);
+    launch(k_ant_tc<NH>, nitems, kTcThreads, smem, s, antL, qT, tpi, nqt, q0, nq, items, degree, part, err);
     TAGI_LAUNCH_CHECK();
 }
 
@@ -807,35 +820,35 @@ void launch_ant_tc_nh(int nq, int nitems, const AntItem* items, int degree, cons
 // [q0, q0 + nq) of the charge tiles qT (nqt columns, k_qtiles) with the basis
 // cache antL of the same items: part[item][col][P] in float64.  err: device
 // int, set to nonzero if a bounded wait of the kernel gave up.
-void launch_ant_tc(int nq, int nitems, const AntItem* items, int degree, const float* antL, const float* qT, int nqt,
-                   int q0, double* part, int* err, cudaStream_t s)
+void launch_ant_tc(int nq, int nitems, const AntItem* items, int tpi, int degree, const float* antL, const float* qT,
+                   int nqt, int q0, double* part, int* err, cudaStream_t s)
 {
     TAGI_REQUIRE(nq >= 1 && nq <= 8, "anterpolation column group must hold 1..8 columns");
     const int npad = ((degree + 1) * nq + 15) / 16 * 16;
     switch (npad / 2) {
-        case 8: launch_ant_tc_nh<8>(nq, nitems, items, degree, antL, qT, nqt, q0, part, err, s); break;
-        case 16: launch_ant_tc_nh<16>(nq, nitems, items, degree, antL, qT, nqt, q0, part, err, s); break;
-        case 24: launch_ant_tc_nh<24>(nq, nitems, items, degree, antL, qT, nqt, q0, part, err, s); break;
-        case 32: launch_ant_tc_nh<32>(nq, nitems, items, degree, antL, qT, nqt, q0, part, err, s); break;
-        case 40: launch_ant_tc_nh<40>(nq, nitems, items, degree, antL, qT, nqt, q0, part, err, s); break;
+        case 8: launch_ant_tc_nh<8>(nq, nitems, items, tpi, degree, antL, qT, nqt, q0, part, err, s); break;
+        case 16: launch_ant_tc_nh<16>(nq, nitems, items, tpi, degree, antL, qT, nqt, q0, part, err, s); break;
+        case 24: launch_ant_tc_nh<24>(nq, nitems, items, tpi, degree, antL, qT, nqt, q0, part, err, s); break;
+        case 32: launch_ant_tc_nh<32>(nq, nitems, items, tpi, degree, antL, qT, nqt, q0, part, err, s); break;
+        case 40: launch_ant_tc_nh<40>(nq, nitems, items, tpi, degree, antL, qT, nqt, q0, part, err, s); break;
         default: throw Error(TAGI_ERR_INVALID_ARG, "tensor-core anterpolation: (degree+1) * columns exceeds 80");
     }
 }
 
-void fill_basis_cache(Tree& T, int nitems, const AntItem* items, DevBuf& cache)
+void fill_basis_cache(Tree& T, int nitems, const AntItem* items, int tpi, DevBuf& cache)
 {
-    cache.ensure(sizeof(float) * (size_t)nitems * kTilesPerItem * kTileFloats);
+    cache.ensure(sizeof(float) * (size_t)nitems * tpi * kTileFloats);
     launch(k_ant_basis, nitems, kAntThreads, 0, T.stream, items, T.px.as<double>(), T.py.as<double>(),
-           T.pz.as<double>(), T.cl_lo.as<double>(), T.cl_hi.as<double>(), T.degree, cache.as<float>());
+           T.pz.as<double>(), T.cl_lo.as<double>(), T.cl_hi.as<double>(), T.degree, tpi, cache.as<float>());
     TAGI_LAUNCH_CHECK();
 }
 
-void fill_charge_tiles(Tree& T, int64_t nitems, const AntItem* items, const float* q, int nf, int64_t ldq,
+void fill_charge_tiles(Tree& T, int64_t nitems, const AntItem* items, int tpi, const float* q, int nf, int64_t ldq,
                        DevBuf& qT)
 {
-    const int64_t total = nitems * kAntChunk * nf;
+    const int64_t total = nitems * tpi * kTcK * nf;
     qT.ensure(sizeof(float) * (size_t)total);
-    launch(k_qtiles, (int)((total + 255) / 256), 256, 0, T.stream, items, nitems, q, nf, ldq, qT.as<float>());
+    launch(k_qtiles, (int)((total + 255) / 256), 256, 0, T.stream, items, nitems, tpi, q, nf, ldq, qT.as<float>());
     TAGI_LAUNCH_CHECK();
 }
 
@@ -846,8 +859,9 @@ void anterpolate_weights(Tree& T)
     if (T.nfar == 0) return;
     cudaStream_t s = T.stream;
     if (T.prec == TAGI_FP32C) {
-        // basis cache (kept with the tree while it fits the budget below)
-        fill_basis_cache(T, (int)T.nant, T.ant_items.as<AntItem>(), T.antL);
+        // basis cache, kept with the tree
+        const int tpi = T.ant_chunk / kTcK;
+        fill_basis_cache(T, (int)T.nant, T.ant_items.as<AntItem>(), tpi, T.antL);
         const float* antL = T.antL.p ? T.antL.as<float>() : nullptr;
         // w^ from the two-float weights (w_hi, w_lo), on the float32 nodes
         // where the proxies sit
@@ -857,13 +871,13 @@ void anterpolate_weights(Tree& T)
         launch(k_split_w, (int)((T.n + 255) / 256), 256, 0, s, T.pw.as<double>(), T.n, w2.as<float>());
         if (antL && T.degree == 8)
             launch(k_ant_pencil<9>, (int)T.nant, Pencil<9>::threads, 0, s, T.ant_items.as<AntItem>(), w2.as<float>(),
-                   T.n, T.antpart.as<double>(), antL);
+                   T.n, T.antpart.as<double>(), antL, tpi);
         else if (antL && T.degree == 6)
             launch(k_ant_pencil<7>, (int)T.nant, Pencil<7>::threads, 0, s, T.ant_items.as<AntItem>(), w2.as<float>(),
-                   T.n, T.antpart.as<double>(), antL);
+                   T.n, T.antpart.as<double>(), antL, tpi);
         else
             launch_ant<float, double>(2, (int)T.nant, T.ant_items.as<AntItem>(), T, w2.as<float>(), T.n,
-                                      T.antpart.as<double>(), s, antL);
+                                      T.antpart.as<double>(), s, antL, tpi);
         launch(k_ant_reduce_w, T.nfar, 256, 0, s, T.far_ant0.as<int>(), T.antpart.as<double>(), T.P, T.n,
                T.rec4.as<float4>());
         TAGI_LAUNCH_CHECK();
@@ -882,11 +896,12 @@ void anterpolate_fields32(Tree& T, int nf)
 {
     if (T.nfar == 0) return;
     cudaStream_t s = T.stream;
-    fill_charge_tiles(T, T.nant, T.ant_items.as<AntItem>(), T.qant.as<float>(), nf, T.n, T.qtiles);
+    const int tpi = T.ant_chunk / kTcK;
+    fill_charge_tiles(T, T.nant, T.ant_items.as<AntItem>(), tpi, T.qant.as<float>(), nf, T.n, T.qtiles);
     for (int g0 = 0; g0 < nf; g0 += 8) {
         int g = nf - g0 < 8 ? nf - g0 : 8;
         T.antpart.ensure(sizeof(double) * (size_t)T.nant * T.P * g);
-        launch_ant_tc(g, (int)T.nant, T.ant_items.as<AntItem>(), T.degree, T.antL.as<float>(), T.qtiles.as<float>(),
+        launch_ant_tc(g, (int)T.nant, T.ant_items.as<AntItem>(), tpi, T.degree, T.antL.as<float>(), T.qtiles.as<float>(),
                       nf, g0, T.antpart.as<double>(), T.errflag.as<int>() + 1, s);
         launch(k_ant_reduce, T.nfar, 256, 0, s, T.nfar, T.far_ant0.as<int>(), T.antpart.as<double>(), g, T.P, T.n, 0,
                                             T.fa.as<float>(), nullptr, g0, T.nrec);
@@ -974,12 +989,13 @@ void anterpolate_all_clusters32(Tree& T, const double* q, int nq, double* qh)
     launch(k_gather_rows32, (int)((T.n * nq + 255) / 256), 256, 0, s, q, nq, T.n, T.perm.as<int>(), qt.as<float>());
     TAGI_LAUNCH_CHECK();
     DevBuf basis, qtiles;
-    fill_basis_cache(T, (int)ni, items.as<AntItem>(), basis);
-    fill_charge_tiles(T, ni, items.as<AntItem>(), qt.as<float>(), nq, T.n, qtiles);
+    constexpr int tpi = kAntChunk / kTcK;
+    fill_basis_cache(T, (int)ni, items.as<AntItem>(), tpi, basis);
+    fill_charge_tiles(T, ni, items.as<AntItem>(), tpi, qt.as<float>(), nq, T.n, qtiles);
     for (int g0 = 0; g0 < nq; g0 += 8) {
         int g = nq - g0 < 8 ? nq - g0 : 8;
         part.ensure(sizeof(double) * (size_t)ni * T.P * g);
-        launch_ant_tc(g, (int)ni, items.as<AntItem>(), T.degree, basis.as<float>(), qtiles.as<float>(), nq, g0,
+        launch_ant_tc(g, (int)ni, items.as<AntItem>(), tpi, T.degree, basis.as<float>(), qtiles.as<float>(), nq, g0,
                       part.as<double>(), T.errflag.as<int>() + 1, s);
         launch(k_all_reduce, nc, 256, 0, s, off.as<int64_t>(), part.as<double>(), g, T.P, g0, nq, qh);
         TAGI_LAUNCH_CHECK();

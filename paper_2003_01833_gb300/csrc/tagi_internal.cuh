@@ -100,7 +100,7 @@ struct ProfScope {
 constexpr int kMaxDepth = 64;
 constexpr int kMaxDegree = 9;
 constexpr int kTargetsPerItem = 256;  // targets of one work item (one CTA)
-constexpr int kAntChunk = 2048;       // points per anterpolation work item
+constexpr int kAntChunk = 2048;       // points per anterpolation work item, at most
 
 // Decay rates of one call (make_rates): the first n_eps fields take
 // k = sqrt(-2 (eps + vshift)) from device eigenvalues, the others val[o]
@@ -155,6 +155,7 @@ struct Tree {
     int64_t nent = 0, nitems = 0, ntchunk = 0, nant = 0, nrec = 0;
     int64_t near_pairs = 0, far_pairs = 0;
     int64_t near_pairs_ng = 0, far_pairs_ng = 0;  // pairs of entries flagged bit2
+    int ant_chunk = kAntChunk;                     // points per anterpolation work item of this tree
     int64_t ant_points = 0;                        // sum of N_S over approximated clusters
 
     // points in tree order

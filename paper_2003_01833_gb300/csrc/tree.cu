@@ -565,6 +565,7 @@ __global__ void k_entry_shift(int64_t nent, const Entry* __restrict__ ent, const
 // position s * seg.  A unit is no longer than seg, so no item is empty, and
 // units are whole folds, so the cut moves no float32 sum.
 constexpr int kItemUnit = 256;
+constexpr int kAntChunkMin = 256, kAntItemsWanted = 1216;
 constexpr int kSegmentMax = 2048;
 constexpr int kItemsWanted = 8192;
 static_assert(kItemUnit % 16 == 0, "whole folds");
@@ -676,12 +677,12 @@ __global__ void __launch_bounds__(128) k_item_fill(int nleaf, const int* leaves,
     }
 }
 
-__global__ void k_ant_counts(int nfar, const int* far_cl, const int* begin, const int* end, int64_t* cnt)
+__global__ void k_ant_counts(int nfar, const int* far_cl, const int* begin, const int* end, int chunk, int64_t* cnt)
 {
     int f = blockIdx.x * blockDim.x + threadIdx.x;
     if (f >= nfar) return;
     int c = far_cl[f];
-    cnt[f] = (end[c] - begin[c] + kAntChunk - 1) / kAntChunk;
+    cnt[f] = (end[c] - begin[c] + chunk - 1) / chunk;
 }
 
 __global__ void k_far_points(int nfar, const int* far_cl, const int* begin, const int* end, int64_t* cnt)
@@ -692,8 +693,8 @@ __global__ void k_far_points(int nfar, const int* far_cl, const int* begin, cons
     cnt[f] = end[c] - begin[c];
 }
 
-__global__ void k_ant_fill(int nfar, const int* far_cl, const int* begin, const int* end, const int64_t* off,
-                           AntItem* items, int* far_ant0)
+__global__ void k_ant_fill(int nfar, const int* far_cl, const int* begin, const int* end, int chunk,
+                           const int64_t* off, AntItem* items, int* far_ant0)
 {
     int f = blockIdx.x * blockDim.x + threadIdx.x;
     if (f > nfar) return;
@@ -701,7 +702,7 @@ __global__ void k_ant_fill(int nfar, const int* far_cl, const int* begin, const 
     if (f == nfar) return;
     int c = far_cl[f];
     int64_t o = off[f];
-    for (int p = begin[c]; p < end[c]; p += kAntChunk) items[o++] = AntItem{p, min(end[c], p + kAntChunk), c, f};
+    for (int p = begin[c]; p < end[c]; p += chunk) items[o++] = AntItem{p, min(end[c], p + chunk), c, f};
 }
 
 // ---------------------------------------------------------------- records
@@ -1113,24 +1114,25 @@ void build_tree(Tree& T, const double* xyz, const double* w)
         DevBuf ac, ao;
         ac.ensure(8 * (size_t)T.nfar);
         ao.ensure(8 * ((size_t)T.nfar + 1));
-        launch(k_ant_counts, nblocks(T.nfar, 128), 128, 0, s, T.nfar, T.far_cl.as<int>(), T.cl_begin.as<int>(),
-                                                          T.cl_end.as<int>(), ac.as<int64_t>());
-        exclusive_scan_i64(ac.as<int64_t>(), ao.as<int64_t>(), T.nfar, s);
-        TAGI_LAUNCH_CHECK();
-        T.nant = read_i64(ao.as<int64_t>() + T.nfar, s, H);
         // sum of N_S over approximated clusters (anterpolation work, reported by tagi_tree_info)
         launch(k_far_points, nblocks(T.nfar, 128), 128, 0, s, T.nfar, T.far_cl.as<int>(), T.cl_begin.as<int>(),
                T.cl_end.as<int>(), ac.as<int64_t>());
         exclusive_scan_i64(ac.as<int64_t>(), ao.as<int64_t>(), T.nfar, s);
         TAGI_LAUNCH_CHECK();
         T.ant_points = read_i64(ao.as<int64_t>() + T.nfar, s, H);
+        // shorter items until there are kAntItemsWanted (four waves of two CTAs
+        // on 152 SMs): an item is a serial chain of point tiles
+        T.ant_chunk = kAntChunk;
+        while (T.ant_chunk > kAntChunkMin && T.ant_points / T.ant_chunk < kAntItemsWanted) T.ant_chunk /= 2;
+        launch(k_ant_counts, nblocks(T.nfar, 128), 128, 0, s, T.nfar, T.far_cl.as<int>(), T.cl_begin.as<int>(),
+                                                          T.cl_end.as<int>(), T.ant_chunk, ac.as<int64_t>());
+        exclusive_scan_i64(ac.as<int64_t>(), ao.as<int64_t>(), T.nfar, s);
+        TAGI_LAUNCH_CHECK();
+        T.nant = read_i64(ao.as<int64_t>() + T.nfar, s, H);
         T.ant_items.ensure(sizeof(AntItem) * (size_t)T.nant);
         T.far_ant0.ensure(4 * ((size_t)T.nfar + 1));
-        launch(k_ant_counts, nblocks(T.nfar, 128), 128, 0, s, T.nfar, T.far_cl.as<int>(), T.cl_begin.as<int>(),
-                                                          T.cl_end.as<int>(), ac.as<int64_t>());
-        exclusive_scan_i64(ac.as<int64_t>(), ao.as<int64_t>(), T.nfar, s);
         launch(k_ant_fill, nblocks(T.nfar + 1, 128), 128, 0, s, T.nfar, T.far_cl.as<int>(), T.cl_begin.as<int>(),
-                                                            T.cl_end.as<int>(), ao.as<int64_t>(),
+                                                            T.cl_end.as<int>(), T.ant_chunk, ao.as<int64_t>(),
                                                             T.ant_items.as<AntItem>(), T.far_ant0.as<int>());
         TAGI_LAUNCH_CHECK();
     }
