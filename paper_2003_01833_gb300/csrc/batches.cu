@@ -51,7 +51,7 @@ std::vector<V> to_host(const DevBuf& b, size_t count, cudaStream_t s)
 // puts the whole tables back.
 struct BatchSubset {
     Tree& T;
-    DevBuf items, tc_item0, tc_t0, tc_t1;
+    DevBuf items, item_order, tc_item0, tc_t0, tc_t1;  // item_order stays empty: the items in their order
     int64_t nitems = 0, ntchunk = 0;
 
     BatchSubset(Tree& t, const int32_t* batches, int nb) : T(t)
@@ -116,6 +116,7 @@ struct BatchSubset {
     void swap()
     {
         std::swap(T.items, items);
+        std::swap(T.item_order, item_order);
         std::swap(T.tc_item0, tc_item0);
         std::swap(T.tc_t0, tc_t0);
         std::swap(T.tc_t1, tc_t1);

@@ -16,12 +16,9 @@
 // the Hartree field) share one pass over the geometry.  Each thread holds a
 // pair of targets, and the near field and the tensor-grid far field run on
 // both with the packed f32x2 FMA/add/multiply (same rounding per lane as
-// scalar code).  Each CTA owns up to 256 targets of one batch (128 threads x
-// 2 targets) and a contiguous segment
-// of the batch's interaction list; its four warps share out the targets and,
-// where there are at most 128, the sources as well (see Share); source tiles
-// of 256 records are staged in
-// shared memory with positions shifted from the record's frame (its leaf or
+// scalar code).  Each CTA owns up to 128 targets of one batch and a contiguous
+// segment of the batch's interaction list; source tiles of 128 records are
+// staged in shared memory with positions shifted from the record's frame (its leaf or
 // cluster center) to the batch center in two-float arithmetic and rounded once.  Near-field
 // values and weights are two-float (see tile_near); proxies are single float.
 // rsqrt and exp2 use the MUFU unit (rsqrt.approx, ex2.approx); their mean
@@ -55,17 +52,21 @@ namespace tagi {
 
 namespace {
 
-constexpr int kTile = 256;
-// targets per thread: 2 (one f32x2 pair), 128 threads per CTA.  Measured
-// against 4 targets per thread (64 threads, 122-128 registers): more warps
-// per SM hide the MUFU latency better than the extra reuse of staged values
-// per thread buys.  The CTA always owns kTargetsPerItem targets.
-template <int NF>
-struct Tpt {
-    static constexpr int value = 2;
-    static constexpr int threads = kTargetsPerItem / value;
-};
-constexpr int kThreads64 = 256;
+constexpr int kTile = 128;
+// Targets per thread: one f32x2 pair.  A second pair would share every staged
+// value, but at 64 threads (32) a CTA it leaves too few warps: H2 iterations
+// 28.2 ms with two pairs, 27.0 with one.
+constexpr int kTpt = 2;
+// 64 threads and tiles of 128 sources: two warps of 64 consecutive targets.
+// Batches of adaptive meshes are small (340 to 500 targets on average on the Li,
+// H2 and CO meshes); with items of 256 targets, and a lane's pair 128 apart, 23
+// to 36% of all pairs were padding, now 3 to 7%.  A lane's pair is 32 apart, so
+// a warp beyond the batch's end has no targets and only stages.  Li at 99,000
+// points (build and Green step) 7.80 -> 6.4 ms, H2 iterations 33.4 -> 26.9 ms,
+// CO fields 276 -> 247 ms; with tiles of 256 (twice the shared memory) 2 to 3%
+// slower; more CTAs by asking for fewer registers, slower.
+constexpr int kThreads32 = kTargetsPerItem / kTpt;
+constexpr int kThreads64 = 128;
 constexpr int kTile64 = 128;
 
 static_assert(kThreads64 == kTargetsPerItem, "item size");
@@ -116,45 +117,28 @@ __device__ __forceinline__ void fold(float (&acc)[TPT][NF], float (&hi)[TPT][NF]
         }
 }
 
-// How the four warps of a CTA share its item.  A warp holds 64 targets (two
-// per lane), and batches of adaptive meshes are small: with one warp per 64
-// targets the item of a 100-target batch would leave half of the warps (and,
-// with a lane pair 128 targets apart, half of the packed arithmetic) on
-// padding.  On the Li, H2 and CO meshes the mean batch holds 340 to 500
-// targets and that padding is 23 to 36% of all pairs.  So items of at most
-// 128 (64) targets take two (four) groups of warps on the same targets, each
-// group every second (fourth) fold of the staged sources, and the groups' sums
-// are added at the end: 64-target granularity, 2 to 5% padding, every warp
-// busy.  Folds stay whole, so a pair's arithmetic and the float32 sum it
-// enters do not depend on the split.  With 129 to 192 targets the fourth warp
-// only helps staging.
-struct Share {
-    int grp, ngrp;  // this warp takes folds grp, grp + ngrp, ... of a tile
-    int slot;       // its lane's first target; the second is slot + 32
-    bool busy;      // the warp has targets
-    __device__ __forceinline__ Share(int nt, int warp, int lane)
-    {
-        const int lw = nt > 128 ? 2 : (nt > 64 ? 1 : 0);  // log2 of the warps across targets
-        const int tw = warp & ((1 << lw) - 1);
-        grp = warp >> lw;
-        ngrp = 4 >> lw;
-        slot = 64 * tw + lane;
-        busy = 64 * tw < nt;
-    }
-};
+// One coordinate of a staged source: the float32 nearest to the float64 sum
+// (hi + lo) + o, its two-float position in its frame plus the frame's offset o
+// = oh + ol from the batch center.  In two-float arithmetic: TwoSum(hi, oh) is
+// exact, what the low parts leave out is below slack = 2^-46 (|hi| + |oh|), and
+// where that could change the rounding (once in 1e5) the float64 sum decides.
+// The float64 form throughout costs 3 conversions and 2 additions at 2 a clock
+// and SM: 1000 clocks of that unit per 128-source tile, against 2500 of
+// arithmetic of a one-field tile.
+__device__ __noinline__ float shifted64(float hi, float lo, const double* __restrict__ cen, int frame, int batch)
+{
+    return (float)(((double)hi + (double)lo) + (cen[frame] - cen[batch]));
+}
 
-// One coordinate of a staged source: the float32 nearest to (hi + lo) +
-// (oh + ol), its two-float position in its frame plus the two-float offset of
-// the frame from the batch center.  TwoSum(hi, oh) is exact and the low parts
-// add 2^-48 of the operands, as much as the two-floats themselves leave out;
-// the same sum in float64 costs 3 conversions and 2 additions at 2 a clock
-// and SM, 60 times what float32 costs here, and took 2000 clocks of that unit
-// per 256-source tile, against 9000 of arithmetic of a one-field tile.
-__device__ __forceinline__ float shifted(float hi, float lo, float oh, float ol)
+__device__ __forceinline__ float shifted(float hi, float lo, float oh, float ol, const double* __restrict__ cen,
+                                         int frame, int batch)
 {
     float s, e;
     two_sum(hi, oh, s, e);
-    return __fadd_rn(s, __fadd_rn(e, __fadd_rn(lo, ol)));
+    const float u = __fadd_rn(e, __fadd_rn(lo, ol));
+    const float slack = 0x1p-46f * (fabsf(hi) + fabsf(oh));
+    const float a = __fadd_rn(s, __fadd_rn(u, slack)), b = __fadd_rn(s, __fsub_rn(u, slack));
+    return a == b ? a : shifted64(hi, lo, cen, frame, batch);
 }
 
 // Shared-memory layout of a staged tile: per source one float4 of position
@@ -196,15 +180,14 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __
 // GZ: the entry's Gaussian of the Coulomb SS is below float32 resolution for
 // every pair (list flag bit2), so the Hartree term is q / r alone.
 template <int NY, bool HH, bool SS, int TPT, bool GZ>
-__device__ __forceinline__ void tile_far(const Share& sh, const float4* __restrict__ srec,
-                                         const float4* __restrict__ sv, int nk,
+__device__ __forceinline__ void tile_far(const float4* __restrict__ srec, const float4* __restrict__ sv, int nk,
                                          const float2 (&ntx)[TPT / 2], const float2 (&nty)[TPT / 2],
                                          const float2 (&ntz)[TPT / 2], const float2 (&nc)[TPT / 2][NY + HH],
                                          float (&hi)[TPT][NY + HH], float (&lo)[TPT][NY + HH], const KParams& kp)
 {
     constexpr int NF = NY + HH;
     constexpr int G = TileLayout<NF>::G;
-    for (int k0 = sh.grp * kFold; k0 < nk; k0 += sh.ngrp * kFold) {
+    for (int k0 = 0; k0 < nk; k0 += kFold) {
         float acc[TPT][NF];
 #pragma unroll
         for (int j = 0; j < TPT; j++)
@@ -301,7 +284,7 @@ struct TensorLayout {
 };
 
 template <int NY, bool HH, bool SS, int TPT, int M, bool GZ>
-__device__ __forceinline__ void tile_far_tensor(const Share& sh, const float* __restrict__ sX,
+__device__ __forceinline__ void tile_far_tensor(const float* __restrict__ sX,
                                                 const float* __restrict__ sY,
                                                 const float2* __restrict__ sZ2, const float4* __restrict__ st, int np,
                                                 const float2 (&ntx)[TPT / 2], const float2 (&nty)[TPT / 2],
@@ -312,7 +295,7 @@ __device__ __forceinline__ void tile_far_tensor(const Share& sh, const float* __
     constexpr int NF = NY + HH;
     constexpr int NP = TPT / 2;
     constexpr int GF2 = TensorLayout<NF>::GF2;
-    for (int pl = 0, k2 = sh.grp; pl < np; pl++, k2 -= M) {
+    for (int pl = 0; pl < np; pl++) {
         float2 dx2[NP];
         const float xk = sX[pl];
 #pragma unroll
@@ -320,7 +303,7 @@ __device__ __forceinline__ void tile_far_tensor(const Share& sh, const float* __
             const float2 d = add2(make_float2(xk, xk), ntx[j]);
             dx2[j] = mul2(d, d);
         }
-        for (; k2 < M; k2 += sh.ngrp) {  // the rows of all planes in turn, every ngrp-th
+        for (int k2 = 0; k2 < M; k2++) {
             float2 a[NP];
             const float yk = sY[k2];
 #pragma unroll
@@ -385,7 +368,7 @@ __device__ __forceinline__ void tile_far_tensor(const Share& sh, const float* __
 // Two targets per instruction (f32x2), each lane rounding exactly as the
 // scalar form would.
 template <int NY, bool HH, bool SS, bool SELF, int TPT, bool GZ>
-__device__ __forceinline__ void tile_near(const Share& sh, const float4* __restrict__ sn, int nk,
+__device__ __forceinline__ void tile_near(const float4* __restrict__ sn, int nk,
                                           const float2 (&ntx)[TPT / 2], const float2 (&nty)[TPT / 2],
                                           const float2 (&ntz)[TPT / 2],
                                           const float2 (&nc)[TPT / 2][NY + HH], float (&hi)[TPT][NY + HH],
@@ -394,13 +377,13 @@ __device__ __forceinline__ void tile_near(const Share& sh, const float4* __restr
     constexpr int NF = NY + HH;
     constexpr int NP = TPT / 2;
     constexpr int NV4 = NearLayout<NF>::NV4;
-    for (int k0 = sh.grp * kFold; k0 < nk; k0 += sh.ngrp * kFold) {
+    for (int k0 = 0; k0 < nk; k0 += kFold) {
         float2 acc[NP][NF];
 #pragma unroll
         for (int j = 0; j < NP; j++)
 #pragma unroll
             for (int o = 0; o < NF; o++) acc[j][o] = make_float2(0.0f, 0.0f);
-#pragma unroll 4
+#pragma unroll(NF <= 3 ? 8 : 4)  // 1% faster than 4 up to three fields, slower above
         for (int k = k0; k < k0 + kFold; k++) {
             float2 v[2 * NV4];  // 0 x, 1 y, 2 z, 3 w_hi, 4 w_lo, 5 + o fh, 5 + NF + o fl
 #pragma unroll
@@ -458,7 +441,6 @@ __device__ __forceinline__ void discard_line(const void* p)
     asm volatile("discard.global.L2 [%0], 128;" ::"l"(p) : "memory");
 }
 
-template <int THREADS>
 __device__ __forceinline__ void chunk_sum(const Item& it, double* __restrict__ part, double* __restrict__ tsum,
                                           int* __restrict__ cnt, int nf_tot, int field0, int nf)
 {
@@ -469,7 +451,7 @@ __device__ __forceinline__ void chunk_sum(const Item& it, double* __restrict__ p
     __syncthreads();
     if (!s_last) return;
     __threadfence();  // the other CTAs' rows after their counts
-    for (int q = threadIdx.x; q < nf * kTargetsPerItem; q += THREADS) {
+    for (int q = threadIdx.x; q < nf * kTargetsPerItem; q += blockDim.x) {
         const int o = field0 + q / kTargetsPerItem, slot = q % kTargetsPerItem;
         if (slot >= it.t1 - it.t0) continue;  // not a target: its row entry is not written
         const double* src = part + (size_t)o * kTargetsPerItem + slot;
@@ -480,7 +462,7 @@ __device__ __forceinline__ void chunk_sum(const Item& it, double* __restrict__ p
     __syncthreads();  // every read of the rows has returned
     constexpr int kLineDoubles = 128 / sizeof(double);
     const int lines = nf * kTargetsPerItem / kLineDoubles;  // per item
-    for (int q = threadIdx.x; q < it.ni * lines; q += THREADS) {
+    for (int q = threadIdx.x; q < it.ni * lines; q += blockDim.x) {
         const int i = it.i0 + q / lines, l = q % lines;
         discard_line(part + ((size_t)i * nf_tot + field0) * kTargetsPerItem + (size_t)l * kLineDoubles);
     }
@@ -490,9 +472,11 @@ __device__ __forceinline__ void chunk_sum(const Item& it, double* __restrict__ p
 // M > 0: approximated clusters use the tensor-grid far path (degree M - 1);
 // M == 0: every entry goes through the record path.
 template <int NY, bool HH, bool SS, int M>
-__global__ void __launch_bounds__(Tpt<NY + HH>::threads) k_interact32(const Item* __restrict__ items,
+__global__ void __launch_bounds__(kThreads32) k_interact32(const Item* __restrict__ items,
+                                                           const int* __restrict__ order,
                                                            const Entry* __restrict__ ents,
                                                            const float4* __restrict__ eoff,
+                                                           const double* __restrict__ cen,
                                                            const float4* __restrict__ rec4,
                                                            const float4* __restrict__ rec4lo,
                                                            const float* __restrict__ fa, int64_t lda,
@@ -504,9 +488,9 @@ __global__ void __launch_bounds__(Tpt<NY + HH>::threads) k_interact32(const Item
     constexpr int NF = NY + HH;
     constexpr int G = TileLayout<NF>::G;
     constexpr int NV4 = NearLayout<NF>::NV4;
-    constexpr int TPT = Tpt<NF>::value;
+    constexpr int TPT = kTpt;
     constexpr int NP = TPT / 2;
-    constexpr int THREADS = Tpt<NF>::threads;
+    constexpr int THREADS = kThreads32;
     constexpr int SB = NV4 > 1 + G ? NV4 : 1 + G;  // float4 per staged source, largest layout
     static_assert(TensorLayout<NF>::GF2 <= SB, "tensor layout fits");
     // exponent factors of this launch's fields, from device memory so that a
@@ -528,17 +512,20 @@ __global__ void __launch_bounds__(Tpt<NY + HH>::threads) k_interact32(const Item
     float4* const sn = sbuf;           // near field: duplicated float2 values
     float4* const st = sbuf;           // tensor far path: (q^, w^)
 
-    const Item it = items[blockIdx.x];
+    const int id = order ? order[blockIdx.x] : (int)blockIdx.x;
+    const Item it = items[id];
     const int tid = threadIdx.x;
     const int nt = it.t1 - it.t0;
-    const Share sh(nt, tid >> 5, tid & 31);
-    static_assert(TPT == 2 && THREADS == 128, "Share's mapping: four warps of 64 targets");
+    // a warp's targets are consecutive, a lane's 32 apart, so that a warp
+    // beyond the batch's end has none and only stages
+    const int slot0 = (tid >> 5) * (32 * TPT) + (tid & 31);
+    const bool busy = (tid >> 5) * (32 * TPT) < nt;
     float2 ntx[NP], nty[NP], ntz[NP];
     float2 nc[NP][NF];
     float hi[TPT][NF], lo[TPT][NF];
 #pragma unroll
     for (int j = 0; j < TPT; j++) {
-        const int p = it.t0 + sh.slot + j * 32;
+        const int p = it.t0 + slot0 + j * 32;
         const bool ok = p < it.t1;
         const float4 r = ok ? rec4[p] : make_float4(0.f, 0.f, 0.f, 0.f);
         const float4 rl = ok ? rec4lo[p] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -586,9 +573,9 @@ __global__ void __launch_bounds__(Tpt<NY + HH>::threads) k_interact32(const Item
                     const float4 rx = rec4[en.src0 + tid * M * M];
                     const float4 ry = rec4[en.src0 + tid * M];
                     const float4 rz = rec4[en.src0 + tid];
-                    sX[tid] = shifted(rx.x, 0.0f, oh.x, ol.x);
-                    sY[tid] = shifted(ry.y, 0.0f, oh.y, ol.y);
-                    const float z = shifted(rz.z, 0.0f, oh.z, ol.z);
+                    sX[tid] = shifted(rx.x, 0.0f, oh.x, ol.x, cen, 3 * en.frame + 0, 3 * it.batch + 0);
+                    sY[tid] = shifted(ry.y, 0.0f, oh.y, ol.y, cen, 3 * en.frame + 1, 3 * it.batch + 1);
+                    const float z = shifted(rz.z, 0.0f, oh.z, ol.z, cen, 3 * en.frame + 2, 3 * it.batch + 2);
                     sZ2[tid] = make_float2(z, z);
                 }
                 for (int p0 = 0; p0 < M; p0 += PL) {
@@ -596,9 +583,8 @@ __global__ void __launch_bounds__(Tpt<NY + HH>::threads) k_interact32(const Item
                     const int nk = np * M * M;
                     const int base = en.src0 + p0 * M * M;
                     __syncthreads();
-#pragma unroll
-                    for (int h = 0; h < kTile / THREADS; h++) {
-                        const int k = tid + h * THREADS;
+#pragma unroll 2
+                    for (int k = tid; k < kTile; k += THREADS) {
                         if (k < nk) {
                             float v[2 * GF2];
 #pragma unroll
@@ -612,12 +598,12 @@ __global__ void __launch_bounds__(Tpt<NY + HH>::threads) k_interact32(const Item
                         }
                     }
                     __syncthreads();
-                    if (!sh.busy) continue;
+                    if (!busy) continue;
                     if (GZOK && gz)
-                        tile_far_tensor<NY, HH, SS, TPT, M, GZOK>(sh, sX + p0, sY, sZ2, st, np, ntx, nty, ntz, nc, hi,
+                        tile_far_tensor<NY, HH, SS, TPT, M, GZOK>(sX + p0, sY, sZ2, st, np, ntx, nty, ntz, nc, hi,
                                                                   lo, kp2);
                     else
-                        tile_far_tensor<NY, HH, SS, TPT, M, false>(sh, sX + p0, sY, sZ2, st, np, ntx, nty, ntz, nc, hi,
+                        tile_far_tensor<NY, HH, SS, TPT, M, false>(sX + p0, sY, sZ2, st, np, ntx, nty, ntz, nc, hi,
                                                                    lo, kp2);
                 }
                 continue;
@@ -631,18 +617,17 @@ __global__ void __launch_bounds__(Tpt<NY + HH>::threads) k_interact32(const Item
             const int nk = (ns + 15) & ~15;
             __syncthreads();
             if (far) {
-#pragma unroll
-                for (int h = 0; h < kTile / THREADS; h++) {
-                    const int k = tid + h * THREADS;
+#pragma unroll 2
+                for (int k = tid; k < kTile; k += THREADS) {
                     float v[4 * G];
 #pragma unroll
                     for (int m = 0; m < 4 * G; m++) v[m] = 0.0f;
                     if (k < ns) {
                         // proxy = cluster center + delta; one rounding to float32
                         float4 r = rec4[s0 + k];
-                        r.x = shifted(r.x, 0.0f, oh.x, ol.x);
-                        r.y = shifted(r.y, 0.0f, oh.y, ol.y);
-                        r.z = shifted(r.z, 0.0f, oh.z, ol.z);
+                        r.x = shifted(r.x, 0.0f, oh.x, ol.x, cen, 3 * en.frame + 0, 3 * it.batch + 0);
+                        r.y = shifted(r.y, 0.0f, oh.y, ol.y, cen, 3 * en.frame + 1, 3 * it.batch + 1);
+                        r.z = shifted(r.z, 0.0f, oh.z, ol.z, cen, 3 * en.frame + 2, 3 * it.batch + 2);
                         srec[k] = r;
 #pragma unroll
                         for (int o = 0; o < NF; o++) v[o] = fa[o * lda + s0 + k];
@@ -656,9 +641,8 @@ __global__ void __launch_bounds__(Tpt<NY + HH>::threads) k_interact32(const Item
                             sv[g * kTile + k] = make_float4(v[4 * g], v[4 * g + 1], v[4 * g + 2], v[4 * g + 3]);
                 }
             } else {
-#pragma unroll
-                for (int h = 0; h < kTile / THREADS; h++) {
-                    const int k = tid + h * THREADS;
+#pragma unroll 2
+                for (int k = tid; k < kTile; k += THREADS) {
                     float v[2 * NV4];  // x y z w_hi w_lo fh[NF] fl[NF], then padding
 #pragma unroll
                     for (int m = 0; m < 2 * NV4; m++) v[m] = 0.0f;
@@ -666,9 +650,9 @@ __global__ void __launch_bounds__(Tpt<NY + HH>::threads) k_interact32(const Item
                         // point = leaf center + (delta_hi + delta_lo); one rounding
                         const float4 r = rec4[s0 + k];
                         const float4 rl = rec4lo[s0 + k];
-                        v[0] = shifted(r.x, rl.x, oh.x, ol.x);
-                        v[1] = shifted(r.y, rl.y, oh.y, ol.y);
-                        v[2] = shifted(r.z, rl.z, oh.z, ol.z);
+                        v[0] = shifted(r.x, rl.x, oh.x, ol.x, cen, 3 * en.frame + 0, 3 * it.batch + 0);
+                        v[1] = shifted(r.y, rl.y, oh.y, ol.y, cen, 3 * en.frame + 1, 3 * it.batch + 1);
+                        v[2] = shifted(r.z, rl.z, oh.z, ol.z, cen, 3 * en.frame + 2, 3 * it.batch + 2);
                         v[3] = r.w;   // weight, high part
                         v[4] = rl.w;  // weight, low part
 #pragma unroll
@@ -687,48 +671,28 @@ __global__ void __launch_bounds__(Tpt<NY + HH>::threads) k_interact32(const Item
                 }
             }
             __syncthreads();
-            if (!sh.busy) continue;
+            if (!busy) continue;
             if (far) {
                 if (GZOK && gz)
-                    tile_far<NY, HH, SS, TPT, GZOK>(sh, srec, sv, nk, ntx, nty, ntz, nc, hi, lo, kp);
+                    tile_far<NY, HH, SS, TPT, GZOK>(srec, sv, nk, ntx, nty, ntz, nc, hi, lo, kp);
                 else
-                    tile_far<NY, HH, SS, TPT, false>(sh, srec, sv, nk, ntx, nty, ntz, nc, hi, lo, kp);
+                    tile_far<NY, HH, SS, TPT, false>(srec, sv, nk, ntx, nty, ntz, nc, hi, lo, kp);
             } else if (self) {
-                tile_near<NY, HH, SS, true, TPT, false>(sh, sn, nk, ntx, nty, ntz, nc, hi, lo, kp2);
+                tile_near<NY, HH, SS, true, TPT, false>(sn, nk, ntx, nty, ntz, nc, hi, lo, kp2);
             } else if (GZOK && gz) {
-                tile_near<NY, HH, SS, false, TPT, GZOK>(sh, sn, nk, ntx, nty, ntz, nc, hi, lo, kp2);
+                tile_near<NY, HH, SS, false, TPT, GZOK>(sn, nk, ntx, nty, ntz, nc, hi, lo, kp2);
             } else {
-                tile_near<NY, HH, SS, false, TPT, false>(sh, sn, nk, ntx, nty, ntz, nc, hi, lo, kp2);
+                tile_near<NY, HH, SS, false, TPT, false>(sn, nk, ntx, nty, ntz, nc, hi, lo, kp2);
             }
         }
     }
-    double* out = part + ((size_t)blockIdx.x * nf_tot + field0) * kTargetsPerItem;
-    // at most 64 * 4 / ngrp targets: (ngrp - 1) NF rows of that many sums fit
-    // (the largest, 3 x 64 NF, against SB >= NF + 3 rows of 512)
-    double* const red = reinterpret_cast<double*>(sbuf);
-    const int rw = kTargetsPerItem / sh.ngrp;
-    if (sh.ngrp > 1) {
-        __syncthreads();  // every warp is done with the staged tile
-        if (sh.grp > 0 && sh.busy)
+    double* out = part + ((size_t)id * nf_tot + field0) * kTargetsPerItem;
 #pragma unroll
-            for (int j = 0; j < TPT; j++)
+    for (int j = 0; j < TPT; j++)
 #pragma unroll
-                for (int o = 0; o < NF; o++)
-                    red[((sh.grp - 1) * NF + o) * rw + sh.slot + j * 32] = (double)hi[j][o] + (double)lo[j][o];
-        __syncthreads();
-    }
-    if (sh.grp == 0)
-#pragma unroll
-        for (int j = 0; j < TPT; j++)
-#pragma unroll
-            for (int o = 0; o < NF; o++) {
-                const int slot = sh.slot + j * 32;
-                if (slot >= nt) continue;
-                double S = (double)hi[j][o] + (double)lo[j][o];
-                for (int g = 1; g < sh.ngrp; g++) S += red[((g - 1) * NF + o) * rw + slot];
-                out[o * kTargetsPerItem + slot] = S;
-            }
-    chunk_sum<THREADS>(it, part, tsum, cnt, nf_tot, field0, NF);
+        for (int o = 0; o < NF; o++)
+            if (slot0 + j * 32 < nt) out[o * kTargetsPerItem + slot0 + j * 32] = (double)hi[j][o] + (double)lo[j][o];
+    chunk_sum(it, part, tsum, cnt, nf_tot, field0, NF);
 }
 
 // ---------------------------------------------------------------- bias calibration
@@ -810,6 +774,7 @@ __device__ __noinline__ double pair_slow(double r2, double k, double q, double n
 
 template <int NY, bool HH, bool SS>
 __global__ void __launch_bounds__(kThreads64) k_interact64(const Item* __restrict__ items,
+                                                           const int* __restrict__ order,
                                                            const Entry* __restrict__ ents,
                                                            const double* __restrict__ rx, const double* __restrict__ ry,
                                                            const double* __restrict__ rz, const double* __restrict__ rw,
@@ -822,7 +787,8 @@ __global__ void __launch_bounds__(kThreads64) k_interact64(const Item* __restric
     constexpr int NF = NY + HH;
     __shared__ double tab[p64::kTab];
     __shared__ double sx[kTile64], sy[kTile64], sz[kTile64], sw[kTile64], sq[NF][kTile64];
-    const Item it = items[blockIdx.x];
+    const int id = order ? order[blockIdx.x] : (int)blockIdx.x;
+    const Item it = items[id];
     const int tid = threadIdx.x;
     const int p = it.t0 + tid;
     const bool ok = p < it.t1;
@@ -882,17 +848,17 @@ __global__ void __launch_bounds__(kThreads64) k_interact64(const Item* __restric
     if (ok)
 #pragma unroll
         for (int o = 0; o < NF; o++)
-            part[((size_t)blockIdx.x * nf_tot + field0 + o) * kTargetsPerItem + tid] = acc[o];
-    chunk_sum<kThreads64>(it, part, tsum, cnt, nf_tot, field0, NF);
+            part[((size_t)id * nf_tot + field0 + o) * kTargetsPerItem + tid] = acc[o];
+    chunk_sum(it, part, tsum, cnt, nf_tot, field0, NF);
 }
 
 template <int NY, bool HH, bool SS, int M>
 void launch32_m(Tree& T, const float* kyd, const float* q, const float* c, double* part, double* tsum, int* cnt,
                 int nf_tot, int field0)
 {
-    launch(k_interact32<NY, HH, SS, M>, (int)T.nitems, Tpt<NY + HH>::threads, 0, T.stream, T.items.as<Item>(),
-           T.ent.as<Entry>(), T.ent_shift.as<float4>(), T.rec4.as<float4>(), T.rec4lo.as<float4>(), q, T.nrec, c, T.n,
-           kyd, part, tsum, cnt, nf_tot, field0);
+    launch(k_interact32<NY, HH, SS, M>, (int)T.nitems, kThreads32, 0, T.stream,
+           T.items.as<Item>(), T.item_order.as<int>(), T.ent.as<Entry>(), T.ent_shift.as<float4>(), T.cl_cen.as<double>(),
+           T.rec4.as<float4>(), T.rec4lo.as<float4>(), q, T.nrec, c, T.n, kyd, part, tsum, cnt, nf_tot, field0);
 }
 
 template <int NY, bool HH>
@@ -1014,7 +980,7 @@ void launch64(Tree& T, const double* kvd, const double* q, const double* c, doub
               int nf_tot, int field0)
 {
     launch(T.ss ? k_interact64<NY, HH, true> : k_interact64<NY, HH, false>, (int)T.nitems, kThreads64, 0, T.stream,
-           T.items.as<Item>(), T.ent.as<Entry>(), T.rx.as<double>(), T.ry.as<double>(), T.rz.as<double>(),
+           T.items.as<Item>(), T.item_order.as<int>(), T.ent.as<Entry>(), T.rx.as<double>(), T.ry.as<double>(), T.rz.as<double>(),
            T.rw.as<double>(), q, T.nrec, c, T.n, kvd, part, tsum, cnt, nf_tot, field0);
     TAGI_LAUNCH_CHECK();
 }

@@ -99,7 +99,7 @@ struct ProfScope {
 // Limits
 constexpr int kMaxDepth = 64;
 constexpr int kMaxDegree = 9;
-constexpr int kTargetsPerItem = 256;  // targets of one work item (one CTA)
+constexpr int kTargetsPerItem = 128;  // targets of one work item (one CTA)
 constexpr int kAntChunk = 2048;       // points per anterpolation work item, at most
 
 // Decay rates of one call (make_rates): the first n_eps fields take
@@ -146,6 +146,7 @@ struct Tree {
     int prec = TAGI_FP32C;
     int ss = 1;
     double alpha = 1.0;
+    bool split_items = false;  // few items: they may begin inside an entry
     int segment = 0;  // sources per work item of the near/far kernel, 0: chosen by build_tree
     int P = 0;  // (degree+1)^3
     cudaStream_t stream = nullptr;
@@ -180,6 +181,7 @@ struct Tree {
 
     // work items
     DevBuf items;       // Item[nitems]
+    DevBuf item_order;  // int[nitems]: item of each CTA (see k_item_fill), or empty: CTA i takes item i
     DevBuf tc_item0;    // int[ntchunk+1]: first item of each target chunk
     DevBuf tc_t0, tc_t1, tc_batch;  // int[ntchunk]
     DevBuf ant_items;   // AntItem[nant]

@@ -558,16 +558,18 @@ __global__ void k_entry_shift(int64_t nent, const Entry* __restrict__ ent, const
 }
 
 // ---------------------------------------------------------------- work items
-// A batch's list as a row of source positions: each entry padded to whole
-// folds of 16, cut into units where an item may begin -- every kItemUnit
-// sources of a direct entry (the kernel's tile), an approximated cluster as
-// one unit.  Item s of a target chunk starts at the first unit at or after
-// position s * seg.  A unit is no longer than seg, so no item is empty, and
-// units are whole folds, so the cut moves no float32 sum.
-constexpr int kItemUnit = 256;
+// A target chunk's items are runs of its batch's list.  Two ways to cut it:
+//   whole: an item takes whole entries until they hold at least seg sources
+//     (padded to 8), the next begins after them;
+//   split: each entry is padded to whole folds of 16 and cut into units where
+//     an item may begin -- every kItemUnit sources of a direct entry (the
+//     kernel's tile), an approximated cluster as one unit -- and item s starts
+//     at the first unit at or after position s * seg.  A unit is no longer
+//     than seg, so no item is empty, and units are whole folds, so the cut
+//     moves no float32 sum.
+constexpr int kItemUnit = 128;
+constexpr int kSegment = 8192, kItemsWanted = 8192, kItemsFew = 2000;
 constexpr int kAntChunkMin = 256, kAntItemsWanted = 1216;
-constexpr int kSegmentMax = 2048;
-constexpr int kItemsWanted = 8192;
 static_assert(kItemUnit % 16 == 0, "whole folds");
 
 __host__ __device__ __forceinline__ int padded(int v) { return (v + 15) & ~15; }
@@ -577,72 +579,98 @@ __device__ __forceinline__ int last_unit(const Entry& x)
     return (x.flags & 2) ? 0 : (x.src1 - x.src0 - 1) / kItemUnit * kItemUnit;
 }
 
+// The segments of one batch's list, by one warp, 32 entries at a time with a
+// warp prefix sum of their lengths.  start(s, e, skip) is called by one lane
+// for each segment s: it begins at source skip of entry e.  Returns their
+// number (all lanes).
+template <class F>
+__device__ int walk_segments(const Entry* __restrict__ ent, int64_t e0, int64_t e1, int seg, bool split, F&& start)
+{
+    const unsigned full = 0xffffffffu;
+    const int lane = threadIdx.x & 31;
+    if (e0 == e1 && lane == 0) start(0, (int)e0, 0);
+    int64_t at = 0, prev = -1;  // split: start of this round's first entry; of the unit before it
+    int nseg = e0 == e1 ? 1 : 0;
+    int64_t open = -1;          // whole: position where the open segment began
+    for (int64_t base = e0; base < e1; base += 32) {
+        const int64_t e = base + lane;
+        const bool live = e < e1;
+        const Entry x = live ? ent[e] : Entry{0, 0, 0, 2};
+        const int len = split ? padded(x.src1 - x.src0) : (x.src1 - x.src0 + 7) & ~7;
+        int64_t incl = len;
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t v = __shfl_up_sync(full, incl, o);
+            if (lane >= o) incl += v;
+        }
+        incl += at;
+        const int m = (int)min((int64_t)31, e1 - 1 - base);
+        if (split) {
+            const int64_t a = incl - len, last = a + (live ? last_unit(x) : 0);
+            int64_t before = __shfl_up_sync(full, last, 1);
+            if (lane == 0) before = prev;
+            if (live)
+                for (int64_t s = before < 0 ? 0 : before / seg + 1; s <= last / seg; s++) {
+                    const int64_t off = s * seg - a;  // first unit at or after off
+                    start((int)s, (int)e, off <= 0 ? 0 : (int)((off + kItemUnit - 1) / kItemUnit * kItemUnit));
+                }
+            prev = __shfl_sync(full, last, m);
+            nseg = (int)(prev / seg) + 1;
+        } else {
+            int first = 0;  // lane where the next segment begins, 32: not in this round
+            while (first <= m) {
+                if (open < 0) {
+                    open = first == 0 ? at : __shfl_sync(full, incl, first - 1);
+                    if (lane == first) start(nseg, (int)e, 0);
+                    nseg++;
+                }
+                const unsigned done = __ballot_sync(full, live && lane >= first && incl - open >= seg);
+                if (!done) break;
+                first = __ffs(done);  // the lane after the one that fills it
+                open = -1;
+            }
+        }
+        at = __shfl_sync(full, incl, m);
+    }
+    return nseg;
+}
+
 // One warp per batch: target chunks and items (chunks times segments).
 __global__ void k_item_counts(int nleaf, const int* leaves, const int* begin, const int* end, const int64_t* eoff,
-                              const Entry* ent, int seg, int64_t* nchunk, int64_t* nitem)
+                              const Entry* ent, int seg, int split, int64_t* nchunk, int64_t* nitem)
 {
-    const int j = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32), lane = threadIdx.x & 31;
+    const int j = (int)((blockIdx.x * (int64_t)blockDim.x + threadIdx.x) / 32);
     if (j >= nleaf) return;  // uniform per warp
-    const int64_t e0 = eoff[j], e1 = eoff[j + 1];
-    int64_t sum = 0;
-    for (int64_t e = e0 + lane; e < e1; e += 32) {
-        const Entry x = ent[e];
-        sum += e + 1 < e1 ? padded(x.src1 - x.src0) : last_unit(x);
-    }
-    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    if (lane == 0) {
+    const int segs = walk_segments(ent, eoff[j], eoff[j + 1], seg, split, [](int, int, int) {});
+    if ((threadIdx.x & 31) == 0) {
         const int b = leaves[j];
         const int ch = (end[b] - begin[b] + kTargetsPerItem - 1) / kTargetsPerItem;
         nchunk[j] = ch;
-        nitem[j] = ch * (sum / seg + 1);  // sum: where the last unit starts
+        nitem[j] = (int64_t)ch * segs;
     }
 }
 
-// One block per batch.  First its warp 0 finds the first unit of every
-// segment (32 entries at a time, a warp prefix sum of their padded lengths)
-// and leaves it in the first chunk's items; then all threads complete the
-// items of all chunks.
+// One block per batch.  Its warp 0 leaves the start of every segment in the
+// first chunk's items; then all threads complete the items of all chunks and
+// the order in which CTAs take them: an item runs for a millisecond on a large
+// tree, so the chunks' last items, which are shorter, come last.
 __global__ void __launch_bounds__(128) k_item_fill(int nleaf, const int* leaves, const int* begin, const int* end,
-                                                   const int64_t* eoff, const Entry* ent, int seg,
+                                                   const int64_t* eoff, const Entry* ent, int seg, int split,
                                                    const int64_t* chunk_off, const int64_t* item_off, Item* items,
-                                                   int* tc_item0, int* tc_t0, int* tc_t1, int* tc_batch)
+                                                   int64_t nitems, int64_t ntchunk, int* order, int* tc_item0, int* tc_t0, int* tc_t1, int* tc_batch)
 {
     const int j = blockIdx.x;
     const int b = leaves[j];
     const int nb = end[b] - begin[b];
-    const int64_t c0 = chunk_off[j], i0 = item_off[j], e0 = eoff[j], e1 = eoff[j + 1];
+    const int64_t c0 = chunk_off[j], i0 = item_off[j], e1 = eoff[j + 1];
     const int ch = (int)(chunk_off[j + 1] - c0);
     const int segs = (int)((item_off[j + 1] - i0) / ch);
-    if (threadIdx.x < 32) {
-        const int lane = threadIdx.x;
-        int64_t at = 0, prev = -1;  // start of this round's first entry; of the unit before it
-        if (e0 == e1 && lane == 0) {
-            items[i0].e0 = (int)e0;
-            items[i0].skip = 0;
-        }
-        for (int64_t base = e0; base < e1; base += 32) {
-            const int64_t e = base + lane;
-            const Entry x = e < e1 ? ent[e] : Entry{0, 0, 0, 2};
-            const int len = padded(x.src1 - x.src0);
-            int64_t incl = len;
-            for (int o = 1; o < 32; o <<= 1) {
-                const int64_t v = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += v;
+    if (threadIdx.x < 32)
+        walk_segments(ent, eoff[j], e1, seg, split, [&](int s, int e, int skip) {
+            if (s < segs) {
+                items[i0 + s].e0 = e;
+                items[i0 + s].skip = skip;
             }
-            const int64_t a = at + incl - len, last = a + (e < e1 ? last_unit(x) : 0);
-            int64_t before = __shfl_up_sync(0xffffffffu, last, 1);
-            if (lane == 0) before = prev;
-            if (e < e1)
-                for (int64_t s = before < 0 ? 0 : before / seg + 1; s <= last / seg && s < segs; s++) {
-                    const int64_t off = s * seg - a;  // first unit at or after off
-                    items[i0 + s].e0 = (int)e;
-                    items[i0 + s].skip = off <= 0 ? 0 : (int)((off + kItemUnit - 1) / kItemUnit * kItemUnit);
-                }
-            const int m = (int)min((int64_t)31, e1 - 1 - base);
-            prev = __shfl_sync(0xffffffffu, last, m);
-            at = __shfl_sync(0xffffffffu, a + len, m);
-        }
-    }
+        });
     __syncthreads();
     for (int q = threadIdx.x; q < ch * segs; q += blockDim.x) {
         const int ci = q / segs, s = q % segs;
@@ -668,6 +696,8 @@ __global__ void __launch_bounds__(128) k_item_fill(int nleaf, const int* leaves,
             it.e0 = f0;
             it.skip = skip;
         }
+        // the CTA that takes it: the last, shorter item of every chunk after all others
+        order[s < segs - 1 ? first + s - tc : nitems - ntchunk + tc] = (int)(first + s);
         if (s == 0) {
             tc_item0[tc] = (int)first;
             tc_t0[tc] = t0;
@@ -1062,22 +1092,20 @@ void build_tree(Tree& T, const double* xyz, const double* w)
     TAGI_LAUNCH_CHECK();
 
     // ---- work items of the near/far kernel
-    // Sources per item.  Where the caller leaves it open: short enough for
-    // kItemsWanted items (nine waves of 152 SMs at 6 CTAs), so that the SMs end
-    // together, and not shorter than a unit.  With one length of 8192 the 5,003
-    // point cube ran 64 CTAs over 5,003 sources each: 204 us, 91 with this
-    // rule; the uniform hydrogen mesh 663 -> 498 us.  At most kSegmentMax: an
-    // item of 8192 sources runs about a millisecond, and the last ones leave
-    // SMs idle.  1024 / 2048 / 4096 / 8192 gave 38.93 / 38.75 / 38.76 / 38.93
-    // ms for the Li step, 26.89 / 26.91 / 27.14 / 27.66 for three H2
-    // iterations and 252.8 / 251.0 / 250.4 / 250.5 for the CO fields.
-    const int unit = std::max(kItemUnit, padded(T.P));
-    int seg = T.segment;
-    if (seg == 0) {
-        const int64_t rows = (T.near_pairs + T.far_pairs) / kTargetsPerItem;
-        seg = (int)std::min<int64_t>(std::max<int64_t>(rows / kItemsWanted, unit), kSegmentMax);
+    // Large trees: whole entries, kSegment sources (or the caller's number) an
+    // item, so that the order in which a target's two-float sums are added
+    // stays as it is.  Where that leaves fewer than kItemsFew items (1.3 waves
+    // of 152 SMs at 10 CTAs) the SMs would wait for a few long ones: the items
+    // are split until there are kItemsWanted.  The 5,003 point cube ran 64 CTAs
+    // over 5,003 sources each, 334 us a call at first, 82 split; the uniform
+    // hydrogen mesh (400 items) 689 -> 446 us.
+    const int64_t rows = (T.near_pairs + T.far_pairs) / kTargetsPerItem;
+    int seg_src = T.segment ? T.segment : kSegment;
+    T.split_items = rows / seg_src < kItemsFew;
+    if (T.split_items) {
+        const int unit = std::max(kItemUnit, padded(T.P));  // no unit is longer than an item
+        seg_src = (int)std::max<int64_t>(std::min<int64_t>(seg_src, rows / kItemsWanted), unit);
     }
-    const int seg_src = std::max(seg, unit);
     DevBuf nch, nit, choff, itoff;
     nch.ensure(8 * (size_t)nleaf);
     nit.ensure(8 * (size_t)nleaf);
@@ -1085,21 +1113,25 @@ void build_tree(Tree& T, const double* xyz, const double* w)
     itoff.ensure(8 * ((size_t)nleaf + 1));
     launch(k_item_counts, nblocks(32 * (int64_t)nleaf, 128), 128, 0, s, nleaf, T.leaves.as<int>(), T.cl_begin.as<int>(),
                                                       T.cl_end.as<int>(), T.ent_off.as<int64_t>(), T.ent.as<Entry>(),
-                                                      seg_src, nch.as<int64_t>(), nit.as<int64_t>());
+                                                      seg_src, T.split_items ? 1 : 0, nch.as<int64_t>(),
+                                                      nit.as<int64_t>());
     exclusive_scan_i64(nch.as<int64_t>(), choff.as<int64_t>(), nleaf, s);
     exclusive_scan_i64(nit.as<int64_t>(), itoff.as<int64_t>(), nleaf, s);
     TAGI_LAUNCH_CHECK();
     T.ntchunk = read_i64(choff.as<int64_t>() + nleaf, s, H);
     T.nitems = read_i64(itoff.as<int64_t>() + nleaf, s, H);
     T.items.ensure(sizeof(Item) * (size_t)std::max<int64_t>(T.nitems, 1));
+    T.item_order.ensure(4 * (size_t)std::max<int64_t>(T.nitems, 1));
     T.tc_item0.ensure(4 * ((size_t)T.ntchunk + 1));
     T.tc_t0.ensure(4 * (size_t)T.ntchunk);
     T.tc_t1.ensure(4 * (size_t)T.ntchunk);
     T.tc_batch.ensure(4 * (size_t)T.ntchunk);
     launch(k_item_fill, nleaf, 128, 0, s, nleaf, T.leaves.as<int>(), T.cl_begin.as<int>(),
                                                     T.cl_end.as<int>(), T.ent_off.as<int64_t>(), T.ent.as<Entry>(),
-                                                    seg_src, choff.as<int64_t>(), itoff.as<int64_t>(),
-                                                    T.items.as<Item>(), T.tc_item0.as<int>(), T.tc_t0.as<int>(),
+                                                    seg_src, T.split_items ? 1 : 0, choff.as<int64_t>(),
+                                                    itoff.as<int64_t>(),
+                                                    T.items.as<Item>(), T.nitems, T.ntchunk,
+                                                    T.item_order.as<int>(), T.tc_item0.as<int>(), T.tc_t0.as<int>(),
                                                     T.tc_t1.as<int>(), T.tc_batch.as<int>());
     TAGI_LAUNCH_CHECK();
     {

@@ -1,6 +1,6 @@
-"""The FP32C near/far kernel's split of an item over its warps: batches whose
-target counts sit at the edges of the groups (64 targets a warp, two or four
-source groups below 129 and 65 targets, 256 targets an item).  Parity with the
+"""The near/far kernel's items: batches whose target counts sit at the edges
+of its warps and items (64 targets a warp, 128 an item), and lists cut into
+items at other places.  Parity with the
 float64 oracle within the stated FP32C tolerance, relative L2 1e-6 per field.
 """
 import numpy as np
@@ -53,7 +53,7 @@ def test_one_batch_at_the_edges(T, n):
 
 @pytest.mark.parametrize("degree", [5, 6, 8])  # record path, tensor-grid path with 7 and 9 nodes
 @pytest.mark.parametrize("leaf", [40, 90, 180, 700])
-def test_far_field_over_groups(T, degree, leaf):
+def test_far_field_over_batch_sizes(T, degree, leaf):
     check(T, 12007, leaf, degree, seed=leaf + degree)
 
 
