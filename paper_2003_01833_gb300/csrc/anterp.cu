@@ -881,7 +881,6 @@ void anterpolate_weights(Tree& T)
         launch(k_ant_reduce_w, T.nfar, 256, 0, s, T.far_ant0.as<int>(), T.antpart.as<double>(), T.P, T.n,
                T.rec4.as<float4>());
         TAGI_LAUNCH_CHECK();
-        TAGI_CUDA(cudaStreamSynchronize(s));
     } else {
         T.antpart.ensure(sizeof(double) * (size_t)T.nant * T.P);
         launch_ant<double, double>(1, (int)T.nant, T.ant_items.as<AntItem>(), T, T.pw.as<double>(), T.n,

@@ -11,6 +11,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <initializer_list>
 #include <cstring>
 #include <utility>
 
@@ -37,29 +38,38 @@ __device__ __forceinline__ double unord64(unsigned long long o)
 }
 
 // ---------------------------------------------------------------- scans
-__global__ void k_scan_i64(const int64_t* __restrict__ in, int64_t* __restrict__ out, int64_t n)
+__global__ void __launch_bounds__(kScanThreads) k_scan_i64(const int64_t* __restrict__ in, int64_t* __restrict__ out,
+                                                           int64_t n)
 {
-    __shared__ int64_t sm[kScanThreads];
-    const int tid = threadIdx.x;
+    __shared__ int64_t ws[kScanThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t per = (n + kScanThreads - 1) / kScanThreads;
     const int64_t a = min(n, (int64_t)tid * per), b = min(n, a + per);
     int64_t s = 0;
     for (int64_t i = a; i < b; i++) s += in[i];
-    sm[tid] = s;
-    __syncthreads();
-    for (int off = 1; off < kScanThreads; off <<= 1) {  // Hillis-Steele inclusive
-        int64_t v = tid >= off ? sm[tid - off] : 0;
-        __syncthreads();
-        sm[tid] += v;
-        __syncthreads();
+    int64_t x = s;  // inclusive over the warp
+    for (int o = 1; o < 32; o <<= 1) {
+        const int64_t v = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += v;
     }
-    int64_t run = sm[tid] - s;
+    if (lane == 31) ws[warp] = x;
+    __syncthreads();
+    if (warp == 0) {
+        int64_t y = ws[lane];
+        for (int o = 1; o < 32; o <<= 1) {
+            const int64_t v = __shfl_up_sync(0xffffffffu, y, o);
+            if (lane >= o) y += v;
+        }
+        ws[lane] = y;
+    }
+    __syncthreads();
+    int64_t run = x - s + (warp > 0 ? ws[warp - 1] : 0);
     for (int64_t i = a; i < b; i++) {
-        int64_t v = in[i];
+        const int64_t v = in[i];
         out[i] = run;
         run += v;
     }
-    if (tid == kScanThreads - 1) out[n] = sm[tid];
+    if (tid == kScanThreads - 1) out[n] = run;
 }
 
 // ---------------------------------------------------------------- level passes
@@ -72,62 +82,90 @@ __global__ void k_init(int* pos, int* seg, int64_t n)
     }
 }
 
-__global__ void k_init_clusters(int first, int last, unsigned long long* blo, unsigned long long* bhi)
+__global__ void k_init_root(int n, int* begin, int* end, int* parent, int* level, int* nchild,
+                            unsigned long long* blo, unsigned long long* bhi)
 {
-    int c = first + blockIdx.x * blockDim.x + threadIdx.x;
-    if (c < last)
-        for (int d = 0; d < 3; d++) {
-            blo[3 * c + d] = ~0ull;
-            bhi[3 * c + d] = 0ull;
-        }
+    begin[0] = 0;
+    end[0] = n;
+    parent[0] = -1;
+    level[0] = 0;
+    nchild[0] = 0;
+    for (int d = 0; d < 3; d++) {
+        blo[d] = ~0ull;
+        bhi[d] = 0ull;
+    }
 }
 
-// Bounding boxes of the clusters owning seg[p] >= 0.
-__global__ void k_bbox(const int* __restrict__ pos, const int* __restrict__ seg, const double* __restrict__ xyz,
-                       int64_t n, unsigned long long* blo, unsigned long long* bhi)
+// Bounding boxes of the clusters owning seg[p] >= 0.  Positions of a cluster
+// are consecutive, so most blocks hold one cluster: its warps reduce by
+// shuffles, the block in shared memory, and six atomics go out instead of six a
+// warp (which serialise on the root's six words).
+constexpr int kBoxThreads = 256;
+__global__ void __launch_bounds__(kBoxThreads) k_bbox(const int* __restrict__ pos, const int* __restrict__ seg,
+                                                      const double* __restrict__ xyz, int64_t n,
+                                                      unsigned long long* blo, unsigned long long* bhi)
 {
-    int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    int c = -1;
+    __shared__ unsigned long long smn[kBoxThreads / 32][3], smx[kBoxThreads / 32][3];
+    const int64_t p = blockIdx.x * (int64_t)kBoxThreads + threadIdx.x;
+    const int c = p < n ? seg[p] : -1;
     unsigned long long v[3] = {0, 0, 0};
-    if (p < n) {
-        c = seg[p];
-        if (c >= 0) {
-            int i = pos[p];
-            v[0] = ord64(xyz[i]);
-            v[1] = ord64(xyz[n + i]);
-            v[2] = ord64(xyz[2 * n + i]);
-        }
+    if (c >= 0) {
+        const int i = pos[p];
+        v[0] = ord64(xyz[i]);
+        v[1] = ord64(xyz[n + i]);
+        v[2] = ord64(xyz[2 * n + i]);
     }
     const unsigned full = 0xffffffffu;
-    int c0 = __shfl_sync(full, c, 0);
-    bool uniform = __all_sync(full, c == c0);
-    if (uniform) {
-        if (c0 < 0) return;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __shared__ int sc;
+    if (threadIdx.x == 0) sc = c;
+    __syncthreads();
+    const bool one = __syncthreads_and(c == sc);
+    if (one && sc < 0) return;
+    if (one || __all_sync(full, c == __shfl_sync(full, c, 0))) {
         unsigned long long mn[3] = {v[0], v[1], v[2]}, mx[3] = {v[0], v[1], v[2]};
         for (int off = 16; off > 0; off >>= 1)
             for (int d = 0; d < 3; d++) {
-                unsigned long long a = __shfl_down_sync(full, mn[d], off);
-                unsigned long long b = __shfl_down_sync(full, mx[d], off);
+                const unsigned long long a = __shfl_down_sync(full, mn[d], off), b = __shfl_down_sync(full, mx[d], off);
                 mn[d] = min(mn[d], a);
                 mx[d] = max(mx[d], b);
             }
-        if ((threadIdx.x & 31) == 0)
+        if (one) {
+            if (lane == 0)
+                for (int d = 0; d < 3; d++) {
+                    smn[warp][d] = mn[d];
+                    smx[warp][d] = mx[d];
+                }
+        } else if (lane == 0 && c >= 0) {
             for (int d = 0; d < 3; d++) {
-                atomicMin(&blo[3 * c0 + d], mn[d]);
-                atomicMax(&bhi[3 * c0 + d], mx[d]);
+                atomicMin(&blo[3 * c + d], mn[d]);
+                atomicMax(&bhi[3 * c + d], mx[d]);
             }
+        }
     } else if (c >= 0) {
         for (int d = 0; d < 3; d++) {
             atomicMin(&blo[3 * c + d], v[d]);
             atomicMax(&bhi[3 * c + d], v[d]);
         }
     }
+    if (!one) return;
+    __syncthreads();
+    if (threadIdx.x < 3) {
+        const int d = threadIdx.x;
+        unsigned long long mn = smn[0][d], mx = smx[0][d];
+        for (int w = 1; w < kBoxThreads / 32; w++) {
+            mn = min(mn, smn[w][d]);
+            mx = max(mx, smx[w][d]);
+        }
+        atomicMin(&blo[3 * c + d], mn);
+        atomicMax(&bhi[3 * c + d], mx);
+    }
 }
 
 // Finish boxes of clusters [first, last): lo/hi, center, radius; decide the split.
 __global__ void k_finalize(int first, int last, const unsigned long long* blo, const unsigned long long* bhi,
                            const int* begin, const int* end, int leaf_size, double* lo, double* hi,
-                           double* cen, double* rad, double* mid, int* smask, int* nsplit)
+                           double* cen, double* rad, double* mid, int* smask)
 {
     int c = first + blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= last) return;
@@ -148,43 +186,37 @@ __global__ void k_finalize(int first, int last, const unsigned long long* blo, c
     if (end[c] - begin[c] > leaf_size && emax > 0.0) {
         for (int d = 0; d < 3; d++)
             if (__dmul_rn(e[d], kSqrt2) >= emax) m |= 1 << d;
-        atomicAdd(nsplit, 1);
     }
     smask[c] = m;
     for (int d = 0; d < 3; d++) mid[3 * c + d] = cen[3 * c + d];
 }
 
-__global__ void k_codes(const int* __restrict__ pos, const int* __restrict__ seg, const double* __restrict__ xyz,
-                        int64_t n, const int* __restrict__ smask, const double* __restrict__ mid,
-                        signed char* code)
+// Child code of every position (-1 outside the clusters being split), and per
+// block of kBlk positions the number of positions with each code, stored
+// bin-major: cnt[b * nblk + blk].
+__global__ void __launch_bounds__(kBlk) k_codes(const int* __restrict__ pos, const int* __restrict__ seg,
+                                                const double* __restrict__ xyz, int64_t n,
+                                                const int* __restrict__ smask, const double* __restrict__ mid,
+                                                signed char* code, int64_t nblk, int64_t* cnt)
 {
-    int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    int c = seg[p];
+    __shared__ int wc[kBlk / 32][8];
+    const int64_t p = blockIdx.x * (int64_t)kBlk + threadIdx.x;
     int k = -1;
+    const int c = p < n ? seg[p] : -1;
     if (c >= 0) {
-        int m = smask[c];
+        const int m = smask[c];
         if (m) {
-            int i = pos[p];
+            const int i = pos[p];
             k = 0;
             for (int d = 0; d < 3; d++)
                 if ((m >> d) & 1)
                     if (xyz[d * n + i] >= mid[3 * c + d]) k |= 1 << d;
         }
     }
-    code[p] = (signed char)k;
-}
-
-// Per block of kBlk positions: number of positions with each code, stored
-// bin-major: cnt[b * nblk + blk].
-__global__ void k_blkcount(const signed char* __restrict__ code, int64_t n, int64_t nblk, int64_t* cnt)
-{
-    __shared__ int wc[kBlk / 32][8];
-    int64_t p = blockIdx.x * (int64_t)kBlk + threadIdx.x;
-    int k = p < n ? code[p] : -1;
-    int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    code[p] = (signed char)k;  // the array holds whole blocks
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int b = 0; b < 8; b++) {
-        unsigned m = __ballot_sync(0xffffffffu, k == b);
+        const unsigned m = __ballot_sync(0xffffffffu, k == b);
         if (lane == 0) wc[warp][b] = __popc(m);
     }
     __syncthreads();
@@ -201,10 +233,12 @@ __device__ void prefix8(const int64_t* off, const signed char* code, int64_t nbl
 {
     const int64_t blk = x / kBlk;
     int cnt[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    for (int64_t q = blk * kBlk + lane; q < x; q += 32) {
-        const int k = code[q];
+    // four codes a load; bytes at or beyond x do not count
+    for (int64_t q = blk * kBlk + 4 * lane; q < x; q += 128) {
+        unsigned w = *reinterpret_cast<const unsigned*>(code + q);
+        if (x - q < 4) w |= 0xffffffffu << (8 * (int)(x - q));
 #pragma unroll
-        for (int b = 0; b < 8; b++) cnt[b] += (k == b);
+        for (int b = 0; b < 8; b++) cnt[b] += __popc(__vcmpeq4(w, b * 0x01010101u)) >> 3;
     }
 #pragma unroll
     for (int b = 0; b < 8; b++) {
@@ -329,6 +363,28 @@ __global__ void k_is_leaf(int nc, const int* nch, int64_t* flag)
 {
     int c = blockIdx.x * blockDim.x + threadIdx.x;
     if (c < nc) flag[c] = nch[c] == 0;
+}
+
+// flag[c] = approximated, size[c] = its points (0 otherwise)
+__global__ void k_far_flags(int nc, const int* is_far, const int* begin, const int* end, int64_t* flag, int64_t* size)
+{
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    if (c >= nc) return;
+    flag[c] = is_far[c];
+    size[c] = is_far[c] ? end[c] - begin[c] : 0;
+}
+
+// Values that the host reads together: one copy and one wait for all of them.
+constexpr int kReadMax = 8;
+struct ReadList {
+    const int64_t* p64[kReadMax];
+    const int* p32[kReadMax];
+    int n;
+};
+__global__ void k_collect(ReadList L, int64_t* out)
+{
+    const int i = threadIdx.x;
+    if (i < L.n) out[i] = L.p64[i] ? *L.p64[i] : (int64_t)*L.p32[i];
 }
 
 __global__ void k_compact(int nc, const int64_t* flag, const int64_t* off, int* out, int* idx_of)
@@ -698,6 +754,7 @@ __global__ void __launch_bounds__(128) k_item_fill(int nleaf, const int* leaves,
         }
         // the CTA that takes it: the last, shorter item of every chunk after all others
         order[s < segs - 1 ? first + s - tc : nitems - ntchunk + tc] = (int)(first + s);
+        if (tc == ntchunk - 1 && s == 0) tc_item0[ntchunk] = (int)nitems;
         if (s == 0) {
             tc_item0[tc] = (int)first;
             tc_t0[tc] = t0;
@@ -713,14 +770,6 @@ __global__ void k_ant_counts(int nfar, const int* far_cl, const int* begin, cons
     if (f >= nfar) return;
     int c = far_cl[f];
     cnt[f] = (end[c] - begin[c] + chunk - 1) / chunk;
-}
-
-__global__ void k_far_points(int nfar, const int* far_cl, const int* begin, const int* end, int64_t* cnt)
-{
-    int f = blockIdx.x * blockDim.x + threadIdx.x;
-    if (f >= nfar) return;
-    int c = far_cl[f];
-    cnt[f] = end[c] - begin[c];
 }
 
 __global__ void k_ant_fill(int nfar, const int* far_cl, const int* begin, const int* end, int chunk,
@@ -769,9 +818,12 @@ __global__ void k_point_records(int64_t n, const double* px, const double* py, c
 __global__ void k_proxy_records(int nfar, const int* far_cl, int degree, int64_t n, const double* lo,
                                 const double* hi, float4* rec4, double* rx, double* ry, double* rz)
 {
+    __shared__ double node[kMaxDegree + 1];
     int f = blockIdx.x;
     int c = far_cl[f];
     int m = degree + 1, P = m * m * m;
+    if (threadIdx.x < m) node[threadIdx.x] = cos(M_PI * threadIdx.x / degree);
+    __syncthreads();
     double cc[3], hh[3];
     for (int d = 0; d < 3; d++) {
         cc[d] = (lo[3 * c + d] + hi[3 * c + d]) * 0.5;
@@ -779,7 +831,7 @@ __global__ void k_proxy_records(int nfar, const int* far_cl, int degree, int64_t
     }
     for (int k = threadIdx.x; k < P; k += blockDim.x) {
         int k1 = k / (m * m), k2 = (k / m) % m, k3 = k % m;
-        double s1 = cos(M_PI * k1 / degree), s2 = cos(M_PI * k2 / degree), s3 = cos(M_PI * k3 / degree);
+        double s1 = node[k1], s2 = node[k2], s3 = node[k3];
         int64_t r = n + (int64_t)f * P + k;
         if (rec4) {
             // the float32 anterpolation interpolates on the float32-rounded
@@ -805,14 +857,27 @@ __global__ void k_check_finite(const double* a, int64_t n, int* bad)
 
 inline int nblocks(int64_t n, int t) { return (int)((n + t - 1) / t); }
 
+// Pinned host words for values read back, once per host thread.
 struct Host1 {
-    // pinned scalars for readbacks, allocated once per host thread
     int64_t* h = nullptr;
+    DevBuf dev;
     Host1()
     {
         thread_local int64_t* buf = nullptr;
-        if (!buf) TAGI_CUDA(cudaMallocHost(&buf, 8 * sizeof(int64_t)));
+        if (!buf) TAGI_CUDA(cudaMallocHost(&buf, kReadMax * sizeof(int64_t)));
         h = buf;
+        dev.ensure(kReadMax * sizeof(int64_t));
+    }
+    // the values at the given device addresses into h[0], h[1], ...
+    void read(cudaStream_t s, std::initializer_list<const int64_t*> p64, std::initializer_list<const int*> p32 = {})
+    {
+        ReadList L{};
+        for (const int64_t* p : p64) L.p64[L.n++] = p;
+        for (const int* p : p32) L.p32[L.n++] = p;
+        launch(k_collect, 1, 32, 0, s, L, dev.as<int64_t>());
+        TAGI_LAUNCH_CHECK();
+        TAGI_CUDA(cudaMemcpyAsync(h, dev.p, L.n * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
+        TAGI_CUDA(cudaStreamSynchronize(s));
     }
 };
 
@@ -822,20 +887,6 @@ void exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, cudaStream_t
 {
     launch(k_scan_i64, 1, kScanThreads, 0, s, in, out, n);
     TAGI_LAUNCH_CHECK();
-}
-
-static int64_t read_i64(const int64_t* dev, cudaStream_t s, Host1& h)
-{
-    TAGI_CUDA(cudaMemcpyAsync(h.h, dev, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-    TAGI_CUDA(cudaStreamSynchronize(s));
-    return h.h[0];
-}
-
-static int read_i32(const int* dev, cudaStream_t s, Host1& h)
-{
-    TAGI_CUDA(cudaMemcpyAsync(h.h, dev, sizeof(int), cudaMemcpyDeviceToHost, s));
-    TAGI_CUDA(cudaStreamSynchronize(s));
-    return (int)((int*)h.h)[0];
 }
 
 // Grow every per-cluster array to hold `cap` clusters, keeping contents.
@@ -852,8 +903,7 @@ static void grow_clusters(Tree& T, int cur, int cap, DevBuf& blo, DevBuf& bhi, c
         DevBuf nb;
         nb.ensure(x.per * (size_t)cap);
         if (x.b->p && cur > 0) TAGI_CUDA(cudaMemcpyAsync(nb.p, x.b->p, x.per * (size_t)cur, cudaMemcpyDeviceToDevice, s));
-        TAGI_CUDA(cudaStreamSynchronize(s));
-        *x.b = std::move(nb);
+        *x.b = std::move(nb);  // the old block goes back to this stream's cache, behind the copy
     }
 }
 
@@ -863,26 +913,25 @@ void build_tree(Tree& T, const double* xyz, const double* w)
     const int64_t n = T.n;
     TAGI_REQUIRE(n <= (int64_t)0x3fffffff, "n too large for 32-bit tree positions");
     Host1 H;
-    // ---- input validation (non-finite coordinates or weights)
+    // ---- input validation (non-finite coordinates or weights): flag[0], read
+    // with the first level's result; flag[1]: partition consistency
     DevBuf flag;
     flag.ensure(64);
     TAGI_CUDA(cudaMemsetAsync(flag.p, 0, 64, s));
     launch(k_check_finite, nblocks(3 * n, 256), 256, 0, s, xyz, 3 * n, flag.as<int>());
     launch(k_check_finite, nblocks(n, 256), 256, 0, s, w, n, flag.as<int>());
     TAGI_LAUNCH_CHECK();
-    TAGI_REQUIRE(read_i32(flag.as<int>(), s, H) == 0, "xyz or w holds a non-finite value");
 
-    DevBuf posA, posB, segA, segB, code, blo, bhi, mid, smask, nsplit;
+    DevBuf posA, posB, segA, segB, code, blo, bhi, mid, smask;
     posA.ensure(4 * n);
     posB.ensure(4 * n);
     segA.ensure(4 * n);
     segB.ensure(4 * n);
-    code.ensure(n);
     const int64_t nblk = (n + kBlk - 1) / kBlk;
+    code.ensure((size_t)nblk * kBlk);
     DevBuf bcnt, boff;
     bcnt.ensure(8 * 8 * nblk);
     boff.ensure(8 * (8 * nblk + 1));
-    nsplit.ensure(16);
 
     int cap = 1024;
     grow_clusters(T, 0, cap, blo, bhi, s);
@@ -890,55 +939,24 @@ void build_tree(Tree& T, const double* xyz, const double* w)
     smask.ensure(4 * (size_t)cap);
 
     launch(k_init, nblocks(n, 256), 256, 0, s, posA.as<int>(), segA.as<int>(), n);
-    {
-        int one_begin = 0, one_end = (int)n, minus1 = -1, zero = 0;
-        TAGI_CUDA(cudaMemcpyAsync(T.cl_begin.p, &one_begin, 4, cudaMemcpyHostToDevice, s));
-        TAGI_CUDA(cudaMemcpyAsync(T.cl_end.p, &one_end, 4, cudaMemcpyHostToDevice, s));
-        TAGI_CUDA(cudaMemcpyAsync(T.cl_parent.p, &minus1, 4, cudaMemcpyHostToDevice, s));
-        TAGI_CUDA(cudaMemcpyAsync(T.cl_level.p, &zero, 4, cudaMemcpyHostToDevice, s));
-        TAGI_CUDA(cudaMemcpyAsync(T.cl_nchild.p, &zero, 4, cudaMemcpyHostToDevice, s));
-        TAGI_CUDA(cudaStreamSynchronize(s));
-    }
-    launch(k_init_clusters, 1, 32, 0, s, 0, 1, blo.as<unsigned long long>(), bhi.as<unsigned long long>());
+    launch(k_init_root, 1, 1, 0, s, (int)n, T.cl_begin.as<int>(), T.cl_end.as<int>(), T.cl_parent.as<int>(),
+           T.cl_level.as<int>(), T.cl_nchild.as<int>(), blo.as<unsigned long long>(), bhi.as<unsigned long long>());
     TAGI_LAUNCH_CHECK();
 
+    // One wait per level: the number of new clusters, which sizes the arrays
+    // that the next kernels write and ends the loop when it is zero.
     int first = 0, last = 1, nc = 1, lvl = 0;
     DevBuf cnt, pfx, nnz, cbase, bfirst, bid;
     while (true) {
         const int nl = last - first;
-        launch(k_bbox, nblocks(n, 256), 256, 0, s, posA.as<int>(), segA.as<int>(), xyz, n, blo.as<unsigned long long>(),
-                                                bhi.as<unsigned long long>());
-        TAGI_CUDA(cudaMemsetAsync(nsplit.p, 0, 4, s));
+        launch(k_bbox, nblocks(n, kBoxThreads), kBoxThreads, 0, s, posA.as<int>(), segA.as<int>(), xyz, n,
+               blo.as<unsigned long long>(), bhi.as<unsigned long long>());
         launch(k_finalize, nblocks(nl, 128), 128, 0, s, first, last, blo.as<unsigned long long>(),
-                                                     bhi.as<unsigned long long>(), T.cl_begin.as<int>(),
-                                                     T.cl_end.as<int>(), T.leaf_size, T.cl_lo.as<double>(),
-                                                     T.cl_hi.as<double>(), T.cl_cen.as<double>(),
-                                                     T.cl_rad.as<double>(), mid.as<double>(), smask.as<int>(),
-                                                     nsplit.as<int>());
-        TAGI_LAUNCH_CHECK();
-        int ns = read_i32(nsplit.as<int>(), s, H);
-        if (ns == 0) {
-            // the last level are all leaves
-            TAGI_CUDA(cudaMemsetAsync(T.cl_nchild.as<int>() + first, 0, 4 * (size_t)nl, s));
-            break;
-        }
-        TAGI_REQUIRE(lvl < kMaxDepth, "tree deeper than 64 levels (degenerate point set)");
-        if (nc + 8 * ns > cap) {
-            int ncap = std::max(2 * cap, nc + 8 * ns);
-            grow_clusters(T, nc, ncap, blo, bhi, s);
-            DevBuf m2, s2;
-            m2.ensure(24 * (size_t)ncap);
-            s2.ensure(4 * (size_t)ncap);
-            TAGI_CUDA(cudaMemcpyAsync(m2.p, mid.p, 24 * (size_t)nc, cudaMemcpyDeviceToDevice, s));
-            TAGI_CUDA(cudaMemcpyAsync(s2.p, smask.p, 4 * (size_t)nc, cudaMemcpyDeviceToDevice, s));
-            TAGI_CUDA(cudaStreamSynchronize(s));
-            mid = std::move(m2);
-            smask = std::move(s2);
-            cap = ncap;
-        }
-        launch(k_codes, nblocks(n, 256), 256, 0, s, posA.as<int>(), segA.as<int>(), xyz, n, smask.as<int>(),
-                                                mid.as<double>(), code.as<signed char>());
-        launch(k_blkcount, (int)nblk, kBlk, 0, s, code.as<signed char>(), n, nblk, bcnt.as<int64_t>());
+               bhi.as<unsigned long long>(), T.cl_begin.as<int>(), T.cl_end.as<int>(), T.leaf_size,
+               T.cl_lo.as<double>(), T.cl_hi.as<double>(), T.cl_cen.as<double>(), T.cl_rad.as<double>(),
+               mid.as<double>(), smask.as<int>());
+        launch(k_codes, (int)nblk, kBlk, 0, s, posA.as<int>(), segA.as<int>(), xyz, n, smask.as<int>(),
+               mid.as<double>(), code.as<signed char>(), nblk, bcnt.as<int64_t>());
         exclusive_scan_i64(bcnt.as<int64_t>(), boff.as<int64_t>(), 8 * nblk, s);
         cnt.ensure(32 * (size_t)nl);
         pfx.ensure(64 * (size_t)nl);
@@ -946,33 +964,46 @@ void build_tree(Tree& T, const double* xyz, const double* w)
         cbase.ensure(8 * ((size_t)nl + 1));
         bfirst.ensure(32 * (size_t)nl);
         bid.ensure(32 * (size_t)nl);
-        launch(k_counts, nblocks(32 * (int64_t)nl, 128), 128, 0, s, first, last, T.cl_begin.as<int>(), T.cl_end.as<int>(),
-                                                   smask.as<int>(), code.as<signed char>(), boff.as<int64_t>(), nblk,
-                                                   cnt.as<int>(), pfx.as<int64_t>(), nnz.as<int64_t>());
+        launch(k_counts, nblocks(32 * (int64_t)nl, 128), 128, 0, s, first, last, T.cl_begin.as<int>(),
+               T.cl_end.as<int>(), smask.as<int>(), code.as<signed char>(), boff.as<int64_t>(), nblk, cnt.as<int>(),
+               pfx.as<int64_t>(), nnz.as<int64_t>());
         exclusive_scan_i64(nnz.as<int64_t>(), cbase.as<int64_t>(), nl, s);
         TAGI_LAUNCH_CHECK();
-        int64_t nnew = read_i64(cbase.as<int64_t>() + nl, s, H);
+        H.read(s, {cbase.as<int64_t>() + nl}, {flag.as<int>(), flag.as<int>() + 1});
+        TAGI_REQUIRE(H.h[1] == 0, "xyz or w holds a non-finite value");
+        TAGI_REQUIRE(H.h[2] == 0, "tree partition consistency check failed");
+        const int nnew = (int)H.h[0];
+        if (nnew == 0) {
+            // the last level are all leaves
+            TAGI_CUDA(cudaMemsetAsync(T.cl_nchild.as<int>() + first, 0, 4 * (size_t)nl, s));
+            break;
+        }
+        TAGI_REQUIRE(lvl < kMaxDepth, "tree deeper than 64 levels (degenerate point set)");
+        if (nc + nnew > cap) {
+            const int ncap = std::max(2 * cap, nc + nnew);
+            grow_clusters(T, nc, ncap, blo, bhi, s);
+            // both are written again for the next level before they are read
+            mid.ensure(24 * (size_t)ncap);
+            smask.ensure(4 * (size_t)ncap);
+            cap = ncap;
+        }
         launch(k_children, nblocks(nl, 128), 128, 0, s, first, last, nc, cbase.as<int64_t>(), T.cl_begin.as<int>(),
-                                                     cnt.as<int>(), lvl, T.cl_begin.as<int>(), T.cl_end.as<int>(),
-                                                     T.cl_parent.as<int>(), T.cl_level.as<int>(),
-                                                     T.cl_nchild.as<int>(), T.cl_child.as<int>(), bfirst.as<int>(),
-                                                     bid.as<int>(), blo.as<unsigned long long>(),
-                                                     bhi.as<unsigned long long>());
+               cnt.as<int>(), lvl, T.cl_begin.as<int>(), T.cl_end.as<int>(), T.cl_parent.as<int>(),
+               T.cl_level.as<int>(), T.cl_nchild.as<int>(), T.cl_child.as<int>(), bfirst.as<int>(), bid.as<int>(),
+               blo.as<unsigned long long>(), bhi.as<unsigned long long>());
         launch(k_scatter, (int)nblk, kBlk, 0, s, posA.as<int>(), segA.as<int>(), code.as<signed char>(), n, nblk,
-                                             boff.as<int64_t>(), first, pfx.as<int64_t>(), bfirst.as<int>(),
-                                             bid.as<int>(), cnt.as<int>(), posB.as<int>(), segB.as<int>(),
-                                             flag.as<int>());
+               boff.as<int64_t>(), first, pfx.as<int64_t>(), bfirst.as<int>(), bid.as<int>(), cnt.as<int>(),
+               posB.as<int>(), segB.as<int>(), flag.as<int>() + 1);
         TAGI_LAUNCH_CHECK();
         std::swap(posA, posB);
         std::swap(segA, segB);
         first = nc;
-        nc += (int)nnew;
+        nc += nnew;
         last = nc;
         lvl++;
     }
     T.nc = nc;
     T.depth = lvl;
-    TAGI_REQUIRE(read_i32(flag.as<int>(), s, H) == 0, "tree partition consistency check failed");
 
     // ---- points in tree order
     T.perm.ensure(4 * n);
@@ -1000,7 +1031,8 @@ void build_tree(Tree& T, const double* xyz, const double* w)
     fo.ensure(8 * ((size_t)nc + 1));
     launch(k_is_leaf, nblocks(nc, 256), 256, 0, s, nc, T.cl_nchild.as<int>(), fl.as<int64_t>());
     exclusive_scan_i64(fl.as<int64_t>(), fo.as<int64_t>(), nc, s);
-    T.nleaf = (int)read_i64(fo.as<int64_t>() + nc, s, H);
+    H.read(s, {fo.as<int64_t>() + nc});
+    T.nleaf = (int)H.h[0];
     T.leaves.ensure(4 * (size_t)T.nleaf);
     launch(k_compact, nblocks(nc, 256), 256, 0, s, nc, fl.as<int64_t>(), fo.as<int64_t>(), T.leaves.as<int>(), nullptr);
     T.pt_leaf.ensure(4 * n);
@@ -1024,15 +1056,17 @@ void build_tree(Tree& T, const double* xyz, const double* w)
                                                    fpair.as<int64_t>(), err.as<int>());
     exclusive_scan_i64(lc.as<int64_t>(), lo_.as<int64_t>(), nleaf, s);
     TAGI_LAUNCH_CHECK();
-    TAGI_REQUIRE(read_i32(err.as<int>(), s, H) == 0, "interaction-list stack overflow");
-    T.nent = read_i64(lo_.as<int64_t>() + nleaf, s, H);
     {
-        DevBuf tmp;
-        tmp.ensure(8 * ((size_t)nleaf + 1));
-        exclusive_scan_i64(npair.as<int64_t>(), tmp.as<int64_t>(), nleaf, s);
-        T.near_pairs = read_i64(tmp.as<int64_t>() + nleaf, s, H);
-        exclusive_scan_i64(fpair.as<int64_t>(), tmp.as<int64_t>(), nleaf, s);
-        T.far_pairs = read_i64(tmp.as<int64_t>() + nleaf, s, H);
+        DevBuf t1, t2;
+        t1.ensure(8 * ((size_t)nleaf + 1));
+        t2.ensure(8 * ((size_t)nleaf + 1));
+        exclusive_scan_i64(npair.as<int64_t>(), t1.as<int64_t>(), nleaf, s);
+        exclusive_scan_i64(fpair.as<int64_t>(), t2.as<int64_t>(), nleaf, s);
+        H.read(s, {lo_.as<int64_t>() + nleaf, t1.as<int64_t>() + nleaf, t2.as<int64_t>() + nleaf}, {err.as<int>()});
+        TAGI_REQUIRE(H.h[3] == 0, "interaction-list stack overflow");
+        T.nent = H.h[0];
+        T.near_pairs = H.h[1];
+        T.far_pairs = H.h[2];
     }
     TAGI_REQUIRE(T.nent < (int64_t)0x7fffffff, "too many interaction entries");
     T.ent.ensure(sizeof(Entry) * (size_t)std::max<int64_t>(T.nent, 1));
@@ -1047,26 +1081,29 @@ void build_tree(Tree& T, const double* xyz, const double* w)
                                                   T.ent_batch.as<int>(), T.ent_clus.as<int>(), isfar.as<int>(),
                                                   err.as<int>());
     TAGI_LAUNCH_CHECK();
-    TAGI_REQUIRE(read_i32(err.as<int>(), s, H) == 0, "interaction-list fill disagrees with its count");
 
     // ---- approximated clusters
     {
-        DevBuf f64, o64;
+        DevBuf f64, o64, z64, zo;
         f64.ensure(8 * (size_t)nc);
         o64.ensure(8 * ((size_t)nc + 1));
-        // widen flags to int64 for the scan
-        std::vector<int> hf(nc);
-        TAGI_CUDA(cudaMemcpyAsync(hf.data(), isfar.p, 4 * (size_t)nc, cudaMemcpyDeviceToHost, s));
-        TAGI_CUDA(cudaStreamSynchronize(s));
-        std::vector<int64_t> hf64(hf.begin(), hf.end());
-        TAGI_CUDA(cudaMemcpyAsync(f64.p, hf64.data(), 8 * (size_t)nc, cudaMemcpyHostToDevice, s));
-        exclusive_scan_i64(f64.as<int64_t>(), o64.as<int64_t>(), nc, s);
-        T.nfar = (int)read_i64(o64.as<int64_t>() + nc, s, H);
-        T.far_cl.ensure(4 * (size_t)std::max(T.nfar, 1));
+        z64.ensure(8 * (size_t)nc);
+        zo.ensure(8 * ((size_t)nc + 1));
+        T.far_cl.ensure(4 * (size_t)nc);
         T.cl_far.ensure(4 * (size_t)nc);
+        launch(k_far_flags, nblocks(nc, 256), 256, 0, s, nc, isfar.as<int>(), T.cl_begin.as<int>(), T.cl_end.as<int>(),
+               f64.as<int64_t>(), z64.as<int64_t>());
+        exclusive_scan_i64(f64.as<int64_t>(), o64.as<int64_t>(), nc, s);
+        exclusive_scan_i64(z64.as<int64_t>(), zo.as<int64_t>(), nc, s);
         launch(k_compact, nblocks(nc, 256), 256, 0, s, nc, f64.as<int64_t>(), o64.as<int64_t>(), T.far_cl.as<int>(),
                                                    T.cl_far.as<int>());
         TAGI_LAUNCH_CHECK();
+        // ant_points: sum of N_S over approximated clusters (anterpolation
+        // work, reported by tagi_tree_info)
+        H.read(s, {o64.as<int64_t>() + nc, zo.as<int64_t>() + nc}, {err.as<int>()});
+        TAGI_REQUIRE(H.h[2] == 0, "interaction-list fill disagrees with its count");
+        T.nfar = (int)H.h[0];
+        T.ant_points = H.h[1];
     }
     T.nrec = n + (int64_t)T.nfar * T.P;
     TAGI_REQUIRE(T.nrec < (int64_t)0x7fffffff, "too many source records");
@@ -1077,18 +1114,27 @@ void build_tree(Tree& T, const double* xyz, const double* w)
         launch(k_entry_shift, nblocks(T.nent, 256), 256, 0, s, T.nent, T.ent.as<Entry>(), T.ent_batch.as<int>(),
                T.cl_cen.as<double>(), T.ent_shift.as<float4>());
     }
-    T.near_pairs_ng = T.far_pairs_ng = 0;
-    if (T.nent > 0) {
-        DevBuf ng;
-        ng.ensure(2 * sizeof(int64_t));
-        TAGI_CUDA(cudaMemsetAsync(ng.p, 0, 2 * sizeof(int64_t), s));
+    DevBuf ng;
+    ng.ensure(2 * sizeof(int64_t));
+    TAGI_CUDA(cudaMemsetAsync(ng.p, 0, 2 * sizeof(int64_t), s));
+    if (T.nent > 0)
         launch(k_gauss_flags, nblocks(T.nent, 256), 256, 0, s, T.nent, T.ent.as<Entry>(), T.ent_batch.as<int>(),
                T.ent_clus.as<int>(), T.cl_lo.as<double>(), T.cl_hi.as<double>(), T.cl_begin.as<int>(),
                T.cl_end.as<int>(), T.alpha, ng.as<unsigned long long>());
-        TAGI_LAUNCH_CHECK();
-        T.near_pairs_ng = read_i64(ng.as<int64_t>(), s, H);
-        T.far_pairs_ng = read_i64(ng.as<int64_t>() + 1, s, H);
-    }
+    TAGI_LAUNCH_CHECK();
+
+    // ---- anterpolation items (counted here, with the work items)
+    DevBuf ac, ao;
+    ac.ensure(8 * (size_t)std::max(T.nfar, 1));
+    ao.ensure(8 * ((size_t)T.nfar + 1));
+    // shorter items until there are kAntItemsWanted (four waves of two CTAs on
+    // 152 SMs): an item is a serial chain of point tiles
+    T.ant_chunk = kAntChunk;
+    while (T.ant_chunk > kAntChunkMin && T.ant_points / T.ant_chunk < kAntItemsWanted) T.ant_chunk /= 2;
+    if (T.nfar > 0)
+        launch(k_ant_counts, nblocks(T.nfar, 128), 128, 0, s, T.nfar, T.far_cl.as<int>(), T.cl_begin.as<int>(),
+               T.cl_end.as<int>(), T.ant_chunk, ac.as<int64_t>());
+    exclusive_scan_i64(ac.as<int64_t>(), ao.as<int64_t>(), T.nfar, s);
     TAGI_LAUNCH_CHECK();
 
     // ---- work items of the near/far kernel
@@ -1118,8 +1164,13 @@ void build_tree(Tree& T, const double* xyz, const double* w)
     exclusive_scan_i64(nch.as<int64_t>(), choff.as<int64_t>(), nleaf, s);
     exclusive_scan_i64(nit.as<int64_t>(), itoff.as<int64_t>(), nleaf, s);
     TAGI_LAUNCH_CHECK();
-    T.ntchunk = read_i64(choff.as<int64_t>() + nleaf, s, H);
-    T.nitems = read_i64(itoff.as<int64_t>() + nleaf, s, H);
+    H.read(s, {choff.as<int64_t>() + nleaf, itoff.as<int64_t>() + nleaf, ng.as<int64_t>(), ng.as<int64_t>() + 1,
+               ao.as<int64_t>() + T.nfar});
+    T.ntchunk = H.h[0];
+    T.nitems = H.h[1];
+    T.near_pairs_ng = H.h[2];
+    T.far_pairs_ng = H.h[3];
+    T.nant = H.h[4];
     T.items.ensure(sizeof(Item) * (size_t)std::max<int64_t>(T.nitems, 1));
     T.item_order.ensure(4 * (size_t)std::max<int64_t>(T.nitems, 1));
     T.tc_item0.ensure(4 * ((size_t)T.ntchunk + 1));
@@ -1134,33 +1185,7 @@ void build_tree(Tree& T, const double* xyz, const double* w)
                                                     T.item_order.as<int>(), T.tc_item0.as<int>(), T.tc_t0.as<int>(),
                                                     T.tc_t1.as<int>(), T.tc_batch.as<int>());
     TAGI_LAUNCH_CHECK();
-    {
-        int tot = (int)T.nitems;
-        TAGI_CUDA(cudaMemcpyAsync(T.tc_item0.as<int>() + T.ntchunk, &tot, 4, cudaMemcpyHostToDevice, s));
-        TAGI_CUDA(cudaStreamSynchronize(s));
-    }
-
-    // ---- anterpolation items
-    T.ant_points = 0;
     if (T.nfar > 0) {
-        DevBuf ac, ao;
-        ac.ensure(8 * (size_t)T.nfar);
-        ao.ensure(8 * ((size_t)T.nfar + 1));
-        // sum of N_S over approximated clusters (anterpolation work, reported by tagi_tree_info)
-        launch(k_far_points, nblocks(T.nfar, 128), 128, 0, s, T.nfar, T.far_cl.as<int>(), T.cl_begin.as<int>(),
-               T.cl_end.as<int>(), ac.as<int64_t>());
-        exclusive_scan_i64(ac.as<int64_t>(), ao.as<int64_t>(), T.nfar, s);
-        TAGI_LAUNCH_CHECK();
-        T.ant_points = read_i64(ao.as<int64_t>() + T.nfar, s, H);
-        // shorter items until there are kAntItemsWanted (four waves of two CTAs
-        // on 152 SMs): an item is a serial chain of point tiles
-        T.ant_chunk = kAntChunk;
-        while (T.ant_chunk > kAntChunkMin && T.ant_points / T.ant_chunk < kAntItemsWanted) T.ant_chunk /= 2;
-        launch(k_ant_counts, nblocks(T.nfar, 128), 128, 0, s, T.nfar, T.far_cl.as<int>(), T.cl_begin.as<int>(),
-                                                          T.cl_end.as<int>(), T.ant_chunk, ac.as<int64_t>());
-        exclusive_scan_i64(ac.as<int64_t>(), ao.as<int64_t>(), T.nfar, s);
-        TAGI_LAUNCH_CHECK();
-        T.nant = read_i64(ao.as<int64_t>() + T.nfar, s, H);
         T.ant_items.ensure(sizeof(AntItem) * (size_t)T.nant);
         T.far_ant0.ensure(4 * ((size_t)T.nfar + 1));
         launch(k_ant_fill, nblocks(T.nfar + 1, 128), 128, 0, s, T.nfar, T.far_cl.as<int>(), T.cl_begin.as<int>(),
@@ -1192,7 +1217,6 @@ void build_tree(Tree& T, const double* xyz, const double* w)
                                                fp32 ? nullptr : T.rz.as<double>());
     TAGI_LAUNCH_CHECK();
     anterpolate_weights(T);
-    TAGI_CUDA(cudaStreamSynchronize(s));
 }
 
 }  // namespace tagi
