@@ -151,6 +151,27 @@ constexpr int kTcK = 32;                             // points per tensor-core t
 constexpr int kTileFloats = 3 * kAntLP * kTcK;       // basis floats of one tile (4608 bytes)
 static_assert(kAntTile % kTcK == 0, "whole tiles per item");
 
+// Nodes cos(pi k / n) and 1 / prod_{j != k} (s_k - s_j), once per tree: out[k],
+// out[kMaxDegree + 1 + k].  (The anterpolation kernels' CTAs would spend longer
+// on them in float64 than on a few tiles of points.)  f32: the FP32C proxies
+// sit on the float32-rounded nodes, where that form interpolates.
+__global__ void k_ant_nodes(int degree, int f32, double* __restrict__ out)
+{
+    __shared__ double node[kMaxDegree + 1];
+    const int k = threadIdx.x;
+    if (k <= degree) {
+        const double s = cos(M_PI * k / degree);
+        node[k] = f32 ? (double)(float)s : s;
+    }
+    __syncthreads();
+    if (k > degree) return;
+    double d = 1.0;
+    for (int j = 0; j <= degree; j++)
+        if (j != k) d *= node[k] - node[j];
+    out[k] = node[k];
+    out[kMaxDegree + 1 + k] = 1.0 / d;
+}
+
 // index of basis value k of dimension d of point j of item `item` in the basis
 // cache: tpi tiles of 32 points an item, each [3][kAntLP][32]
 __host__ __device__ inline size_t antl_index(size_t item, int tpi, int j, int d, int k)
@@ -170,10 +191,10 @@ __global__ void __launch_bounds__(kAntThreads) k_ant_basis(const AntItem* __rest
                                                            const double* __restrict__ py,
                                                            const double* __restrict__ pz,
                                                            const double* __restrict__ lo,
-                                                           const double* __restrict__ hi, int degree, int tpi,
+                                                           const double* __restrict__ hi,
+                                                           const double* __restrict__ nodes, int degree, int tpi,
                                                            float* __restrict__ antL)
 {
-    __shared__ double dnodes[kMaxDegree + 1], inv[kMaxDegree + 1];
     __shared__ float fnodes[kMaxDegree + 1];
     __shared__ F2 finv[kMaxDegree + 1];
     const AntItem it = items[blockIdx.x];
@@ -184,16 +205,9 @@ __global__ void __launch_bounds__(kAntThreads) k_ant_basis(const AntItem* __rest
         hh[d] = (hi[3 * c + d] - lo[3 * c + d]) * 0.5;
         ih[d] = hh[d] == 0.0 ? 0.0 : 1.0 / hh[d];
     }
-    if (threadIdx.x == 0) {
-        for (int k = 0; k <= degree; k++) dnodes[k] = (double)(float)cos(M_PI * k / degree);
-        for (int k = 0; k <= degree; k++) {
-            double d = 1.0;
-            for (int j = 0; j <= degree; j++)
-                if (j != k) d *= dnodes[k] - dnodes[j];
-            inv[k] = 1.0 / d;
-            fnodes[k] = (float)dnodes[k];
-            finv[k] = df_of(inv[k]);
-        }
+    if (threadIdx.x <= degree) {
+        fnodes[threadIdx.x] = (float)nodes[threadIdx.x];
+        finv[threadIdx.x] = df_of(nodes[kMaxDegree + 1 + threadIdx.x]);
     }
     __syncthreads();
     const int np = it.p1 - it.p0;
@@ -223,13 +237,13 @@ template <class R, class A, int NQ>
 __global__ void __launch_bounds__(kAntThreads) k_ant(const AntItem* __restrict__ items, const double* __restrict__ px,
                                                      const double* __restrict__ py, const double* __restrict__ pz,
                                                      const double* __restrict__ lo, const double* __restrict__ hi,
-                                                     int degree, int f32nodes, const R* __restrict__ q,
+                                                     const double* __restrict__ nodes, int degree,
+                                                     const R* __restrict__ q,
                                                      int64_t ldq, double* __restrict__ part,
                                                      const float* __restrict__ antL, int tpi)
 {
     __shared__ R Ls[kAntTile][3][kMaxDegree + 1];
     __shared__ R qs[NQ][kAntTile];
-    __shared__ R nodes[kMaxDegree + 1];
     const AntItem it = items[blockIdx.x];
     const int m = degree + 1, P = m * m * m;
     const int c = it.cluster;
@@ -240,19 +254,9 @@ __global__ void __launch_bounds__(kAntThreads) k_ant(const AntItem* __restrict__
         ih[d] = hh[d] == 0.0 ? 0.0 : 1.0 / hh[d];
     }
     __shared__ double dnodes[kMaxDegree + 1], inv[kMaxDegree + 1];
-    if (threadIdx.x == 0) {
-        // FP32C proxies sit on the float32-rounded nodes; interpolate there
-        for (int k = 0; k <= degree; k++) {
-            const double sk = cos(M_PI * k / degree);
-            nodes[k] = f32nodes ? (R)(float)sk : (R)sk;
-            dnodes[k] = (double)nodes[k];
-        }
-        for (int k = 0; k <= degree; k++) {
-            double d = 1.0;
-            for (int j = 0; j <= degree; j++)
-                if (j != k) d *= dnodes[k] - dnodes[j];
-            inv[k] = 1.0 / d;
-        }
+    if (threadIdx.x <= degree) {
+        dnodes[threadIdx.x] = nodes[threadIdx.x];
+        inv[threadIdx.x] = nodes[kMaxDegree + 1 + threadIdx.x];
     }
     int k1[kMaxPPT], k2[kMaxPPT], k3[kMaxPPT];
     A acc[kMaxPPT][NQ];
@@ -727,37 +731,51 @@ __global__ void k_qtiles(const AntItem* __restrict__ items, int64_t nitems, int 
     qT[e] = it.p0 + j < it.p1 ? q[col * ldq + it.p0 + j] : 0.0f;
 }
 
-// Sum the partials of every item of far cluster f (fixed order) and store.
+// Sum the partials of every item of far cluster f = blockIdx.x (fixed order)
+// and store; one entry a thread.  The root's cluster has hundreds of items:
+// eight of them are in flight at a time.
 // mode 0: float rows dst32[(col0+col) * ldd + n + f P + k];
 // mode 1: double rows dst64[...].
-__global__ void k_ant_reduce(int nfar, const int* far_ant0, const double* part, int nq, int P, int64_t n,
-                             int mode, float* dst32, double* dst64, int col0, int64_t ldd)
+constexpr int kReduceThreads = 128;
+__global__ void __launch_bounds__(kReduceThreads) k_ant_reduce(const int* far_ant0, const double* __restrict__ part,
+                                                               int nq, int P, int64_t n, int mode, float* dst32,
+                                                               double* dst64, int col0, int64_t ldd)
 {
     const int f = blockIdx.x;
     const int a0 = far_ant0[f], a1 = far_ant0[f + 1];
-    for (int e = threadIdx.x; e < nq * P; e += blockDim.x) {
-        int col = e / P, k = e % P;
-        double s = 0.0;
-        for (int a = a0; a < a1; a++) s += part[((size_t)a * nq + col) * P + k];
-        int64_t r = n + (int64_t)f * P + k;
-        if (mode == 0)
-            dst32[(col0 + col) * ldd + r] = (float)s;
-        else
-            dst64[(col0 + col) * ldd + r] = s;
-    }
+    const int e = blockIdx.y * kReduceThreads + threadIdx.x;
+    if (e >= nq * P) return;
+    const double* p = part + (size_t)a0 * nq * P + e;
+    double s = 0.0;
+#pragma unroll 8
+    for (int a = 0; a < a1 - a0; a++) s += p[(size_t)a * nq * P];
+    const int col = e / P, k = e % P;
+    const int64_t r = n + (int64_t)f * P + k;
+    if (mode == 0)
+        dst32[(col0 + col) * ldd + r] = (float)s;
+    else
+        dst64[(col0 + col) * ldd + r] = s;
 }
 
 // w^ of far cluster f from the two columns (w_hi, w_lo) of a two-float weight:
 // rec4[n + f P + k].w = sum over items and both columns.
-__global__ void k_ant_reduce_w(const int* far_ant0, const double* part, int P, int64_t n, float4* rec4)
+__global__ void __launch_bounds__(kReduceThreads) k_ant_reduce_w(const int* far_ant0, const double* __restrict__ part,
+                                                                 int P, int64_t n, float4* rec4)
 {
     const int f = blockIdx.x;
     const int a0 = far_ant0[f], a1 = far_ant0[f + 1];
-    for (int k = threadIdx.x; k < P; k += blockDim.x) {
-        double s = 0.0;
-        for (int a = a0; a < a1; a++) s += part[((size_t)a * 2 + 0) * P + k] + part[((size_t)a * 2 + 1) * P + k];
-        rec4[n + (int64_t)f * P + k].w = (float)s;
-    }
+    const int k = blockIdx.y * kReduceThreads + threadIdx.x;
+    if (k >= P) return;
+    const double* p = part + (size_t)a0 * 2 * P + k;
+    double s = 0.0;
+#pragma unroll 8
+    for (int a = 0; a < a1 - a0; a++) s += p[(size_t)a * 2 * P] + p[(size_t)a * 2 * P + P];
+    rec4[n + (int64_t)f * P + k].w = (float)s;
+}
+
+inline dim3 reduce_grid(int nfar, int entries)
+{
+    return dim3((unsigned)nfar, (unsigned)((entries + kReduceThreads - 1) / kReduceThreads));
 }
 
 __global__ void k_split_w(const double* w, int64_t n, float* out)
@@ -778,7 +796,7 @@ void launch_ant(int nq, int nitems, const AntItem* items, Tree& T, const R* q, i
     case NQ:                                                                                                \
         launch(k_ant<R, A, NQ>, nitems, kAntThreads, 0, s, items, T.px.as<double>(), T.py.as<double>(),         \
                                                        T.pz.as<double>(), T.cl_lo.as<double>(),             \
-                                                       T.cl_hi.as<double>(), T.degree, T.prec == TAGI_FP32C, q, ldq, part, antL, tpi); \
+                                                       T.cl_hi.as<double>(), T.ant_nodes.as<double>(), T.degree, q, ldq, part, antL, tpi); \
         break;
     switch (nq) {
         TAGI_ANT_CASE(1)
@@ -839,7 +857,8 @@ void fill_basis_cache(Tree& T, int nitems, const AntItem* items, int tpi, DevBuf
 {
     cache.ensure(sizeof(float) * (size_t)nitems * tpi * kTileFloats);
     launch(k_ant_basis, nitems, kAntThreads, 0, T.stream, items, T.px.as<double>(), T.py.as<double>(),
-           T.pz.as<double>(), T.cl_lo.as<double>(), T.cl_hi.as<double>(), T.degree, tpi, cache.as<float>());
+           T.pz.as<double>(), T.cl_lo.as<double>(), T.cl_hi.as<double>(), T.ant_nodes.as<double>(), T.degree, tpi,
+           cache.as<float>());
     TAGI_LAUNCH_CHECK();
 }
 
@@ -856,8 +875,11 @@ void fill_charge_tiles(Tree& T, int64_t nitems, const AntItem* items, int tpi, c
 
 void anterpolate_weights(Tree& T)
 {
-    if (T.nfar == 0) return;
     cudaStream_t s = T.stream;
+    T.ant_nodes.ensure(sizeof(double) * 2 * (kMaxDegree + 1));
+    launch(k_ant_nodes, 1, 32, 0, s, T.degree, T.prec == TAGI_FP32C ? 1 : 0, T.ant_nodes.as<double>());
+    TAGI_LAUNCH_CHECK();
+    if (T.nfar == 0) return;
     if (T.prec == TAGI_FP32C) {
         // basis cache, kept with the tree
         const int tpi = T.ant_chunk / kTcK;
@@ -878,14 +900,15 @@ void anterpolate_weights(Tree& T)
         else
             launch_ant<float, double>(2, (int)T.nant, T.ant_items.as<AntItem>(), T, w2.as<float>(), T.n,
                                       T.antpart.as<double>(), s, antL, tpi);
-        launch(k_ant_reduce_w, T.nfar, 256, 0, s, T.far_ant0.as<int>(), T.antpart.as<double>(), T.P, T.n,
+        launch(k_ant_reduce_w, reduce_grid(T.nfar, T.P), kReduceThreads, 0, s, T.far_ant0.as<int>(), T.antpart.as<double>(), T.P, T.n,
                T.rec4.as<float4>());
         TAGI_LAUNCH_CHECK();
     } else {
         T.antpart.ensure(sizeof(double) * (size_t)T.nant * T.P);
         launch_ant<double, double>(1, (int)T.nant, T.ant_items.as<AntItem>(), T, T.pw.as<double>(), T.n,
                                    T.antpart.as<double>(), s);
-        launch(k_ant_reduce, T.nfar, 256, 0, s, T.nfar, T.far_ant0.as<int>(), T.antpart.as<double>(), 1, T.P, T.n,
+        launch(k_ant_reduce, reduce_grid(T.nfar, T.P), kReduceThreads, 0, s, T.far_ant0.as<int>(),
+               T.antpart.as<double>(), 1, T.P, T.n,
                1, nullptr, T.rw.as<double>(), 0, 0);
         TAGI_LAUNCH_CHECK();
     }
@@ -902,7 +925,8 @@ void anterpolate_fields32(Tree& T, int nf)
         T.antpart.ensure(sizeof(double) * (size_t)T.nant * T.P * g);
         launch_ant_tc(g, (int)T.nant, T.ant_items.as<AntItem>(), tpi, T.degree, T.antL.as<float>(), T.qtiles.as<float>(),
                       nf, g0, T.antpart.as<double>(), T.errflag.as<int>() + 1, s);
-        launch(k_ant_reduce, T.nfar, 256, 0, s, T.nfar, T.far_ant0.as<int>(), T.antpart.as<double>(), g, T.P, T.n, 0,
+        launch(k_ant_reduce, reduce_grid(T.nfar, g * T.P), kReduceThreads, 0, s, T.far_ant0.as<int>(),
+               T.antpart.as<double>(), g, T.P, T.n, 0,
                                             T.fa.as<float>(), nullptr, g0, T.nrec);
         TAGI_LAUNCH_CHECK();
     }
@@ -917,7 +941,8 @@ void anterpolate_fields64(Tree& T, int nf)
         T.antpart.ensure(sizeof(double) * (size_t)T.nant * T.P * g);
         launch_ant<double, double>(g, (int)T.nant, T.ant_items.as<AntItem>(), T, T.q64.as<double>() + g0 * T.nrec,
                                    T.nrec, T.antpart.as<double>(), s);
-        launch(k_ant_reduce, T.nfar, 256, 0, s, T.nfar, T.far_ant0.as<int>(), T.antpart.as<double>(), g, T.P, T.n, 1,
+        launch(k_ant_reduce, reduce_grid(T.nfar, g * T.P), kReduceThreads, 0, s, T.far_ant0.as<int>(),
+               T.antpart.as<double>(), g, T.P, T.n, 1,
                                             nullptr, T.q64.as<double>(), g0, T.nrec);
         TAGI_LAUNCH_CHECK();
     }

@@ -201,6 +201,7 @@ struct Tree {
     DevBuf part;        // double partial sums [nitems][nf][kTargetsPerItem]
     DevBuf tsum;        // double [ntchunk][nf][kTargetsPerItem]: partials summed per target chunk
     DevBuf tc_cnt;      // int [ntchunk]: items of the chunk finished in the current launch (0 between launches)
+    DevBuf ant_nodes;   // double: interpolation nodes and their weights (anterp.cu)
     DevBuf antpart;     // double anterpolation partials
     DevBuf antL;        // FP32C: float32 basis rows of every anterpolation point (anterp.cu)
     DevBuf qtiles;      // FP32C: charge tiles of the tensor-core anterpolation (anterp.cu)
