@@ -753,14 +753,14 @@ __global__ void k_calibrate(int mode, long long n, double* out)
 
 // ---------------------------------------------------------------- FP64 plain form
 // Up to kMax64 fields share one pass over the geometry: the kernel is bound by
-// the float64 unit (1.68 operations a clock and SM), and a pair costs it 10
-// operations for 1/r and r and 4 a field (pair64.cuh); with the math library's
+// the float64 unit (1.68 operations a clock and SM), and a pair costs it 8
+// operations of geometry and 4 a field (pair64.cuh); with the math library's
 // sqrt, exp and a division it took 47 slots a field.  One thread per target:
 // two warps a scheduler keep that unit busy, so there is nothing to gain from
 // more targets a thread, and warps without targets only stage.  The uniform
-// hydrogen mesh (32,768 points, 8.3e8 pairs, one field) takes 23.0 ms a call,
+// hydrogen mesh (32,768 points, 8.3e8 pairs, one field) takes 18.7 ms a call,
 // 75.5 before; the errors of ri, r and the exponential are below the math
-// library's (0.62 / 0.81 against 0.75 / 0.96 units of 2^-52 (1 + k r)).
+// library's (0.62 / 0.73 against 0.75 / 0.96 units of 2^-52 (1 + k r)).
 constexpr int kMax64 = 4;
 
 // a pair that the fast forms do not take (r = 0 is skipped, Eq. direct-sum)
@@ -831,16 +831,17 @@ __global__ void __launch_bounds__(kThreads64) k_interact64(const Item* __restric
                         acc[o] += pair_slow(r2, kv[o], sq[o][k], nc[o], sw[k], o >= NY, SS);
                     continue;
                 }
-                double ri, r;
-                p64::inv_sqrt(r2, ri, r);
+                const p64::Root R = p64::root(r2);
+                const float h = p64::small32(R.h);
 #pragma unroll
                 for (int o = 0; o < NY; o++) {
                     const double d = SS ? fma(nc[o], sw[k], sq[o][k]) : sq[o][k];
-                    acc[o] = fma(p64::exp_neg(r, rate[o], tab), ri * d, acc[o]);
+                    acc[o] = fma(p64::exp_neg(R.t, h, h, rate[o], tab), R.y * d, acc[o]);
                 }
                 if (HH) {
-                    const double d = SS ? fma(nc[NY] * sw[k], p64::exp_neg(r2, rate[NY], tab), sq[NY][k]) : sq[NY][k];
-                    acc[NY] = fma(d, ri, acc[NY]);
+                    const double d =
+                        SS ? fma(nc[NY] * sw[k], p64::exp_neg(r2, 0.0f, 0.0f, rate[NY], tab), sq[NY][k]) : sq[NY][k];
+                    acc[NY] = fma(d, R.ri(), acc[NY]);
                 }
             }
         }

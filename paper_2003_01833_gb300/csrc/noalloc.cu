@@ -44,9 +44,9 @@ struct NaRates {
 // partial[(s * nf + o) * n + i] = sum over sources j in slice s, r_ij != 0, of
 //   exp(-k_o r) / r * (f_o[j] - f_o[i]) w_j
 // for the NF fields from o0 on.  Bound by the float64
-// unit: 11 operations a pair and 4 a field (pair64.cuh) instead of 47 a field
+// unit: 9 operations a pair and 4 a field (pair64.cuh) instead of 47 a field
 // with the geometry formed again for each: 12,007 points with two fields take
-// 6.6 ms, 22.3 before.
+// 5.4 ms, 22.3 before.
 template <int NF>
 __global__ void __launch_bounds__(kNaThreads) k_direct_noalloc(const double* __restrict__ xyz,
                                                                const double* __restrict__ w,
@@ -97,12 +97,12 @@ __global__ void __launch_bounds__(kNaThreads) k_direct_noalloc(const double* __r
                 for (int o = 0; o < NF; o++) acc[o] += exp(-k[o] * r) / r * (sf[o][q] - fi[o]) * sw[q];
                 continue;
             }
-            double ri, r;
-            p64::inv_sqrt(r2, ri, r);
-            const double riw = ri * sw[q];
+            const p64::Root R = p64::root(r2);
+            const float h = p64::small32(R.h);
+            const double yw = R.y * sw[q];
 #pragma unroll
             for (int o = 0; o < NF; o++)
-                acc[o] = fma(p64::exp_neg(r, rate[o], tab), riw * (sf[o][q] - fi[o]), acc[o]);
+                acc[o] = fma(p64::exp_neg(R.t, h, h, rate[o], tab), yw * (sf[o][q] - fi[o]), acc[o]);
         }
     }
     if (ok)

@@ -6,10 +6,12 @@
 // and float64 costs as much), against 123 of float32: one float64
 // instruction of a warp takes as long as 70 others.  sqrt, exp and a division
 // from the math library come to 47 such slots a pair with the rest of a
-// Yukawa term.  Here a pair costs 10 for its geometry and 4 a field; the rest
+// Yukawa term.  Here a pair costs 8 for its geometry and 4 a field; the rest
 // is float32 and integer work that hides behind them:
-//   1/r   the float32 approximation of rsqrt corrected once in two-float
-//         arithmetic (to 2^-44) and once in float64 (Newton);
+//   1/r   the float32 approximation of rsqrt corrected in two-float arithmetic
+//         (y, to 2^-44), and its defect h = (1 - r2 y^2) / 2 in float64: 1/r =
+//         y (1 + h) and r = r2 y (1 + h) to 2^-87.  Ten bits of h are enough,
+//         and the factors go into the exponential's float32 part;
 //   2^v   Tang's table-driven exponential (ACM TOMS 15, 1989): v = (n + f)/512,
 //         2^v = 2^(n >> 9) T[n & 511] 2^(f/512), T in float64, the factor's
 //         difference from 1 (below 2^-10) in two-float arithmetic, added to
@@ -68,8 +70,14 @@ __device__ __forceinline__ bool fast_range(double r2)
     return (uint32_t)(__double2hiint(r2) - 0x3B900000) < 0x44500000u - 0x3B900000u;
 }
 
-// ri = 1/sqrt(r2) and r = sqrt(r2), within an ulp
-__device__ __forceinline__ void inv_sqrt(double r2, double& ri, double& r)
+// 1/sqrt(r2) = y (1 + h) and sqrt(r2) = t (1 + h), |h| < 2^-43
+struct Root {
+    double y, t, h;
+    __device__ __forceinline__ double ri() const { return fma(y, h, y); }
+    __device__ __forceinline__ double r() const { return fma(t, h, t); }
+};
+
+__device__ __forceinline__ Root root(double r2)
 {
     const int hi = __double2hiint(r2);
     const uint32_t lo = (uint32_t)__double2loint(r2);
@@ -94,9 +102,23 @@ __device__ __forceinline__ void inv_sqrt(double r2, double& ri, double& r)
     const double y0 = __longlong_as_double(y64);
     const double yhalf = __longlong_as_double(y64 - (1ll << 52));
     const double t = r2 * y0;
-    const double h = fma(-t, yhalf, 0.5);  // (1 - r2 y0^2) / 2, about 2^-45
-    ri = fma(y0, h, y0);
-    r = fma(t, h, t);
+    return Root{y0, t, fma(-t, yhalf, 0.5)};
+}
+
+// 1/r and r within an ulp
+__device__ __forceinline__ void inv_sqrt(double r2, double& ri, double& r)
+{
+    const Root R = root(r2);
+    ri = R.ri();
+    r = R.r();
+}
+
+// a float64 below 2^-40 in size, to float32's precision (zero stays zero)
+__device__ __forceinline__ float small32(double h)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(h), mag = hi & 0x7fffffffu;
+    const uint32_t v = (mag - 0x38000000u) << 3 | (uint32_t)__double2loint(h) >> 29 | (hi & 0x80000000u);
+    return mag < 0x38100000u ? 0.0f : __uint_as_float(v);
 }
 
 // Exponent factor of e^(-k a) = 2^(c a / 512): c = -512 k log2(e) as a
@@ -112,9 +134,9 @@ __device__ __forceinline__ Rate make_rate(double k)
     return Rate{c, (float)(fma(k5, lh, -c) + k5 * ll), (float)c};
 }
 
-// e^(-k a) for a >= 0 in float32's range, to an ulp beside the rounding of a;
-// 0 where it is below 2^-1021
-__device__ __forceinline__ double exp_neg(double a, const Rate& k, const double* __restrict__ tab)
+// e^(-k a (1 + da)) (1 + h) for a >= 0 in float32's range and |da|, |h| < 2^-42,
+// to an ulp beside the rounding of a; 0 where it is below 2^-1021
+__device__ __forceinline__ double exp_neg(double a, float da, float h, const Rate& k, const double* __restrict__ tab)
 {
     const float af = trunc32(__double2hiint(a), (uint32_t)__double2loint(a));
     // n = the integer nearest c a (from the float32 product; never positive)
@@ -128,9 +150,9 @@ __device__ __forceinline__ double exp_neg(double a, const Rate& k, const double*
     const uint32_t ghi = (uint32_t)__double2hiint(g), glo = (uint32_t)__double2loint(g);
     const int fi = (int)(__funnelshift_l(glo, ghi, 12) ^ 0x80000000u);  // f in units of 2^-31, rounded down
     const float fh = __int2float_rn(fi & ~0x7f) * 0x1p-31f;             // 24 bits
-    const float fl =
-        __fmaf_rn(af, k.cl, __uint2float_rn(((uint32_t)fi & 0x7fu) << 20 | (glo & 0xfffffu)) * 0x1p-51f);
-    // P = 2^(f/512) - 1 = f (c1 + f (c2 + f (c3 + f c4))), c_i = (ln 2 / 512)^i / i!
+    const float fl = __fmaf_rn(
+        v, da, __fmaf_rn(af, k.cl, __uint2float_rn(((uint32_t)fi & 0x7fu) << 20 | (glo & 0xfffffu)) * 0x1p-51f));
+    // P - h = 2^(f/512) - 1 = f (c1 + f (c2 + f (c3 + f c4))), c_i = (ln 2 / 512)^i / i!
     constexpr float c1h = 0x1.62e430p-10f, c1l = -0x1.05c610p-38f, c2h = 0x1.ebfbe0p-21f, c2l = -0x1.f4e9c6p-51f,
                     c3 = 0x1.c6b08ep-32f, c4 = 0x1.3b2ab6p-43f;
     const float w = __fmul_rn(fh, __fmaf_rn(fh, c4, c3));
@@ -139,7 +161,7 @@ __device__ __forceinline__ double exp_neg(double a, const Rate& k, const double*
     const float sl = __fmaf_rn(fl, qh, __fmaf_rn(fh, ql, __fmaf_rn(fh, qh, -sh)));
     const float ih = __fadd_rn(c1h, sh), il = __fadd_rn(__fadd_rn(__fsub_rn(c1h, ih), sh), __fadd_rn(sl, c1l));
     const float ph = __fmul_rn(fh, ih);
-    const float pl = __fmaf_rn(fl, ih, __fmaf_rn(fh, il, __fmaf_rn(fh, ih, -ph)));
+    const float pl = __fadd_rn(h, __fmaf_rn(fl, ih, __fmaf_rn(fh, il, __fmaf_rn(fh, ih, -ph))));
     // G = T P, |G| < 2^-9, added to T as an integer in units of 2^-52
     const double T = tab[n & (kTab - 1)];
     const int thi = __double2hiint(T);
