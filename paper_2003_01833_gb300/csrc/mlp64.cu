@@ -35,7 +35,7 @@
 // weight gradients, whose K are the points; W2 likewise serves Z2 and dH1.
 // That takes 100 KB, so two CTAs share an SM and one computes while the other
 // waits.  With transposed copies stored value by value (160 KB, one CTA of 512
-// threads) a training step over 10.9M points took 4.63 ms, now 1.77 (131 and 50
+// threads) a training step over 10.9M points took 4.63 ms, now 1.73 (131 and 49
 // SM clocks a point), the same bits.
 //
 // The float32 sums in TMEM are those of one CTA per SM: virtual CTA v owns
@@ -98,9 +98,23 @@ __device__ __forceinline__ void store_row(uint8_t* tile, int r, int c0, const fl
                        bf16x2(v[c + 6], v[c + 7]));
 }
 
-struct Bias {
+struct __align__(16) Bias {
     float b1[kH], b2[kH], w3[kH], b3;
 };
+
+// 16 consecutive values from shared memory, four a load (all lanes of a warp
+// read the same ones; one by one they were a tenth of a tile's instructions)
+__device__ __forceinline__ void load16(const float* p, float (&v)[16])
+{
+#pragma unroll
+    for (int c = 0; c < 16; c += 4) {
+        const float4 t = *reinterpret_cast<const float4*>(p + c);
+        v[c] = t.x;
+        v[c + 1] = t.y;
+        v[c + 2] = t.z;
+        v[c + 3] = t.w;
+    }
+}
 
 // MMAs of one stage, issued by thread 0, then all threads wait for them
 struct Sync {
@@ -163,10 +177,11 @@ __device__ __forceinline__ void activate(const Who& w, const float* b, float (&h
 {
 #pragma unroll
     for (int c = 0; c < kCB; c += 16) {
-        float v[16];
+        float v[16], bc[16];
+        load16(b + w.c0 + c, bc);
         tc::tmem_ld16(w.lane_base + cZ + w.c0 + c, v);
 #pragma unroll
-        for (int i = 0; i < 16; i++) h[c + i] = tanhf(v[i] + b[w.c0 + c + i]);
+        for (int i = 0; i < 16; i++) h[c + i] = tanhf(v[i] + bc[i]);
     }
 }
 
@@ -202,9 +217,10 @@ __device__ float forward_tile(uint8_t* sm, const Bias& B, uint4 xv, const Who& w
     activate(w, B.b2, h2);
 #pragma unroll
     for (int c = 0; c < kCB; c += 16) {
-        float yp = 0.0f;
+        float yp = 0.0f, w3[16];
+        load16(B.w3 + w.c0 + c, w3);
 #pragma unroll
-        for (int i = 0; i < 16; i++) yp = fmaf(B.w3[w.c0 + c + i], h2[c + i], yp);
+        for (int i = 0; i < 16; i++) yp = fmaf(w3[i], h2[c + i], yp);
         ypart[(w.c0 + c) / 16 * kT + w.pl] = yp;
     }
     tc::fence_before_sync();
@@ -367,7 +383,12 @@ __global__ void __launch_bounds__(kThreads, 2) k_mlp64_grad(const uint16_t* __re
         // h2 and dz2 = dy W3 (1 - h2^2)
         store_row<kCB>(sm + sH2, w.pl, w.c0, h2);
 #pragma unroll
-        for (int j = 0; j < kCB; j++) h2[j] = dy * B.w3[w.c0 + j] * (1.0f - h2[j] * h2[j]);
+        for (int c = 0; c < kCB; c += 16) {
+            float w3[16];
+            load16(B.w3 + w.c0 + c, w3);
+#pragma unroll
+            for (int i = 0; i < 16; i++) h2[c + i] = dy * w3[i] * (1.0f - h2[c + i] * h2[c + i]);
+        }
         store_row<kCB>(sm + sDZ2, w.pl, w.c0, h2);
         if (w.g == 0)
             st16(sm, sB2 + (w.pl >> 6) * 16 * 128 + swz2(0, w.pl & 63), (uint16_t)(bf16x2(dy, 0.0f) & 0xFFFFu));
