@@ -234,7 +234,10 @@ __device__ void prefix8(const int64_t* off, const signed char* code, int64_t nbl
     const int64_t blk = x / kBlk;
     int cnt[8] = {0, 0, 0, 0, 0, 0, 0, 0};
     // four codes a load; bytes at or beyond x do not count
-    for (int64_t q = blk * kBlk + 4 * lane; q < x; q += 128) {
+#pragma unroll
+    for (int i = 0; i < kBlk / 128; i++) {
+        const int64_t q = blk * kBlk + 4 * lane + 128 * i;
+        if (q >= x) continue;
         unsigned w = *reinterpret_cast<const unsigned*>(code + q);
         if (x - q < 4) w |= 0xffffffffu << (8 * (int)(x - q));
 #pragma unroll
@@ -857,16 +860,15 @@ __global__ void k_check_finite(const double* a, int64_t n, int* bad)
 
 inline int nblocks(int64_t n, int t) { return (int)((n + t - 1) / t); }
 
-// Pinned host words for values read back, once per host thread.
+// Pinned host words for values read back, once per host thread; the device
+// writes them itself (pinned memory is mapped), so there is no copy to wait for.
 struct Host1 {
     int64_t* h = nullptr;
-    DevBuf dev;
     Host1()
     {
         thread_local int64_t* buf = nullptr;
         if (!buf) TAGI_CUDA(cudaMallocHost(&buf, kReadMax * sizeof(int64_t)));
         h = buf;
-        dev.ensure(kReadMax * sizeof(int64_t));
     }
     // the values at the given device addresses into h[0], h[1], ...
     void read(cudaStream_t s, std::initializer_list<const int64_t*> p64, std::initializer_list<const int*> p32 = {})
@@ -874,9 +876,8 @@ struct Host1 {
         ReadList L{};
         for (const int64_t* p : p64) L.p64[L.n++] = p;
         for (const int* p : p32) L.p32[L.n++] = p;
-        launch(k_collect, 1, 32, 0, s, L, dev.as<int64_t>());
+        launch(k_collect, 1, 32, 0, s, L, h);
         TAGI_LAUNCH_CHECK();
-        TAGI_CUDA(cudaMemcpyAsync(h, dev.p, L.n * sizeof(int64_t), cudaMemcpyDeviceToHost, s));
         TAGI_CUDA(cudaStreamSynchronize(s));
     }
 };
