@@ -919,7 +919,6 @@ void anterpolate_fields32(Tree& T, int nf)
     if (T.nfar == 0) return;
     cudaStream_t s = T.stream;
     const int tpi = T.ant_chunk / kTcK;
-    fill_charge_tiles(T, T.nant, T.ant_items.as<AntItem>(), tpi, T.qant.as<float>(), nf, T.n, T.qtiles);
     for (int g0 = 0; g0 < nf; g0 += 8) {
         int g = nf - g0 < 8 ? nf - g0 : 8;
         T.antpart.ensure(sizeof(double) * (size_t)T.nant * T.P * g);

@@ -121,16 +121,16 @@ void run_convolution(Tree& T, const double* f, const RateSrc& R, const double* e
 {
     const int nf = R.nf;
     ensure_part(T, nf);
-    make_rates(T, R, eps_dev);
     if (T.prec == TAGI_FP32C) {
         {
             ProfScope ps(kProfAnterp, T.stream);
-            prepare_points32(T, f, nf);
+            prepare32(T, f, R, eps_dev);
             anterpolate_fields32(T, nf);
         }
         ProfScope ps(kProfInteract, T.stream);
         interact32(T, nf, R.kind, T.rates32.as<float>(), T.part.as<double>(), T.tsum.as<double>(), T.tc_cnt.as<int>());
     } else {
+        make_rates(T, R, eps_dev);
         {
             ProfScope ps(kProfAnterp, T.stream);
             prepare_points64(T, f, nf);

@@ -6,6 +6,7 @@
 // so results are bitwise reproducible run to run.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
@@ -21,20 +22,83 @@ constexpr double kPi = 3.14159265358979323846;
 
 inline int nblocks(int64_t n, int t) { return (int)((n + t - 1) / t); }
 
-// Two-float split of each field value, f = fh + fl, and the rounded charge
-// f w for the anterpolation.
-__global__ void k_prepare32(const double* __restrict__ f, int nf, int64_t n, const int* __restrict__ perm,
-                            const double* __restrict__ pw, float* fa, int64_t lda, float* fb, float* qa)
+// Decay rates of one call, on the device: kyd[o] = fl32(-k_o log2 e) for
+// Yukawa fields and fl32(-log2 e / alpha^2) for the Coulomb field (the
+// float32 kernel's exponent factors); kvd[o] = the k or alpha the kernel
+// therefore applies (FP32C) or the exact one (FP64).  The first n_eps fields
+// take k = sqrt(-2 (eps_o + vshift)) from device eigenvalues; a
+// non-positive eps + vshift sets *err.
+__device__ __forceinline__ void field_rate(const RateSrc& R, int o, const double* __restrict__ eps_dev, float* kyd,
+                                           double* kvd, int* err)
 {
-    int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    if (i >= n * nf) return;
-    int64_t o = i / n, p = i % n;
-    double v = f[o * n + perm[p]];
-    float h = (float)v;
-    fa[o * lda + p] = h;
-    fb[o * n + p] = (float)(v - (double)h);
-    qa[o * n + p] = (float)(v * pw[p]);
+    const double L2E = 1.4426950408889634;
+    double v;
+    if (o < R.n_eps) {
+        const double es = eps_dev[o] + R.vshift;
+        if (!(es < 0.0)) atomicOr(err, 1);
+        v = sqrt(-2.0 * es);
+    } else {
+        v = R.val[o];
+    }
+    if (R.kind[o] == 0) {
+        const float ky = (float)(-v * L2E);
+        kyd[o] = ky;
+        kvd[o] = R.fp32 ? -(double)ky / L2E : v;
+    } else {
+        const float ga = (float)(-L2E / (v * v));
+        kyd[o] = ga;
+        kvd[o] = R.fp32 ? sqrt(-L2E / (double)ga) : v;
+    }
 }
+
+__global__ void k_make_rates(const __grid_constant__ RateSrc R, const double* __restrict__ eps_dev, float* kyd,
+                             double* kvd, int* err)
+{
+    const int o = threadIdx.x;
+    if (o < R.nf) field_rate(R, o, eps_dev, kyd, kvd, err);
+}
+
+// What the FP32C kernels need of a call's fields, in one launch (three small
+// kernels in a row cost a small tree 6 of its 80 us):
+//   blocks [0, pblk): the two-float split f = fh + fl of each field value, in
+//     tree order;
+//   blocks [pblk, gridDim.x - 1): the charges fl32(f w) in the tiles of the
+//     anterpolation, qT[(item * tpi + tile) * nf + o][32] (zero beyond the
+//     item's end);
+//   the last block: the rates.
+constexpr int kPrepThreads = 256;
+__global__ void __launch_bounds__(kPrepThreads) k_prepare32(const __grid_constant__ RateSrc R,
+                                                            const double* __restrict__ eps_dev, float* kyd,
+                                                            double* kvd, int* err, const double* __restrict__ f,
+                                                            int64_t n, const int* __restrict__ perm,
+                                                            const double* __restrict__ pw, float* fa, int64_t lda,
+                                                            float* fb, unsigned pblk,
+                                                            const AntItem* __restrict__ items, int64_t ncharge,
+                                                            int tpi, float* qT)
+{
+    if (blockIdx.x == gridDim.x - 1) {
+        if ((int)threadIdx.x < R.nf) field_rate(R, threadIdx.x, eps_dev, kyd, kvd, err);
+    } else if (blockIdx.x < pblk) {
+        const int64_t i = blockIdx.x * (int64_t)kPrepThreads + threadIdx.x;
+        if (i >= n * R.nf) return;
+        const int64_t o = i / n, p = i % n;
+        const double v = f[o * n + perm[p]];
+        const float h = (float)v;
+        fa[o * lda + p] = h;
+        fb[o * n + p] = (float)(v - (double)h);
+    } else {
+        const int64_t e = (blockIdx.x - pblk) * (int64_t)kPrepThreads + threadIdx.x;
+        if (e >= ncharge) return;
+        const int jj = (int)(e & 31);
+        const int64_t rest = e >> 5;
+        const int o = (int)(rest % R.nf);
+        const int64_t tile = rest / R.nf;
+        const AntItem it = items[tile / tpi];
+        const int p = it.p0 + (int)(tile % tpi) * 32 + jj;
+        qT[e] = p < it.p1 ? (float)(f[o * n + perm[p]] * pw[p]) : 0.0f;
+    }
+}
+static_assert(kMaxCallFields <= kPrepThreads, "one thread per rate");
 
 __global__ void k_prepare64(const double* __restrict__ f, int nf, int64_t n, const int* __restrict__ perm,
                             const double* __restrict__ pw, double* q, int64_t ldq, double* c)
@@ -172,14 +236,21 @@ void weighted_dots(Tree& T, const std::vector<DotJob>& jobs, double* out_dev)
     }
 }
 
-void prepare_points32(Tree& T, const double* f, int nf)
+void prepare32(Tree& T, const double* f, const RateSrc& R, const double* eps_dev)
 {
+    const int nf = R.nf;
+    T.rates32.ensure(sizeof(float) * kMaxCallFields);
+    T.rates64.ensure(sizeof(double) * kMaxCallFields);
     T.fa.ensure(sizeof(float) * (size_t)nf * T.nrec);
     T.fb.ensure(sizeof(float) * (size_t)nf * T.n);
-    T.qant.ensure(sizeof(float) * (size_t)nf * T.n);
-    launch(k_prepare32, nblocks(T.n * nf, 256), 256, 0, T.stream, f, nf, T.n, T.perm.as<int>(), T.pw.as<double>(),
-                                                             T.fa.as<float>(), T.nrec, T.fb.as<float>(),
-                                                             T.qant.as<float>());
+    const int tpi = T.ant_chunk / 32;
+    const int64_t charges = T.nfar > 0 ? T.nant * tpi * 32 * nf : 0;
+    T.qtiles.ensure(sizeof(float) * (size_t)std::max<int64_t>(charges, 1));
+    const unsigned pblk = nblocks(T.n * nf, kPrepThreads);
+    launch(k_prepare32, pblk + (unsigned)nblocks(charges, kPrepThreads) + 1, kPrepThreads, 0, T.stream, R, eps_dev,
+           T.rates32.as<float>(), T.rates64.as<double>(), T.errflag.as<int>(), f, T.n, T.perm.as<int>(),
+           T.pw.as<double>(), T.fa.as<float>(), T.nrec, T.fb.as<float>(), pblk, T.ant_items.as<AntItem>(), charges, tpi,
+           T.qtiles.as<float>());
     TAGI_LAUNCH_CHECK();
 }
 
@@ -190,36 +261,6 @@ void prepare_points64(Tree& T, const double* f, int nf)
     launch(k_prepare64, nblocks(T.n * nf, 256), 256, 0, T.stream, f, nf, T.n, T.perm.as<int>(), T.pw.as<double>(),
                                                              T.q64.as<double>(), T.nrec, T.c64.as<double>());
     TAGI_LAUNCH_CHECK();
-}
-
-// Decay rates of one call, on the device: kyd[o] = fl32(-k_o log2 e) for
-// Yukawa fields and fl32(-log2 e / alpha^2) for the Coulomb field (the
-// float32 kernel's exponent factors); kvd[o] = the k or alpha the kernel
-// therefore applies (FP32C) or the exact one (FP64).  The first n_eps fields
-// take k = sqrt(-2 (eps_o + vshift)) from device eigenvalues; a
-// non-positive eps + vshift sets *err.
-__global__ void k_make_rates(RateSrc R, const double* __restrict__ eps_dev, float* kyd, double* kvd, int* err)
-{
-    const int o = threadIdx.x + blockIdx.x * blockDim.x;
-    if (o >= R.nf) return;
-    const double L2E = 1.4426950408889634;
-    double v;
-    if (o < R.n_eps) {
-        const double es = eps_dev[o] + R.vshift;
-        if (!(es < 0.0)) atomicOr(err, 1);
-        v = sqrt(-2.0 * es);
-    } else {
-        v = R.val[o];
-    }
-    if (R.kind[o] == 0) {
-        const float ky = (float)(-v * L2E);
-        kyd[o] = ky;
-        kvd[o] = R.fp32 ? -(double)ky / L2E : v;
-    } else {
-        const float ga = (float)(-L2E / (v * v));
-        kyd[o] = ga;
-        kvd[o] = R.fp32 ? sqrt(-L2E / (double)ga) : v;
-    }
 }
 
 void make_rates(Tree& T, const RateSrc& R, const double* eps_dev)

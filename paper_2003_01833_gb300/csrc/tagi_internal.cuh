@@ -194,7 +194,6 @@ struct Tree {
     // per-call work buffers
     DevBuf fa;          // float [nf][nrec]: fh = f rounded (points), qh (proxies)
     DevBuf fb;          // float [nf][n]: fl = f - fh (points)
-    DevBuf qant;        // float [nf][n]: f w rounded, the anterpolation input
     DevBuf q64;         // double [nf][nrec]
     DevBuf c64;         // double [nf][n] field values in tree order (FP64 SS constants)
     DevBuf wc;          // double [n] quadrature weights in the caller's order
@@ -220,7 +219,7 @@ struct Tree {
 void build_tree(Tree& T, const double* xyz, const double* w);
 // anterp.cu
 void anterpolate_weights(Tree& T);  // w^ for every approximated cluster (FP32C and FP64)
-void anterpolate_fields32(Tree& T, int nf);  // q^ rows [0, nf) of T.fa from T.qant
+void anterpolate_fields32(Tree& T, int nf);  // q^ rows [0, nf) of T.fa from T.qtiles
 void anterpolate_fields64(Tree& T, int nf);
 void anterpolate_all_clusters64(Tree& T, const double* q, int nq, double* qh);
 void anterpolate_all_clusters32(Tree& T, const double* q, int nq, double* qh);  // FP32C form (tensor cores)
@@ -233,7 +232,8 @@ void fp32_bias(cudaStream_t s, double* beta_y, double* beta_g);
 double effective_k32(double k);
 double effective_alpha32(double a);
 // green.cu
-void prepare_points32(Tree& T, const double* f, int nf);   // fa, fb, qant from caller-order fields
+// FP32C: rates, fa, fb and the anterpolation's charge tiles of a call's R.nf caller-order fields
+void prepare32(Tree& T, const double* f, const RateSrc& R, const double* eps_dev);
 void prepare_points64(Tree& T, const double* f, int nf);   // q64 from caller-order fields
 // rates of a call into T.rates32 / T.rates64 (see RateSrc)
 void make_rates(Tree& T, const RateSrc& R, const double* eps_dev);
