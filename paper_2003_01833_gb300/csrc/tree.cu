@@ -377,7 +377,7 @@ __global__ void k_far_flags(int nc, const int* is_far, const int* begin, const i
     size[c] = is_far[c] ? end[c] - begin[c] : 0;
 }
 
-// Values that the host reads together: one copy and one wait for all of them.
+// Values that the host reads together: one launch and one wait for all of them.
 constexpr int kReadMax = 8;
 struct ReadList {
     const int64_t* p64[kReadMax];
