@@ -129,6 +129,15 @@ struct Sync {
     }
 };
 
+// After a wait that gave up, thread 0: flag it, and wait (bounded) for every
+// MMA it has issued, whichever commits they belong to
+__device__ __noinline__ void give_up(uint64_t* drained, int* err)
+{
+    atomicOr(err, 1);
+    tc::commit(drained);
+    tc::mbar_wait(drained, 0, kWait);
+}
+
 // A and B K-major, `ksteps` K-steps of 16 from the start of a row
 __device__ __forceinline__ void mma_chain(uint32_t d, uint32_t a, uint32_t b, int ksteps, uint32_t idesc)
 {
@@ -185,18 +194,20 @@ __device__ __forceinline__ void activate(const Who& w, const float* b, float (&h
     }
 }
 
-// Forward pass of point pl of the tile whose features xv (warpgroup 0) holds;
-// returns y, false in sy.ok if a wait of any thread gave up.  h1, h2: this
-// thread's activations (float32).  ypart: [4][kT] shared partial sums of
-// W3 . h2 over 16 units each, added in unit order.
-__device__ float forward_tile(uint8_t* sm, const Bias& B, uint4 xv, const Who& w, uint32_t tmem, Sync& sy,
-                              float* ypart, float (&h1)[kCB], float (&h2)[kCB])
+// Forward pass of point pl of the tile whose features xv (warpgroup 0) holds:
+// y.  Returns false, in all threads, if a wait of any thread gave up before this
+// tile; callers leave their loops on that alone, since sy.ok, the thread's own,
+// may differ between threads from the tile's first wait on.  h1, h2: this
+// thread's activations (float32).  ypart: [4][kT] shared partial sums of W3 . h2
+// over 16 units each, added in unit order.
+__device__ bool forward_tile(uint8_t* sm, const Bias& B, uint4 xv, const Who& w, uint32_t tmem, Sync& sy,
+                             float* ypart, float (&h1)[kCB], float (&h2)[kCB], float& y)
 {
     if (w.g == 0) *reinterpret_cast<uint4*>(sm + sX + swz2(w.pl, 0)) = xv;
     tc::fence_async_smem();
     tc::fence_before_sync();
     sy.ok = __syncthreads_and(sy.ok);
-    if (!sy.ok) return 0.0f;
+    if (!sy.ok) return false;
     if (w.t == 0) {
         tc::fence_after_sync();
         mma_chain(tmem + cZ, tc::smem_u32(sm + sX), tc::smem_u32(sm + sW1), 1, tc::idesc_bf16(128, 64));
@@ -225,10 +236,10 @@ __device__ float forward_tile(uint8_t* sm, const Bias& B, uint4 xv, const Who& w
     }
     tc::fence_before_sync();
     __syncthreads();
-    float y = B.b3;
+    y = B.b3;
 #pragma unroll
     for (int q = 0; q < 4; q++) y += ypart[q * kT + w.pl];
-    return y;
+    return true;
 }
 
 // features of point p (zeros beyond n)
@@ -249,13 +260,16 @@ __global__ void __launch_bounds__(kThreads, 2) k_mlp64_fwd(const uint16_t* __res
     uint8_t* sm =
         reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023)) - sFwd;
     __shared__ Bias B;
-    __shared__ uint64_t bar;
+    __shared__ uint64_t bar, drained;
     __shared__ uint32_t slot;
     __shared__ float ypart[4 * kT];
     const int t = threadIdx.x;
     setup(sm, sFwd, &B, master);
     if ((t >> 5) == 0) tc::tmem_alloc(&slot, kColsFwd);
-    if (t == 0) tc::mbar_init(&bar, 1);
+    if (t == 0) {
+        tc::mbar_init(&bar, 1);
+        tc::mbar_init(&drained, 1);
+    }
     tc::fence_async_smem();
     tc::fence_before_sync();
     __syncthreads();
@@ -270,15 +284,11 @@ __global__ void __launch_bounds__(kThreads, 2) k_mlp64_fwd(const uint16_t* __res
         const int64_t p = tile * kT + w.pl;
         const uint4 xv = next;
         if (w.g == 0) next = load_features(feat, p + (int64_t)gridDim.x * kT, n);
-        float h1[kCB], h2[kCB];
-        const float out = forward_tile(sm, B, xv, w, tmem, sy, ypart, h1, h2);
-        if (!sy.ok) break;
+        float h1[kCB], h2[kCB], out;
+        if (!forward_tile(sm, B, xv, w, tmem, sy, ypart, h1, h2, out)) break;
         if (w.g == 0 && p < n) y[p] = out;
     }
-    if (!__syncthreads_and(sy.ok) && t == 0) {
-        atomicOr(err, 1);
-        tc::mbar_wait(&bar, sy.phase ^ 1, kWait);  // the MMAs of the last commit, bounded
-    }
+    if (!__syncthreads_and(sy.ok) && t == 0) give_up(&drained, err);
     tc::fence_before_sync();
     __syncthreads();
     if ((t >> 5) == 0) {
@@ -299,7 +309,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_mlp64_grad(const uint16_t* __re
     extern __shared__ uint8_t raw[];
     uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(raw) + 1023) & ~uintptr_t(1023));
     __shared__ Bias B;
-    __shared__ uint64_t bar;
+    __shared__ uint64_t bar, drained;
     __shared__ uint32_t slot;
     __shared__ float ypart[4 * kT];
     __shared__ double lsum[kT];
@@ -308,7 +318,10 @@ __global__ void __launch_bounds__(kThreads, 2) k_mlp64_grad(const uint16_t* __re
     for (int e = t; e <= kParams; e += kThreads) out[e] = 0.0;
     setup(sm, 0, &B, master);
     if ((t >> 5) == 0) tc::tmem_alloc(&slot, kColsGrad);
-    if (t == 0) tc::mbar_init(&bar, 1);
+    if (t == 0) {
+        tc::mbar_init(&bar, 1);
+        tc::mbar_init(&drained, 1);
+    }
     tc::fence_async_smem();
     tc::fence_before_sync();
     __syncthreads();
@@ -374,9 +387,8 @@ __global__ void __launch_bounds__(kThreads, 2) k_mlp64_grad(const uint16_t* __re
         const float tv = nt, wv = nw;
         const int64_t knext = after(k);
         load(knext);
-        float h1[kCB], h2[kCB];
-        const float yv = forward_tile(sm, B, xv, w, tmem, sy, ypart, h1, h2);
-        if (!sy.ok) break;
+        float h1[kCB], h2[kCB], yv;
+        if (!forward_tile(sm, B, xv, w, tmem, sy, ypart, h1, h2, yv)) break;
         const float r = p < n ? yv - tv : 0.0f;
         if (w.g == 0) loss += (double)wv * (double)r * (double)r;
         const float dy = 2.0f * wv * r;
@@ -443,10 +455,7 @@ __global__ void __launch_bounds__(kThreads, 2) k_mlp64_grad(const uint16_t* __re
     }
     if (w.g == 0) lsum[w.pl] = loss;
     const bool ok = __syncthreads_and(sy.ok);
-    if (!ok && t == 0) {
-        atomicOr(err, 1);
-        tc::mbar_wait(&bar, sy.phase ^ 1, kWait);  // the MMAs of the last commit, bounded
-    }
+    if (!ok && t == 0) give_up(&drained, err);
     if (ok && t == 0) {
         double s = 0.0;
         for (int q = 0; q < kT; q++) s += lsum[q];
