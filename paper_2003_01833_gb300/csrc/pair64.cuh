@@ -10,8 +10,9 @@
 // is float32 and integer work that hides behind them:
 //   1/r   the float32 approximation of rsqrt corrected in two-float arithmetic
 //         (y, to 2^-44), and its defect h = (1 - r2 y^2) / 2 in float64: 1/r =
-//         y (1 + h) and r = r2 y (1 + h) to 2^-87.  Ten bits of h are enough,
-//         and the factors go into the exponential's float32 part;
+//         y (1 + h) and r = r2 y (1 + h).  The series ends at 2^-86; the rounding
+//         of r2 y leaves 2^-54 in h.  Ten bits of h are enough in the
+//         exponential, and the factors go into its float32 part;
 //   2^v   Tang's table-driven exponential (ACM TOMS 15, 1989): v = (n + f)/512,
 //         2^v = 2^(n >> 9) T[n & 511] 2^(f/512), T in float64, the factor's
 //         difference from 1 (below 2^-10) in two-float arithmetic, added to
@@ -93,12 +94,17 @@ __device__ __forceinline__ Root root(double r2)
     e = __fmaf_rn(-rh, pe, e);
     e = __fmaf_rn(-rl, p, e);
     const float yl = __fmul_rn(y, __fmul_rn(e, __fmaf_rn(0.375f, e, 0.5f)));
-    // y + yl as a float64: yl in units of the last place of y's mantissa, half
-    // as large where y is a power of two and yl is negative
+    // y + yl as a float64: yl in units of the last place of y's mantissa.  Where
+    // that passes a power of two (the approximation may lie on either side of
+    // one), the units beyond it are half, or twice, as large
     const uint32_t yb = __float_as_uint(y);
-    int q = __float2int_rn(yl * __uint_as_float((306u << 23) - (yb & 0x7f800000u)));
-    if ((yb & 0x7fffffu) == 0 && q < 0) q += q;
-    const int64_t y64 = ((int64_t)((yb >> 3) + 0x38000000u) << 32 | (uint32_t)(yb << 29)) + q;
+    const int q = __float2int_rn(yl * __uint_as_float((306u << 23) - (yb & 0x7f800000u)));
+    const int64_t base = (int64_t)((yb >> 3) + 0x38000000u) << 32 | (uint32_t)(yb << 29);
+    int64_t y64 = base + q;
+    if (((uint32_t)(y64 >> 32) ^ (uint32_t)(base >> 32)) >> 20) {
+        constexpr int64_t mantissa = (1ll << 52) - 1;
+        y64 += q < 0 ? y64 - (base & ~mantissa) : -((y64 & mantissa) >> 1);
+    }
     const double y0 = __longlong_as_double(y64);
     const double yhalf = __longlong_as_double(y64 - (1ll << 52));
     const double t = r2 * y0;

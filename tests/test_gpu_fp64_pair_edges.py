@@ -1,0 +1,57 @@
+"""Single pairs of the float64 forms, one source seen by every target, where the
+reciprocal root's approximation may lie on the other side of a power of two.
+Against float64 and extended arithmetic on the host.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def T():
+    import __graft_entry__ as g
+
+    g.build()
+    import paper_2003_01833_gb300.tagi as T
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return T
+
+
+def dev(a):
+    return torch.tensor(np.ascontiguousarray(a), dtype=torch.float64, device="cuda")
+
+
+def pair_values(T, r, k, weight):
+    """4 pi times the field that a source of value 1 and quadrature weight
+    `weight` at the origin makes at distances r along x, where nothing else has
+    a weight: by the direct sum and by the tree form with and without subtraction."""
+    n = len(r) + 1
+    xyz = np.zeros((3, n))
+    xyz[0, 1:] = r
+    w, f = np.zeros(n), np.zeros((1, n))
+    w[0], f[0, 0] = weight, 1.0
+    u = torch.empty((1, n), dtype=torch.float64, device="cuda")
+    T.tagi_yukawa_direct_noalloc(dev(xyz), dev(w), dev(f), [k], u)
+    yield u.cpu().numpy()[0, 1:] * 4 * np.pi
+    for ss in (True, False):
+        with T.Tree(dev(xyz), dev(w), theta=0.0, degree=2, leaf_size=n, prec=T.TAGI_FP64, ss=ss) as tr:
+            T.tagi_yukawa_conv(tr.handle, dev(f), [k], u)
+        yield u.cpu().numpy()[0, 1:] * 4 * np.pi
+
+
+def test_distances_next_to_powers_of_two(T):
+    """32 float32 values of r^2 on each side of every power of four in the fast
+    range.  Units of 2^-52: an ulp of the exponential, half of the final product
+    and of k r (here below 2^-5), three roundings of the factor 4 pi and its
+    quotient here."""
+    p = np.arange(-34, 35)
+    r2 = np.concatenate([(np.float32(4.0) ** p.astype(np.float32)).view(np.int32) + j for j in range(-32, 33)])
+    r = np.sqrt(np.unique(r2).astype(np.int32).view(np.float32).astype(np.float64))
+    k = 2.0 ** -40
+    exact = np.exp(-k * r.astype(np.longdouble)) / r
+    for got in pair_values(T, r, k, 1.0):
+        assert np.max(np.abs(got / exact - 1)) <= 5 * 2.0 ** -52
