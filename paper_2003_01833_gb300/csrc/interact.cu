@@ -771,13 +771,24 @@ __global__ void k_calibrate(int mode, long long n, double* out)
 // library's (0.62 / 0.73 against 0.75 / 0.96 units of 2^-52 (1 + k r)).
 constexpr int kMax64 = 4;
 
-// a pair that the fast forms do not take (r = 0 is skipped, Eq. direct-sum)
-__device__ __noinline__ double pair_slow(double r2, double k, double q, double nc, double w, bool coulomb, bool ss)
+// A pair that the loop does not take: acc with the field's term added.  r = 0 is
+// skipped (Eq. direct-sum).  Inside the fast range the loop's own operations,
+// with the exponential's subnormal values.
+__device__ __noinline__ double pair_slow(double acc, double r2, double k, double q, double nc, double w, bool coulomb,
+                                         bool ss, const double* __restrict__ tab)
 {
-    if (r2 == 0.0) return 0.0;
+    if (r2 == 0.0) return acc;
+    if (p64::fast_range(r2)) {
+        const p64::Root R = p64::root(r2);
+        const p64::Rate rate = p64::make_rate(k);
+        if (coulomb)
+            return fma(ss ? fma(nc * w, p64::exp_neg<true>(r2, 0.0f, 0.0f, rate, tab), q) : q, R.ri(), acc);
+        const float h = p64::small32(R.h);
+        return fma(p64::exp_neg<true>(R.t, h, h, rate, tab), R.y * (ss ? fma(nc, w, q) : q), acc);
+    }
     const double r = sqrt(r2);
-    if (!coulomb) return exp(-k * r) / r * (ss ? fma(nc, w, q) : q);
-    return (ss ? fma(nc * w, exp(-r2 * k), q) : q) / r;
+    if (!coulomb) return acc + exp(-k * r) / r * (ss ? fma(nc, w, q) : q);
+    return acc + (ss ? fma(nc * w, exp(-r2 * k), q) : q) / r;
 }
 
 template <int NY, bool HH, bool SS>
@@ -833,10 +844,13 @@ __global__ void __launch_bounds__(kThreads64) k_interact64(const Item* __restric
             for (int k = 0; k < ns; k++) {
                 const double dx = x - sx[k], dy = y - sy[k], dz = z - sz[k];
                 const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-                if (!p64::fast_range(r2)) {
+                bool slow = !p64::fast_range(r2);
+#pragma unroll
+                for (int o = 0; o < NY; o++) slow |= p64::subnormal(r2, rate[o]);
+                if (slow) {
 #pragma unroll
                     for (int o = 0; o < NF; o++)
-                        acc[o] += pair_slow(r2, kv[o], sq[o][k], nc[o], sw[k], o >= NY, SS);
+                        acc[o] = pair_slow(acc[o], r2, kv[o], sq[o][k], nc[o], sw[k], o >= NY, SS, tab);
                     continue;
                 }
                 const p64::Root R = p64::root(r2);
@@ -844,11 +858,11 @@ __global__ void __launch_bounds__(kThreads64) k_interact64(const Item* __restric
 #pragma unroll
                 for (int o = 0; o < NY; o++) {
                     const double d = SS ? fma(nc[o], sw[k], sq[o][k]) : sq[o][k];
-                    acc[o] = fma(p64::exp_neg(R.t, h, h, rate[o], tab), R.y * d, acc[o]);
+                    acc[o] = fma(p64::exp_neg<false>(R.t, h, h, rate[o], tab), R.y * d, acc[o]);
                 }
                 if (HH) {
                     const double d =
-                        SS ? fma(nc[NY] * sw[k], p64::exp_neg(r2, 0.0f, 0.0f, rate[NY], tab), sq[NY][k]) : sq[NY][k];
+                        SS ? fma(nc[NY] * sw[k], p64::exp_neg<true>(r2, 0.0f, 0.0f, rate[NY], tab), sq[NY][k]) : sq[NY][k];
                     acc[NY] = fma(d, R.ri(), acc[NY]);
                 }
             }

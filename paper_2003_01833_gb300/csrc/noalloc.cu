@@ -41,6 +41,22 @@ struct NaRates {
     double k[kNaMaxFields];
 };
 
+// A pair that the loop does not take: acc with the field's term added.  r = 0 is
+// skipped (the singular r' = r term).  Inside the fast range the loop's own
+// operations, with the exponential's subnormal values.
+__device__ __noinline__ double pair_slow(double acc, double r2, double k, double d, double w,
+                                         const double* __restrict__ tab)
+{
+    if (r2 == 0.0) return acc;
+    if (p64::fast_range(r2)) {
+        const p64::Root R = p64::root(r2);
+        const float h = p64::small32(R.h);
+        return fma(p64::exp_neg<true>(R.t, h, h, p64::make_rate(k), tab), R.y * w * d, acc);
+    }
+    const double r = sqrt(r2);
+    return acc + exp(-k * r) / r * d * w;
+}
+
 // partial[(s * nf + o) * n + i] = sum over sources j in slice s, r_ij != 0, of
 //   exp(-k_o r) / r * (f_o[j] - f_o[i]) w_j
 // for the NF fields from o0 on.  Bound by the float64
@@ -90,11 +106,12 @@ __global__ void __launch_bounds__(kNaThreads) k_direct_noalloc(const double* __r
         for (int q = 0; q < nt; q++) {
             const double dx = x - sx[q], dy = y - sy[q], dz = z - sz[q];
             const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-            if (!p64::fast_range(r2)) {
-                if (r2 == 0.0) continue;  // the singular r' = r term is skipped
-                const double r = sqrt(r2);
+            bool slow = !p64::fast_range(r2);
 #pragma unroll
-                for (int o = 0; o < NF; o++) acc[o] += exp(-k[o] * r) / r * (sf[o][q] - fi[o]) * sw[q];
+            for (int o = 0; o < NF; o++) slow |= p64::subnormal(r2, rate[o]);
+            if (slow) {
+#pragma unroll
+                for (int o = 0; o < NF; o++) acc[o] = pair_slow(acc[o], r2, k[o], sf[o][q] - fi[o], sw[q], tab);
                 continue;
             }
             const p64::Root R = p64::root(r2);
@@ -102,7 +119,7 @@ __global__ void __launch_bounds__(kNaThreads) k_direct_noalloc(const double* __r
             const double yw = R.y * sw[q];
 #pragma unroll
             for (int o = 0; o < NF; o++)
-                acc[o] = fma(p64::exp_neg(R.t, h, h, rate[o], tab), yw * (sf[o][q] - fi[o]), acc[o]);
+                acc[o] = fma(p64::exp_neg<false>(R.t, h, h, rate[o], tab), yw * (sf[o][q] - fi[o]), acc[o]);
         }
     }
     if (ok)

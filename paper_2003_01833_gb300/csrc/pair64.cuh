@@ -128,20 +128,34 @@ __device__ __forceinline__ float small32(double h)
 }
 
 // Exponent factor of e^(-k a) = 2^(c a / 512): c = -512 k log2(e) as a
-// float64, what the rounding left (a float32), and c as a float32
+// float64, what the rounding left (a float32), and c as a float32; sub: see
+// subnormal()
 struct Rate {
     double c;
     float cl, cf;
+    uint32_t sub;
 };
 __device__ __forceinline__ Rate make_rate(double k)
 {
     constexpr double lh = 0x1.71547652b82fep+0, ll = 0x1.777d0ffda0d24p-56;  // log2(e)
     const double k5 = -512.0 * k, c = k5 * lh;
-    return Rate{c, (float)(fma(k5, lh, -c) + k5 * ll), (float)c};
+    const double r = 707.5 / k;  // e^-707.5 = 2^-1020.7
+    return Rate{c, (float)(fma(k5, lh, -c) + k5 * ll), (float)c, (uint32_t)__double2hiint(r * r)};
+}
+
+// whether e^(-k r) may be below the normal range and not round to zero: 707.5 <=
+// k r < 746, outwards, by the high word of r2 (the square of 746 / 707.5 is
+// 1.112: at most 0.202 of a binade's 2^20 high words above)
+__device__ __forceinline__ bool subnormal(double r2, const Rate& k)
+{
+    return (uint32_t)(__double2hiint(r2) - (int)k.sub) < 0x34000u;
 }
 
 // e^(-k a (1 + da)) (1 + h) for a >= 0 in float32's range and |da|, |h| < 2^-42,
-// to an ulp beside the rounding of a; 0 where it is below 2^-1021
+// to an ulp beside the rounding of a.  Below 2^-1021: with TAIL rounded to a
+// multiple of 2^-1074, without it 0 (a branch here costs a kernel of two fields
+// 6%; its callers keep such pairs away, subnormal())
+template <bool TAIL>
 __device__ __forceinline__ double exp_neg(double a, float da, float h, const Rate& k, const double* __restrict__ tab)
 {
     const float af = trunc32(__double2hiint(a), (uint32_t)__double2loint(a));
@@ -181,8 +195,12 @@ __device__ __forceinline__ double exp_neg(double a, float da, float h, const Rat
     int64_t E = ((int64_t)thi << 32 | tlo) + ((int64_t)i1 << 21) + i2;
     constexpr int64_t one = 0x3FF0000000000000ll;
     if (E < one) E += E - one;  // below 1 the units are half as large (only from T = 1)
-    E += (int64_t)(n >> 9) << 52;
-    return n < -1021 * kTab ? 0.0 : __longlong_as_double(E);
+    if (!TAIL) return n < -1021 * kTab ? 0.0 : __longlong_as_double(E + ((int64_t)(n >> 9) << 52));
+    if (n < -1021 * kTab) {  // below the normal range: the one rounding is the product's
+        const double v = __longlong_as_double(E + ((int64_t)((n >> 9) + 64) << 52)) * 0x1p-64;
+        return n < -1076 * kTab ? 0.0 : v;
+    }
+    return __longlong_as_double(E + ((int64_t)(n >> 9) << 52));
 }
 
 }  // namespace p64

@@ -1,6 +1,7 @@
 """Single pairs of the float64 forms, one source seen by every target, where the
-reciprocal root's approximation may lie on the other side of a power of two.
-Against float64 and extended arithmetic on the host.
+reciprocal root's approximation may lie on the other side of a power of two, and
+where the exponential is below float64's normal range.  Against float64 and
+extended arithmetic on the host.
 """
 import numpy as np
 import pytest
@@ -55,3 +56,16 @@ def test_distances_next_to_powers_of_two(T):
     exact = np.exp(-k * r.astype(np.longdouble)) / r
     for got in pair_values(T, r, k, 1.0):
         assert np.max(np.abs(got / exact - 1)) <= 5 * 2.0 ** -52
+
+
+def test_exponentials_below_the_normal_range(T):
+    """k r from 690 to 750, a weight of 2^1000: the exponential's subnormal values
+    (spacing 2^-1074) count.  Half a spacing beside the relative bound: an ulp of
+    the exponential, half of the final product and of k r, four roundings of the
+    weight, the factor 4 pi and its quotient here."""
+    r = np.arange(690.0, 750.0, 0.25)
+    e = np.exp(-r.astype(np.longdouble))
+    exact = e / r * 2.0 ** 1000
+    bound = (np.longdouble(2.0) ** -1075 + (6 + r) * 2.0 ** -52 * e) / r * 2.0 ** 1000
+    for got in pair_values(T, r, 1.0, 2.0 ** 1000):
+        assert np.all(np.abs(got - exact) <= bound)

@@ -11,6 +11,10 @@ Bounds: |h| < 2^-43 as the header states; 1/r to 1.5 units of 2^-53 relative to
 the value (its rounding, and the square's r2 y in h); the Yukawa value e^(-k r)/r
 to 2 (1 + k r) units of 2^-52 (an ulp of the exponential, the final product's
 rounding and k times r's).
+
+The exponential's tail, likewise: where subnormal() does not send a pair to the
+math library e^(-k r) has to be normal or round to zero, and the TAIL form has to
+return the subnormal values, to half their spacing beside the bound above.
 """
 import os
 import subprocess
@@ -76,26 +80,50 @@ int main()
                     er = fmax(er, (double)fabsl(R.ri() * r - 1.0L) * 0x1p53);
                     if (k * (double)r > 700.0) continue;
                     const float h = small32(R.h);
-                    const double v = exp_neg(R.t, h, h, rate, kExp2Table.v) * R.y;
+                    const double v = exp_neg<false>(R.t, h, h, rate, kExp2Table.v) * R.y;
                     const long double exact = expl(-k * r) / r;
                     ey = fmax(ey, (double)(fabsl(v / exact - 1.0L) / (1.0L + k * r)) * 0x1p52);
                 }
             }
         }
-    printf("%ld %.17g %.4g %.4g\n", n, eh, er, ey);
+    // the tail: errors in units of the bounds
+    double et = 0, eg = 0;
+    for (double kt = 1e-9; kt < 1e10; kt *= 1.37) {
+        const Rate rt = make_rate(kt);
+        for (double x = 690.0; x < 790.0; x += 0.0137) {
+            const double r2 = (x / kt) * (x / kt);
+            if (!fast_range(r2)) continue;
+            seed = (float)(1.0 / sqrt(r2));
+            const Root R = root(r2);
+            const float h = small32(R.h);
+            const long double kr = kt * sqrtl((long double)r2), e = expl(-kr);
+            const double tiny = subnormal(r2, rt) ? 0 : exp_neg<false>(R.t, h, 0.0f, rt, kExp2Table.v);
+            if (!subnormal(r2, rt))
+                et = fmax(et, (double)(fabsl(tiny - e) / (0x1p-1075L + (2.0L + 2.0L * kr) * 0x1p-52L * e)));
+            if (subnormal(r2, rt) && (kr < 706.0L || kr > 790.0L)) et = INFINITY;
+        }
+        for (double x = 690.0; x < 790.0; x += 0.0137) {
+            const double a = x / kt;
+            const long double ka = (long double)kt * a, e = expl(-ka);
+            const double g = exp_neg<true>(a, 0.0f, 0.0f, rt, kExp2Table.v);
+            eg = fmax(eg, (double)(fabsl(g - e) / (0x1p-1075L + (2.0L + 2.0L * ka) * 0x1p-52L * e)));
+        }
+    }
+    printf("%ld %.17g %.4g %.4g %.4g %.4g\n", n, eh, er, ey, et, eg);
     return 0;
 }
 """
 
 
-def test_root_next_to_powers_of_two(tmp_path):
+def test_root_and_exponential(tmp_path):
     (tmp_path / "cuda_runtime.h").write_text(CUDA)
     (tmp_path / "main.cpp").write_text(MAIN)
     exe = str(tmp_path / "pair64")
     subprocess.check_call(["g++", "-std=c++17", "-O1", "-w", "-ffp-contract=off", "-I", str(tmp_path), "-I", CSRC,
                            str(tmp_path / "main.cpp"), "-o", exe, "-lm"])
-    n, h, ri, yukawa = (float(v) for v in subprocess.check_output([exe], text=True, timeout=300).split())
+    n, h, ri, yukawa, tail, gauss = (float(v) for v in subprocess.check_output([exe], text=True, timeout=300).split())
     assert n > 40000
     assert h < 2.0 ** -43
     assert ri <= 1.5
     assert yukawa <= 2.0
+    assert tail <= 1.0 and gauss <= 1.0
