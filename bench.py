@@ -775,7 +775,7 @@ def main():
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": t_max, "higher_is_better": True, "scaling": "weak",
         "vs_baseline": None, "dtype": "f32c", "data": "synthetic",
-        "config": {"workload": workload_name(wl), "segment": seg or 8192,
+        "config": {"workload": workload_name(wl), "segment": seg or "default", "items": info["n_items"],
                    "step": "tree+lists+items, fields, anterpolation, near/far kernel, SS epilogue, "
                            "eps update, MGS, residuals, E_H",
                    "interactions_per_step": inter, "near_pairs": info["near_pairs"], "far_pairs": info["far_pairs"],

@@ -57,10 +57,11 @@ typedef enum {
  *   ss         1: singularity subtraction (Eq. yukawa-conv-ss, coulomb-conv-ss); 0: none.
  *   alpha      Gaussian width of the Coulomb subtraction (Eq. coulomb-conv-ss), > 0.
  *   segment    sources per work item of the near/far kernel (a batch's 128
- *              targets against a run of its interaction list), 1024 <= segment
- *              <= 65536, or 0 for 8192; fewer where that leaves few items.
- *              Longer segments mean fewer partial sums, shorter ones a finer
- *              balance of the work; partial sums are added in float64. */
+ *              targets against whole entries of its interaction list until
+ *              they hold that many), 1024 <= segment <= 65536, or 0: 8192,
+ *              fewer where that leaves few items.  Longer segments mean fewer
+ *              partial sums, shorter ones a finer balance of the work; partial
+ *              sums are added in float64. */
 typedef struct {
     double theta;
     int degree;

@@ -1139,16 +1139,17 @@ void build_tree(Tree& T, const double* xyz, const double* w)
     TAGI_LAUNCH_CHECK();
 
     // ---- work items of the near/far kernel
-    // Large trees: whole entries, kSegment sources (or the caller's number) an
-    // item, so that the order in which a target's two-float sums are added
-    // stays as it is.  Where that leaves fewer than kItemsFew items (1.3 waves
-    // of 152 SMs at 10 CTAs) the SMs would wait for a few long ones: the items
-    // are split until there are kItemsWanted.  The 5,003 point cube ran 64 CTAs
-    // over 5,003 sources each, 334 us a call at first, 82 split; the uniform
-    // hydrogen mesh (400 items) 689 -> 446 us.
+    // Whole entries, the caller's number of sources an item or kSegment: the
+    // order in which a target's two-float sums are added follows from the
+    // segment and the list alone.  Where no number was given and kSegment leaves
+    // fewer than kItemsFew items (1.3 waves of 152 SMs at the 10 CTAs of the
+    // three-field kernel) the SMs would wait for a few long ones: there the
+    // items are split until there are kItemsWanted.  The 5,003 point cube ran 64
+    // CTAs over 5,003 sources each, 334 us a call at first, 82 split; the
+    // uniform hydrogen mesh (400 items) 689 -> 446 us.
     const int64_t rows = (T.near_pairs + T.far_pairs) / kTargetsPerItem;
     int seg_src = T.segment ? T.segment : kSegment;
-    T.split_items = rows / seg_src < kItemsFew;
+    T.split_items = T.segment == 0 && rows / seg_src < kItemsFew;
     if (T.split_items) {
         const int unit = std::max(kItemUnit, padded(T.P));  // no unit is longer than an item
         seg_src = (int)std::max<int64_t>(std::min<int64_t>(seg_src, rows / kItemsWanted), unit);
