@@ -1,10 +1,13 @@
 """Single pairs of the float64 forms, one source seen by every target, where the
 reciprocal root's approximation may lie on the other side of a power of two, and
 where the exponential is below float64's normal range.  Against float64 and
-extended arithmetic on the host.
+extended arithmetic on the host.  Groups of fields against the float64 oracle.
 """
 import numpy as np
 import pytest
+
+import oracle
+from paper_2003_01833_gb300 import workloads as W
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -69,3 +72,28 @@ def test_exponentials_below_the_normal_range(T):
     bound = (np.longdouble(2.0) ** -1075 + (6 + r) * 2.0 ** -52 * e) / r * 2.0 ** 1000
     for got in pair_values(T, r, 1.0, 2.0 ** 1000):
         assert np.all(np.abs(got - exact) <= bound)
+
+
+@pytest.mark.parametrize("ss", [True, False])
+@pytest.mark.parametrize("nf_y", [1, 3, 4, 5])
+def test_groups_of_yukawa_fields(T, ss, nf_y):
+    """With Hartree beside them, points 1e-6 apart and two coincident.  1e-12 of
+    the field's largest value, as the other float64 parity tests, and beside it
+    the rounding of the charges f w, which the tree form stores as float64 and the
+    oracle does not form: 2^-53 of each |f w| times its kernel value."""
+    n = 1003
+    xyz, w = W.random_cube(n, seed=9)
+    xyz[:, 1::7] = xyz[:, 0:-1:7][:, :xyz[:, 1::7].shape[1]] * (1 + 1e-6)
+    xyz[:, 5] = xyz[:, 4]
+    xyz *= 3.0
+    rho = np.exp(-np.sum(xyz * xyz, axis=0))
+    f = np.stack([np.cos(xyz[0] + o) for o in range(nf_y)])
+    k = [0.5 + o for o in range(nf_y)]
+    u, vh = torch.empty((nf_y, n), dtype=torch.float64, device="cuda"), torch.empty(n, dtype=torch.float64,
+                                                                                   device="cuda")
+    with T.Tree(dev(xyz), dev(w), theta=0.0, degree=2, leaf_size=300, prec=T.TAGI_FP64, ss=ss) as tr:
+        T.tagi_fields_conv(tr.handle, dev(f), k, u, rho=dev(rho), vh=vh)
+    for o in range(nf_y):
+        ref = oracle.direct_yukawa(xyz, w, f[o], k[o], ss=ss)
+        charges = 2.0 ** -53 * oracle.direct_yukawa(xyz, np.abs(w), np.abs(f[o]), k[o], ss=False)
+        assert np.all(np.abs(u[o].cpu().numpy() - ref) <= 1e-12 * np.abs(ref).max() + charges)
