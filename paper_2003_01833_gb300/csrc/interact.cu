@@ -441,9 +441,11 @@ __device__ __forceinline__ void tile_near(const float4* __restrict__ sn, int nk,
 // (the fixed order, so the result does not depend on which CTA finishes
 // last), stores the sum, resets the counter for the next launch, and drops
 // the partial rows' lines from L2 without writing them back: the rows are
-// dead, so they never reach DRAM while they fit in L2 together with the
-// in-flight chunks.  Rows of fields [field0, field0 + nf) of each item are
-// contiguous (nf x 2 KB), so they are whole 128-byte lines.
+// dead.  A whole tree runs every chunk's last item after all others
+// (k_item_fill), so rows wait for it, and those that L2 does not hold until
+// then do reach DRAM: 253 MB a launch of 35 ms on the Li step of 309,000 points
+// (34 with a chunk's items in sequence, which took longer).  Rows of fields
+// [field0, field0 + nf) of each item are contiguous, nf x 1 KB.
 __device__ __forceinline__ void discard_line(const void* p)
 {
     asm volatile("discard.global.L2 [%0], 128;" ::"l"(p) : "memory");
@@ -469,6 +471,7 @@ __device__ __forceinline__ void chunk_sum(const Item& it, double* __restrict__ p
     }
     __syncthreads();  // every read of the rows has returned
     constexpr int kLineDoubles = 128 / sizeof(double);
+    static_assert(kTargetsPerItem % kLineDoubles == 0, "a row is whole lines");
     const int lines = nf * kTargetsPerItem / kLineDoubles;  // per item
     for (int q = threadIdx.x; q < it.ni * lines; q += blockDim.x) {
         const int i = it.i0 + q / lines, l = q % lines;

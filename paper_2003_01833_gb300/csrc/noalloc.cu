@@ -5,8 +5,8 @@
 // exceed its budget), and latency-critical loops in which an allocation's
 // implicit device synchronisation would stall other streams.  The caller
 // passes inputs and outputs; the only other device memory used is one
-// file-scope scratch array of fixed size that the library's module carries on
-// every GPU that loads it, until process exit.
+// file-scope scratch array of fixed size and the 4 KB table of pair64.cuh, which
+// the library's module carries on every GPU that loads it, until process exit.
 //
 // It is a variant of the float64 near/far interaction kernel (k_interact64)
 // that needs no tree: every target sums over every source (the theta = 0 case

@@ -13,7 +13,7 @@ to 2 (1 + k r) units of 2^-52 (an ulp of the exponential, the final product's
 rounding and k times r's).
 
 The exponential's tail, likewise: where subnormal() does not send a pair to the
-math library e^(-k r) has to be normal or round to zero, and the TAIL form has to
+TAIL form e^(-k r) has to be normal or round to zero, and the TAIL form has to
 return the subnormal values, to half their spacing beside the bound above.
 """
 import os
