@@ -698,9 +698,9 @@ def main():
     h2d = 8 * n * (3 + 1 + 1 + 1 + nw)
     d2h = 8 * n * (nw + 1)
 
-    # ---- plain FP64 form: one orbital per launch, same tree, no graph.  One
-    # warm-up and three timed Green iterations on a tree built once, beside
-    # the FP32C eager Green iteration timed the same way.
+    # ---- plain FP64 form: both orbitals and Hartree in one launch, same tree,
+    # no graph.  One warm-up and three timed Green iterations on a tree built
+    # once, beside the FP32C eager Green iteration timed the same way.
     plain = None
     if not args.no_plain and rank == 0 and lithium:
         def time_steps(prm, count, warm):

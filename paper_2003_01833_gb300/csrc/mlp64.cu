@@ -35,7 +35,7 @@
 // weight gradients, whose K are the points; W2 likewise serves Z2 and dH1.
 // That takes 100 KB, so two CTAs share an SM and one computes while the other
 // waits.  With transposed copies stored value by value (160 KB, one CTA of 512
-// threads) a training step over 10.9M points took 4.63 ms, now 1.73 (131 and 49
+// threads) a training step over 10.9M points took 4.63 ms, now 1.74 (131 and 49
 // SM clocks a point), the same bits.
 //
 // The float32 sums in TMEM are those of one CTA per SM: virtual CTA v owns
